@@ -85,7 +85,7 @@ def parse():
                     help="with --profile-substeps: instead of substeps, that many list builds of the sorted state "
                          "(gic_sort + gic_neighbors_build), for a capture of the staged build")
     ap.add_argument("--profile-direct", action="store_true",
-                    help="with --profile-substeps: gic_sort + gic_substep every substep (no CUDA graph), so that "
+                    help="with --profile-substeps: gic_sort + gic_substep every substep , so that "
                          "a profiler sees each kernel")
     return ap.parse_args()
 
@@ -589,7 +589,7 @@ def run_e2e(prob, sim, gic, torch, np, dev, stream, steps):
                 p(o_v), p(o_a), *[p(f) for f in o_fs], p(o_s), p(ws), ws.numel(), C.c_void_p(stream.cuda_stream))
         assert rc == 0, gic.last_error()
 
-    for _ in range(2):  # warm-up (graphs instantiated, kernels loaded)
+    for _ in range(2):  # warm-up (kernels loaded)
         call()
     times = []
     for _ in range(steps):

@@ -90,8 +90,9 @@ enum {
   GIC_STATUS_RADIUS = 8u,        /* a radius exceeds h_c / 2: contacts beyond the 27 cells are missed */
   GIC_STATUS_BAD_CELL = 16u,     /* an input cell id lay outside the contact grid */
   GIC_STATUS_FAST = 32u,         /* a granule moved more than one contact cell in a substep */
-  GIC_STATUS_DEBUG_INDEX = 64u   /* a library built with GIC_DEBUG found an index out of its array; the access
+  GIC_STATUS_DEBUG_INDEX = 64u,  /* a library built with GIC_DEBUG found an index out of its array; the access
                                     was skipped (release builds never set it) */
+  GIC_STATUS_STALL = 128u        /* a wait inside a kernel ran out of its limit; the call's results are not valid */
 };
 
 typedef struct GicGrid {
@@ -244,7 +245,8 @@ typedef struct GicNeighbors {
   int32_t* at;       /* [n] slot of each current sorted index (written by every call) */
   uint32_t* flags;   /* [8]: [0] rebuild in this call, [1] bit 0 rebuild requested, bit 1 a list overflowed at the
                       * last build, [2] CTA counter, [3] overflow during a build, [4] builds performed, [5] a
-                      * granule written by the last substep kernel is beyond skin / 2 (read by gic_step) */
+                      * granule written by the last substep kernel is beyond skin / 2 (read by gic_step),
+                      * [6] arrivals at the sort's grid barriers */
 } GicNeighbors;
 
 int gic_contact_verlet(const GicGrid* grid, const GicParams* params, const GicGranules* sorted,
@@ -291,18 +293,15 @@ int gic_substep(const GicGrid* grid, const GicParams* params, const GicGranules*
  * The caller swaps state and next between calls.
  *   FP32: `next` receives float positions (posf, if set) for the next
  *   call's contact pre-tests, read from `state` (if set) when no sort runs.
- *   The call runs as a CUDA graph: a one-thread decision kernel sets the
- *   conditionals of two branches (sort + substep, or substep alone), so a
- *   substep without a rebuild launches only the decision and the substep
- *   kernel and nothing waits on the host.  The first call with a given
- *   configuration (every argument's value, the params and the structs'
- *   contents) builds and instantiates the graph; up to eight configurations
- *   stay cached (least recently used replaced).  The graph bakes in the
- *   pointers: buffers must stay allocated while calls with them may come.
+ *   Two launches (four with alpha_s), the same in every call, and no host
+ *   sync: a cooperative kernel that sorts when the flags ask for it and
+ *   returns at once otherwise, and the substep kernel, which then builds the
+ *   rows of `sorted` and reads it, or reads `state`.  Nothing is kept between
+ *   calls.
  *   Arguments as for gic_sort and gic_substep (state, next and sorted must
- *   carry ids and share no array); errors as for those calls, plus
- *   GIC_ERR_CUDA if a graph cannot be built.  With sums2 the first 32 bytes
- *   of ws also hold the exact alpha_s totals while the call runs. */
+ *   carry ids and share no array); errors as for those calls.  With sums2
+ *   the first 32 bytes of ws also hold the exact alpha_s totals while the
+ *   call runs. */
 int gic_step(const GicGrid* grid, const GicParams* params, const GicGranules* state, GicGranules* next,
              GicGranules* sorted, int32_t* perm, void* cell_table, void* ws, size_t ws_bytes, const GicNeighbors* nb,
              const void* u, const void* v, const void* w, const void* p, const void* alpha_f, double* alpha_s,

@@ -102,7 +102,7 @@ __device__ __forceinline__ bool pair_geom_signed(const DGrid& G, int Dx, int Dy,
   float Rh = ri + rj;
   float bb = Rh - ri;
   float Rl = (ri - (Rh - bb)) + (rj - bb);
-  float Ph = Rh * G.s_hi;
+  float Ph = __fmul_rn(Rh, G.s_hi);  // not to be fused into Ph - dh: Pl holds its rounding
   float Pl = fmaf(Rh, G.s_hi, -Ph) + fmaf(Rh, G.s_lo, Rl * G.s_hi);
   unsigned long long d2 = (unsigned long long)((long long)Dx * Dx) + (unsigned long long)((long long)Dy * Dy) +
                           (unsigned long long)((long long)Dz * Dz);

@@ -11,7 +11,7 @@
 //   F_n = (k_n overlap - c_n v_n) n,   c_n = 2 zeta sqrt(k_n m_eff),
 //   f_t = -k_t v_t,  k_t = kt_over_cn c_n,   F_t = min(|f_t|, mu |F_n|) f_t/|f_t|.
 // Walls are partners of infinite mass at rest (m_eff = m_i).
-#include "gic_contact.cuh"
+#include "gic_tile.cuh"
 
 namespace gic {
 
@@ -35,16 +35,7 @@ __global__ void __launch_bounds__(128) k_contact(DGrid G, DParams<T> P, int64_t 
   bool coincident = false;
   for_each_contact<T>(G, table, epoch, i, cx, cy, cz, pi, ri, pos, posf, [&](int64_t j, const PairGeom<T>& g) {
     vec_t<T> vj = ldg(&vel[j]);
-    T mj = granule_mass(P, radius_of(ldg(&pos[j])));
-    T f0, f1, f2;
-    if (pair_force(P, g.x0, g.x1, g.x2, g.d, g.overlap, vi.x - vj.x, vi.y - vj.y, vi.z - vj.z, mi * mj / (mi + mj), f0,
-                   f1, f2)) {
-      F0 += f0;
-      F1 += f1;
-      F2 += f2;
-    } else {
-      coincident = true;
-    }
+    add_force(P, g, vi, vj, mi, radius_of(ldg(&pos[j])), F0, F1, F2, coincident);
   });
   if (P.walls) {
     const int c3[3] = {cx, cy, cz};
@@ -71,181 +62,7 @@ __global__ void __launch_bounds__(128) k_contact(DGrid G, DParams<T> P, int64_t 
   F[i] = make_vec<T>(F0, F1, F2);
 }
 
-// ----------------------------------------------------------------- staged FP32 contact
-//
-// One CTA = 128 consecutive granules of the Morton-sorted state: a compact
-// blob of contact cells.  The CTA stages the cell-table entries of the
-// blob's bounding box (+1 cell halo) and the float positions of every
-// granule in those cells in shared memory, then each thread walks its 27
-// neighbour cells there.  A CTA whose box or granule count exceeds the
-// shared-memory budget (a Morton range that jumps across the domain) takes
-// the global-memory path instead; the results are identical.
-
-constexpr int kTileThreads = 128;
-constexpr int kTileMaxCells = 512;
-constexpr int kTileMaxGranules = 1152;
-
-__device__ __forceinline__ void add_pair_force(const DParams<float>& P, const PairGeom<float>& g, const float4& vi,
-                                               const float4& vj, float mi, float mj, float& F0, float& F1, float& F2,
-                                               bool& coincident) {
-  float f0, f1, f2;
-  if (pair_force(P, g.x0, g.x1, g.x2, g.d, g.overlap, vi.x - vj.x, vi.y - vj.y, vi.z - vj.z, mi * mj / (mi + mj), f0,
-                 f1, f2)) {
-    F0 += f0;
-    F1 += f1;
-    F2 += f2;
-  } else {
-    coincident = true;
-  }
-}
-
-// The CTA's staged neighbourhood in shared memory.
-struct TileShared {
-  int lo[3], hi[3];
-  uint32_t start[kTileMaxCells];
-  uint32_t cnt[kTileMaxCells];
-  uint32_t off[kTileMaxCells + 1];
-  float4 pf[kTileMaxGranules];
-  uint32_t wsum[kTileThreads / 32];
-  int mode;             // 0: staged, 1: global fallback
-  unsigned rmax_bits;   // the largest staged radius (float bits)
-};
-
-struct TileBox {
-  int bx0, by0, bz0, bx, by, bz;
-};
-
-// CTA-wide (every thread calls it): the bounding box of the CTA's contact
-// cells with a one-cell halo, clipped to the grid; its table entries (start,
-// count of this epoch), their exclusive scan and the float positions of every
-// granule in the box, relative to the box corner.  sh.mode = 1 when the box or
-// its granules exceed the tile.  valid / ci: this thread's granule and cell.
-__device__ __forceinline__ TileBox tile_stage(TileShared& sh, const DGrid& G, const uint4* __restrict__ table,
-                                              uint32_t epoch, const float4* __restrict__ posf, bool valid,
-                                              int32_t ci) {
-  if (threadIdx.x < 3) {
-    sh.lo[threadIdx.x] = 1 << 30;
-    sh.hi[threadIdx.x] = -1;
-  }
-  if (threadIdx.x == 0) sh.rmax_bits = 0u;
-  __syncthreads();
-  if (valid) {
-    atomicMin(&sh.lo[0], cell_x(ci));
-    atomicMin(&sh.lo[1], cell_y(ci));
-    atomicMin(&sh.lo[2], cell_z(ci));
-    atomicMax(&sh.hi[0], cell_x(ci));
-    atomicMax(&sh.hi[1], cell_y(ci));
-    atomicMax(&sh.hi[2], cell_z(ci));
-  }
-  __syncthreads();
-  TileBox T;
-  T.bx0 = max(sh.lo[0] - 1, 0);
-  T.by0 = max(sh.lo[1] - 1, 0);
-  T.bz0 = max(sh.lo[2] - 1, 0);
-  T.bx = min(sh.hi[0] + 1, G.nc[0] - 1) - T.bx0 + 1;
-  T.by = min(sh.hi[1] + 1, G.nc[1] - 1) - T.by0 + 1;
-  T.bz = min(sh.hi[2] + 1, G.nc[2] - 1) - T.bz0 + 1;
-  const int ncell = T.bx * T.by * T.bz;
-  if (threadIdx.x == 0) sh.mode = (ncell > kTileMaxCells || sh.hi[0] < 0) ? 1 : 0;
-  __syncthreads();
-  if (sh.mode == 0) {
-    // stage the table entries of the box
-    // box index -> coordinates with float reciprocals (exact for these small integers)
-    const float ibx = 1.0f / (float)T.bx, ibxy = 1.0f / (float)(T.bx * T.by);
-    constexpr int kU = 4;  // loads in flight per thread
-    for (int b0 = threadIdx.x; b0 < ncell; b0 += kU * kTileThreads) {
-      uint4 e[kU];
-#pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const int b = b0 + u * kTileThreads;
-        if (b >= ncell) break;
-        int z = (int)(((float)b + 0.5f) * ibxy);
-        int rem = b - z * T.bx * T.by;
-        int y = (int)(((float)rem + 0.5f) * ibx);
-        int x = T.bx0 + rem - y * T.bx;
-        y += T.by0;
-        z += T.bz0;
-        e[u] = __ldg(&table[table_index(G, x, y, z)]);
-      }
-#pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const int b = b0 + u * kTileThreads;
-        if (b >= ncell) break;
-        const bool ok = e[u].z == epoch;
-        sh.start[b] = ok ? e[u].x : 0u;
-        sh.cnt[b] = ok ? e[u].y : 0u;
-      }
-    }
-    __syncthreads();
-    // exclusive scan of the counts (ncell <= 512: 4 per thread)
-    {
-      const int per = (kTileMaxCells + kTileThreads - 1) / kTileThreads;
-      uint32_t loc[per];
-      uint32_t sum = 0;
-#pragma unroll
-      for (int k = 0; k < per; ++k) {
-        int b = threadIdx.x * per + k;
-        loc[k] = b < ncell ? sh.cnt[b] : 0u;
-        sum += loc[k];
-      }
-      uint32_t incl = sum;
-      for (int off = 1; off < 32; off <<= 1) {
-        uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane_id() >= off) incl += o;
-      }
-      if (lane_id() == 31) sh.wsum[threadIdx.x >> 5] = incl;
-      __syncthreads();
-      uint32_t base = 0;
-      for (int w = 0; w < (threadIdx.x >> 5); ++w) base += sh.wsum[w];
-      uint32_t run = base + incl - sum;
-#pragma unroll
-      for (int k = 0; k < per; ++k) {
-        int b = threadIdx.x * per + k;
-        if (b < kTileMaxCells) sh.off[b] = run;
-        run += loc[k];
-      }
-      if (threadIdx.x == kTileThreads - 1) sh.off[kTileMaxCells] = run;
-    }
-    __syncthreads();
-    const uint32_t total = sh.off[kTileMaxCells];
-    if (total > (uint32_t)kTileMaxGranules) {
-      if (threadIdx.x == 0) sh.mode = 1;
-    } else {
-      // stage the float positions: slot t belongs to cell b with off[b] <= t < off[b + 1]
-      float rmax = 0.f;
-      for (uint32_t t0 = threadIdx.x; t0 < total; t0 += kU * kTileThreads) {
-        float4 pv[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const uint32_t t = t0 + u * kTileThreads;
-          if (t >= total) break;
-          int lo = 0, hi = ncell - 1;  // last b with off[b] <= t
-          while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (sh.off[mid] <= t) lo = mid;
-            else hi = mid - 1;
-          }
-          pv[u] = __ldg(&posf[sh.start[lo] + (t - sh.off[lo])]);
-        }
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          const uint32_t t = t0 + u * kTileThreads;
-          if (t >= total) break;
-          // position in units of contact cells relative to the box corner (exact
-          // differences of the absolute copies): the three cells of an x-row are
-          // consecutive slots, and no cell offset is needed
-          const float4 p = pv[u];
-          sh.pf[t] = make_float4(p.x - (float)T.bx0, p.y - (float)T.by0, p.z - (float)T.bz0, p.w);
-          rmax = fmaxf(rmax, p.w);
-        }
-      }
-      const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(rmax));  // radii >= 0
-      if (lane_id() == 0) atomicMax(&sh.rmax_bits, m);
-    }
-    __syncthreads();
-  }
-  return T;
-}
+// ----------------------------------------------------------------- staged FP32 contact (gic_tile.cuh)
 
 __global__ void __launch_bounds__(kTileThreads) k_contact_tile(DGrid G, DParams<float> P, int64_t n,
                                                                const int32_t* __restrict__ cell,
@@ -254,16 +71,16 @@ __global__ void __launch_bounds__(kTileThreads) k_contact_tile(DGrid G, DParams<
                                                                const float4* __restrict__ vel,
                                                                const uint4* __restrict__ table,
                                                                float4* __restrict__ F, uint32_t* status) {
-  __shared__ TileShared sh;
+  __shared__ TileShared<kTileThreads> sh;
   const int64_t i = blockIdx.x * (int64_t)kTileThreads + threadIdx.x;
   const bool valid = i < n;
   const uint32_t epoch = __ldg(&table[0].x);
   const int32_t ci = valid ? cell[i] : 0;
   const int cx = cell_x(ci), cy = cell_y(ci), cz = cell_z(ci);
-  const TileBox T = tile_stage(sh, G, table, epoch, posf, valid, ci);
+  const TileBox T = tile_stage<kTileThreads, float>(sh, G, table, epoch, FloatPos<float>{cell, pos, posf, 0.0}, valid, ci);
   const int bx0 = T.bx0, by0 = T.by0, bz0 = T.bz0, bx = T.bx, by = T.by, bz = T.bz;
   uint32_t* const s_start = sh.start;
-  uint32_t* const s_off = sh.off;
+  const uint32_t* const s_off = sh.off;
   const float4* const s_pf = sh.pf;
   const int s_mode = sh.mode;
   if (!valid) return;
@@ -307,13 +124,13 @@ __global__ void __launch_bounds__(kTileThreads) k_contact_tile(DGrid G, DParams<
           int_sep(pi, pj, ox, oy, oz, Dx, Dy, Dz);
           PairGeom<float> g;
           if (!pair_geom_exact(G, Dx, Dy, Dz, ri, fj.w, g)) continue;
-          add_pair_force(P, g, vi, __ldg(&vel[j]), mi, granule_mass(P, fj.w), F0, F1, F2, coincident);
+          add_force(P, g, vi, __ldg(&vel[j]), mi, fj.w, F0, F1, F2, coincident);
         }
       }
     }
   } else {
     for_each_contact<float>(G, table, epoch, i, cx, cy, cz, pi, ri, pos, posf, [&](int64_t j, const PairGeom<float>& g) {
-      add_pair_force(P, g, vi, __ldg(&vel[j]), mi, granule_mass(P, radius_of(__ldg(&pos[j]))), F0, F1, F2, coincident);
+      add_force(P, g, vi, __ldg(&vel[j]), mi, radius_of(__ldg(&pos[j])), F0, F1, F2, coincident);
     });
   }
   if (P.walls) {
@@ -341,105 +158,25 @@ __global__ void __launch_bounds__(kTileThreads) k_contact_tile(DGrid G, DParams<
   F[i] = make_float4(F0, F1, F2, 0.f);
 }
 
-// The list build of gic_step's rebuilding substep (FP32 path with float
-// copies, contact law only), on the staged neighbourhood: every granule's row
-// -- the partners within r_i + r_j + skin by the float pre-test of
-// verlet_pair, in the order of the 27-cell walk, slot = sorted index -- and its
-// reference entries; no forces (the substep then walks the fresh rows, so the
-// forces and their order are those of a build inside the substep).  The last
-// CTA records the build; if a row overflowed it leaves the rebuild word set,
-// and the substep's own 27-cell walk takes over as before.
-__global__ void __launch_bounds__(kTileThreads) k_verlet_build_tile(DGrid G, int64_t n, const int32_t* __restrict__ cell,
-                                                                    const uint4* __restrict__ pos,
-                                                                    const float4* __restrict__ posf,
-                                                                    const int32_t* __restrict__ id,
-                                                                    const uint4* __restrict__ table, NbDev nb,
+// gic_neighbors_build: the rows of the whole sorted state, one CTA per 128
+// granules.  The last CTA records the build; if a row overflowed it leaves the
+// request set, and the next call rebuilds.
+__global__ void __launch_bounds__(kTileThreads) k_verlet_build_tile(DGrid G, int64_t n, FloatPos<float> fpos,
+                                                                    const int32_t* id, const uint4* table, NbDev nb,
                                                                     float skin) {
-  __shared__ TileShared sh;
-  const bool rebuild = (nb.flags[kNbRebuild] | nb.flags[kNbSticky]) != 0u;  // uniform over the launch
+  __shared__ TileShared<kTileThreads> sh;
   const int64_t i = blockIdx.x * (int64_t)kTileThreads + threadIdx.x;
   const bool valid = i < n;
+  const int32_t ci = valid ? __ldg(&fpos.cell[i]) : 0;
   const uint32_t epoch = __ldg(&table[0].x);
-  const int32_t ci = valid ? cell[i] : 0;
-  const int cx = cell_x(ci), cy = cell_y(ci), cz = cell_z(ci);
-  const TileBox T = tile_stage(sh, G, table, epoch, posf, valid, ci);
-  if (valid && rebuild) {
-    const uint4 pi = pos[i];
-    const float ri = __uint_as_float(pi.w);
-    const float4 fi = __ldg(&posf[i]);
-    int32_t* row = nb.list + i * nb.cap;
-    int cnt = 0;
-    bool over = false;
-    auto keep = [&](int64_t j) {
-      if (cnt < nb.cap)
-        row[cnt++] = (int32_t)j;
-      else
-        over = true;
-    };
-    if (sh.mode == 0) {
-      const int lx = cx - T.bx0, ly = cy - T.by0, lz = cz - T.bz0;
-      const float xi = fi.x - (float)T.bx0, yi = fi.y - (float)T.by0, zi = fi.z - (float)T.bz0;
-      const int bown = lx + T.bx * (ly + T.by * lz);
-      const uint32_t tself = sh.off[bown] + (uint32_t)(i - (int64_t)sh.start[bown]);
-      // Cells farther than the largest pre-test radius of any staged partner
-      // (plus a margin past the float rounding of d2) hold no partner: whole
-      // rows (oy, oz) and the end cells of a row are skipped.  A staged copy
-      // lies in its closed cell, so its distance is at least the cell's.
-      const float Rmax = fmaf(ri + __uint_as_float(sh.rmax_bits) + skin, G.inv_hc_f, kPosfTol) + 1e-3f;
-      const float R2 = Rmax * Rmax;
-      const float dxl = xi - (float)lx, dxh = (float)(lx + 1) - xi;  // to the own cell's x faces
-      for (int oz = -1; oz <= 1; ++oz) {
-        const int z = lz + oz;
-        if (z < 0 || z >= T.bz) continue;
-        const float dz = oz < 0 ? zi - (float)lz : (oz > 0 ? (float)(lz + 1) - zi : 0.f);
-        for (int oy = -1; oy <= 1; ++oy) {
-          const int y = ly + oy;
-          if (y < 0 || y >= T.by) continue;
-          const float dy = oy < 0 ? yi - (float)ly : (oy > 0 ? (float)(ly + 1) - yi : 0.f);
-          const float dyz = fmaf(dy, dy, dz * dz);
-          if (dyz >= R2) continue;
-          const int xa = (lx > 0 && fmaf(dxl, dxl, dyz) < R2) ? lx - 1 : lx;
-          const int xb = (lx + 1 < T.bx && fmaf(dxh, dxh, dyz) < R2) ? lx + 1 : lx;
-          const int rb = T.bx * (y + T.by * z);
-          const uint32_t t0 = sh.off[rb + xa], t1 = sh.off[rb + xb + 1];
-          for (uint32_t t = t0; t < t1; ++t) {
-            if (t == tself) continue;
-            const float4 fj = sh.pf[t];
-            const float rx = fj.x - xi, ry = fj.y - yi, rz = fj.z - zi;
-            const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-            const float Rs = fmaf(ri + fj.w + skin, G.inv_hc_f, kPosfTol);
-            if (d2 < Rs * Rs) {
-              int bj = rb + xa;
-              while (sh.off[bj + 1] <= t) ++bj;  // the cell of slot t (cells of the row in x order)
-              keep((int64_t)sh.start[bj] + (t - sh.off[bj]));
-            }
-          }
-        }
-      }
-    } else {
-      for_each_partner(G, table, epoch, i, cx, cy, cz, [&](int64_t j, int, int, int) {
-        const float4 fj = __ldg(&posf[j]);
-        const float rx = fj.x - fi.x, ry = fj.y - fi.y, rz = fj.z - fi.z;
-        const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-        const float Rs = fmaf(ri + fj.w + skin, G.inv_hc_f, kPosfTol);
-        if (d2 < Rs * Rs) keep(j);
-      });
-    }
-    nb.count[i] = cnt;
-    nb.at[i] = (int32_t)i;
-    nb.cur[i] = (int32_t)i;
-    nb.ref_cell[i] = ci;
-    reinterpret_cast<uint4*>(nb.ref_pos)[i] = pi;
-    const int32_t idi = id[i];
-    if (idi >= 0 && (int64_t)idi < n) nb.slot[idi] = (int32_t)i;
-    if (over) atomicOr(&nb.flags[kNbOverflow], 1u);
-  }
+  const TileBox B = tile_stage<kTileThreads, float>(sh, G, table, epoch, fpos, valid, ci);
+  build_row<kTileThreads, float, false, false>(sh, B, G, n, i, ci, fpos, id, table, epoch, nb, skin, 1.f);
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     if (atomicAdd(&nb.flags[kNbCounter], 1u) == gridDim.x - 1) {
       __threadfence();
-      if (rebuild && atomicExch(&nb.flags[kNbOverflow], 0u) == 0u) {  // a complete build: the substep walks it
+      if (atomicExch(&nb.flags[kNbOverflow], 0u) == 0u) {  // a complete build
         nb.flags[kNbSticky] = 0u;
         nb.flags[kNbRebuild] = 0u;
         nb.flags[kNbBuilds] += 1u;
@@ -448,15 +185,6 @@ __global__ void __launch_bounds__(kTileThreads) k_verlet_build_tile(DGrid G, int
       __threadfence();
     }
   }
-}
-
-int launch_build_tile(const DGrid& G, const GicGranules* sorted, const void* table, const NbDev& d, double skin,
-                      cudaStream_t stream) {
-  if (sorted->n == 0) return GIC_OK;
-  k_verlet_build_tile<<<grid_blocks(sorted->n, kTileThreads), kTileThreads, 0, stream>>>(
-      G, sorted->n, sorted->cell, (const uint4*)sorted->pos, (const float4*)sorted->posf, sorted->id,
-      (const uint4*)table, d, (float)skin);
-  return GIC_OK;
 }
 
 // kList: walk the Verlet rows (nb) instead of the 27 cells; the last CTA
@@ -487,9 +215,8 @@ __global__ void __launch_bounds__(128) k_contact_adj(DGrid G, DParams<T> P, int6
     auto pair = [&](int64_t j, const PairGeom<T>& g) {
       vec_t<T> vj = ldg(&vel[j]);
       vec_t<T> lj = ldg(&gF[j]);
-      T mj = granule_mass(P, radius_of(ldg(&pos[j])));
       gm += pair_force_adj(P, g.x0, g.x1, g.x2, g.d, g.overlap, vi.x - vj.x, vi.y - vj.y, vi.z - vj.z,
-                           mi * mj / (mi + mj), li.x - lj.x, li.y - lj.y, li.z - lj.z, li.x, li.y, li.z, gx0, gx1, gx2,
+                           pair_mass(P, mi, radius_of(ldg(&pos[j]))), li.x - lj.x, li.y - lj.y, li.z - lj.z, li.x, li.y, li.z, gx0, gx1, gx2,
                            gv0, gv1, gv2);
     };
     if constexpr (kList) {
@@ -906,7 +633,9 @@ extern "C" int gic_neighbors_build(const GicGrid* grid, const GicGranules* sorte
   if ((rc = verlet_view(G, sorted, cell_table, nb, "gic_neighbors_build", true, &d))) return rc;
   if (sorted->n == 0) return GIC_OK;
   k_request_build<<<1, 1, 0, (cudaStream_t)stream>>>(nb->flags);
-  if ((rc = launch_build_tile(G, sorted, cell_table, d, nb->skin, (cudaStream_t)stream))) return rc;
+  k_verlet_build_tile<<<grid_blocks(sorted->n, kTileThreads), kTileThreads, 0, (cudaStream_t)stream>>>(
+      G, sorted->n, FloatPos<float>{sorted->cell, (const uint4*)sorted->pos, (const float4*)sorted->posf, 0.0},
+      sorted->id, (const uint4*)cell_table, d, (float)nb->skin);
   count_launches(2);
   GIC_CHECK_LAUNCH("gic_neighbors_build");
   return GIC_OK;

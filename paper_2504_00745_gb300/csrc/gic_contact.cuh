@@ -13,8 +13,18 @@ __device__ __forceinline__ T granule_mass(const DParams<T>& P, T r) {
   return P.rho_s * (T(4.0 / 3.0 * kPi) * r * r * r);
 }
 
+// Reduced mass of granule i (mass mi) and one of radius rj, with the sum of the
+// masses rounded once.
+template <typename T>
+__device__ __forceinline__ T pair_mass(const DParams<T>& P, T mi, T rj) {
+  const T V = T(4.0 / 3.0 * kPi) * rj * rj * rj;
+  return mi * (P.rho_s * V) / fma(P.rho_s, V, mi);
+}
+
 // Pair force on i (x = x_i - x_j, v = v_i - v_j) at distance d with
-// overlap = r_i + r_j - d > 0.  Returns false for coincident centres.
+// overlap = r_i + r_j - d > 0.  Returns false for coincident centres.  The
+// fused multiply-adds are written out, so that every kernel that holds a copy
+// of the law rounds the same way.
 template <typename T>
 __device__ __forceinline__ bool pair_force(const DParams<T>& P, T x0, T x1, T x2, T d, T overlap, T v0, T v1, T v2,
                                            T meff, T& F0, T& F1, T& F2) {
@@ -22,17 +32,17 @@ __device__ __forceinline__ bool pair_force(const DParams<T>& P, T x0, T x1, T x2
   T inv_d = T(1) / d;
   T n0 = x0 * inv_d, n1 = x1 * inv_d, n2 = x2 * inv_d;
   T cn = T(2) * P.zeta * sqrt(P.k_n * meff);
-  T vn = v0 * n0 + v1 * n1 + v2 * n2;
-  T Fn = P.k_n * overlap - cn * vn;
-  T t0 = v0 - vn * n0, t1 = v1 - vn * n1, t2 = v2 - vn * n2;
+  T vn = fma(v2, n2, fma(v0, n0, v1 * n1));
+  T Fn = fma(P.k_n, overlap, -(cn * vn));
+  T t0 = fma(-vn, n0, v0), t1 = fma(-vn, n1, v1), t2 = fma(-vn, n2, v2);
   T kt = P.kt_over_cn * cn;
-  T ftn = kt * sqrt(t0 * t0 + t1 * t1 + t2 * t2);
+  T ftn = kt * sqrt(fma(t2, t2, fma(t0, t0, t1 * t1)));
   T cap = P.mu * fabs(Fn);
   T s = ftn > cap ? cap / ftn : T(1);
   T a = s * kt;
-  F0 = Fn * n0 - a * t0;
-  F1 = Fn * n1 - a * t1;
-  F2 = Fn * n2 - a * t2;
+  F0 = fma(Fn, n0, -(a * t0));
+  F1 = fma(Fn, n1, -(a * t1));
+  F2 = fma(Fn, n2, -(a * t2));
   return true;
 }
 
@@ -126,7 +136,7 @@ __device__ __forceinline__ bool pair_geom_exact(const DGrid& G, int Dx, int Dy, 
   float Rh = ri + rj;
   float bb = Rh - ri;
   float Rl = (ri - (Rh - bb)) + (rj - bb);  // TwoSum error
-  float Ph = Rh * G.s_hi;
+  float Ph = __fmul_rn(Rh, G.s_hi);  // not to be fused into Ph - dh: Pl holds its rounding
   float Pl = fmaf(Rh, G.s_hi, -Ph) + fmaf(Rh, G.s_lo, Rl * G.s_hi);
   // exact |D|^2 and a corrected square root
   unsigned long long d2 = (unsigned long long)((long long)Dx * Dx) + (unsigned long long)((long long)Dy * Dy) +
@@ -192,8 +202,8 @@ __device__ __forceinline__ bool wall_geom(const DGrid& G, const uint4& p, int a,
                                           float& overlap) {
   uint32_t q = pcomp(p, a);
   long long gq = side == 0 ? (long long)q : (long long)kFracOne - (long long)q;
-  float Ph = r * G.s_hi;
-  float Pl = fmaf(r, G.s_hi, -Ph) + r * G.s_lo;
+  float Ph = __fmul_rn(r, G.s_hi);
+  float Pl = fmaf(r, G.s_lo, fmaf(r, G.s_hi, -Ph));
   float ov;
   // gq <= 2^30; 32-bit conversions where the values fit (the 64-bit ones run on the FP64 pipe)
   if (Ph >= 2147483648.0f)
@@ -332,7 +342,8 @@ __device__ __forceinline__ void for_each_contact(const DGrid& G, const uint4* __
 // every call); kNbCounter -- CTAs done; kNbOverflow -- overflow during this
 // build; kNbBuilds -- builds so far; kNbNext -- a granule written by a
 // k_substep is beyond skin / 2 of its reference (gic_step's next call
-// rebuilds; gic_step consumes the word).
+// rebuilds; gic_step consumes the word); kNbBarrier -- arrivals at the grid
+// barriers of gic_step's sort (0 between calls).
 
 enum : int {
   kNbRebuild = 0,
@@ -341,8 +352,12 @@ enum : int {
   kNbOverflow = 3,
   kNbBuilds = 4,
   kNbNext = 5,
+  kNbBarrier = 6,
   kNbWords = 8
 };
+// The count of a row that overflowed in gic_step's build: the granule's contact
+// force comes from the 27 cells.
+constexpr int32_t kNbWalked = -1;
 
 struct NbDev {
   int cap;
@@ -384,10 +399,10 @@ __device__ __forceinline__ bool moved_far(const DGrid& G, int32_t c, const d4& p
 
 template <typename T>
 __device__ __forceinline__ void add_force(const DParams<T>& P, const PairGeom<T>& g, const vec_t<T>& vi,
-                                          const vec_t<T>& vj, T mi, T mj, T& F0, T& F1, T& F2, bool& coincident) {
+                                          const vec_t<T>& vj, T mi, T rj, T& F0, T& F1, T& F2, bool& coincident) {
   T f0, f1, f2;
-  if (pair_force(P, g.x0, g.x1, g.x2, g.d, g.overlap, vi.x - vj.x, vi.y - vj.y, vi.z - vj.z, mi * mj / (mi + mj), f0,
-                 f1, f2)) {
+  if (pair_force(P, g.x0, g.x1, g.x2, g.d, g.overlap, vi.x - vj.x, vi.y - vj.y, vi.z - vj.z, pair_mass(P, mi, rj), f0, f1,
+                 f2)) {
     F0 += f0;
     F1 += f1;
     F2 += f2;
@@ -583,11 +598,16 @@ int verlet_view(const DGrid& G, const GicGranules* s, const void* table, const G
 int verlet_check(const DGrid& G, const GicGranules* s, const void* table, const GicNeighbors* nb,
                  cudaStream_t stream, const char* what, NbDev* out, GicGranules* copy_to, int32_t* perm);
 
-// The staged list build of gic_step's rebuilding substep (FP32 path with
-// float copies): rows and reference entries of the sorted state, no forces;
-// records the build unless a row overflowed (see gic_contact.cu).
-int launch_build_tile(const DGrid& G, const GicGranules* sorted, const void* table, const NbDev& d, double skin,
-                      cudaStream_t stream);
+// This gic_step call rebuilds: a granule was beyond skin / 2 of its reference
+// after the last one, or a rebuild was requested.
+__device__ __forceinline__ bool step_rebuilds(const uint32_t* flags) {
+  return (flags[kNbNext] | flags[kNbSticky]) != 0u;
+}
+
+// gic_step's sort (gic_step_sort.cu): if the call rebuilds, `in` is sorted into
+// `out` (perm, cell table as gic_sort; scratch in ws); one launch either way.
+int launch_step_sort(const DGrid& G, const GicGranules* in, const GicGranules* out, int32_t* perm, void* table,
+                     void* ws, uint32_t* flags, cudaStream_t st);
 
 // The list build of granule i: walks the 27 cells with the pre-test radius
 // r_i + r_j + skin, writes row i (slot = sorted index) and its reference
@@ -637,7 +657,7 @@ __device__ __forceinline__ void verlet_build_granule(const DGrid& G, const DPara
                                                      bool& coincident) {
   verlet_build_row<T>(G, nb, table, n, i, cx, cy, cz, ci, pi, ri, has_f, fi, skin, id, pos, posf,
                       [&](int64_t j, const PairGeom<T>& g) {
-                        add_force(P, g, vi, ldg(&vel[j]), mi, granule_mass(P, radius_of(ldg(&pos[j]))), F0, F1, F2,
+                        add_force(P, g, vi, ldg(&vel[j]), mi, radius_of(ldg(&pos[j])), F0, F1, F2,
                                   coincident);
                       });
 }
@@ -656,6 +676,30 @@ __device__ __forceinline__ void verlet_call_done(const NbDev& nb, bool rebuild) 
         nb.flags[kNbBuilds] += 1u;
       }
       nb.flags[kNbRebuild] = 0u;
+      nb.flags[kNbCounter] = 0u;
+      __threadfence();
+    }
+  }
+}
+
+// The same for a gic_step call: only one that rebuilt has anything to record.
+// far: a granule of this CTA is beyond skin / 2 (the next call rebuilds).
+__device__ __forceinline__ void step_call_done(const NbDev& nb, bool rebuilt, bool far) {
+  if (!rebuilt) {  // uniform over the launch
+    if (far) atomicOr(&nb.flags[kNbNext], 1u);
+    return;
+  }
+  // the rebuild words are read by every CTA at its start: what this call asks of
+  // the next one goes to kNbRebuild until the last CTA is done
+  if (far) atomicOr(&nb.flags[kNbRebuild], 1u);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&nb.flags[kNbCounter], 1u) == gridDim.x - 1) {
+      __threadfence();
+      nb.flags[kNbNext] = atomicExch(&nb.flags[kNbRebuild], 0u);
+      nb.flags[kNbSticky] = atomicExch(&nb.flags[kNbOverflow], 0u) ? 2u : 0u;
+      nb.flags[kNbBuilds] += 1u;
       nb.flags[kNbCounter] = 0u;
       __threadfence();
     }
@@ -730,7 +774,7 @@ __device__ __forceinline__ void verlet_list_force(const DGrid& G, const DParams<
                                                   T& F0, T& F1, T& F2, bool& coincident) {
   for_each_list_contact<T>(G, nb, i, cx, cy, cz, ci, pi, ri, has_f, fi, cell, pos, posf,
                            [&](int64_t j, const PairGeom<T>& g) {
-                             add_force(P, g, vi, ldg(&vel[j]), mi, granule_mass(P, radius_of(ldg(&pos[j]))), F0, F1,
+                             add_force(P, g, vi, ldg(&vel[j]), mi, radius_of(ldg(&pos[j])), F0, F1,
                                        F2, coincident);
                            });
 }

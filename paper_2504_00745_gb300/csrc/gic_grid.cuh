@@ -63,15 +63,15 @@ __device__ __forceinline__ T g2p_granule_with(const DGrid& G, const DParams<T>& 
   T r = radius_of(pi);
   T V = T(4.0 / 3.0 * kPi) * r * r * r;
   T d0 = uf[0] - vi.x, d1 = uf[1] - vi.y, d2 = uf[2] - vi.z;
-  T sp = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
+  T sp = sqrt(fma(d2, d2, fma(d0, d0, d1 * d1)));
   T cd = P.c_drag * T(kPi) * r * r * P.rho_f * sp;
-  F[0] = cd * d0 - V * gp[0];
-  F[1] = cd * d1 - V * gp[1];
-  F[2] = cd * d2 - V * gp[2];
+  F[0] = fma(cd, d0, -(V * gp[0]));
+  F[1] = fma(cd, d1, -(V * gp[1]));
+  F[2] = fma(cd, d2, -(V * gp[2]));
   if (P.rho_f > T(0)) {
-    a[0] = P.g[0] - gp[0] * P.inv_rho_f;
-    a[1] = P.g[1] - gp[1] * P.inv_rho_f;
-    a[2] = P.g[2] - gp[2] * P.inv_rho_f;
+    a[0] = fma(-gp[0], P.inv_rho_f, P.g[0]);
+    a[1] = fma(-gp[1], P.inv_rho_f, P.g[1]);
+    a[2] = fma(-gp[2], P.inv_rho_f, P.g[2]);
   } else {
     a[0] = P.g[0];
     a[1] = P.g[1];

@@ -9,7 +9,7 @@ namespace gic {
 
 template <typename T>
 struct Masses {
-  T m, ma;
+  T m, ma, sum;  // granule, added mass, their sum (rounded once)
 };
 
 template <typename T>
@@ -18,6 +18,7 @@ __device__ __forceinline__ Masses<T> masses(const DParams<T>& P, T r) {
   Masses<T> M;
   M.m = P.rho_s * V;
   M.ma = P.vm ? T(0.5) * P.rho_f * V : T(0);
+  M.sum = fma(P.rho_s, V, M.ma);
   return M;
 }
 
@@ -48,11 +49,11 @@ __device__ __forceinline__ void advance_axis(const DGrid& G, float dt, float v, 
 
 __device__ __forceinline__ void advance_axis(const DGrid& G, double dt, double v, double o, int c, int nc,
                                              double& o_out, int& c_out, uint32_t& flags) {
-  double x = o + dt * v;
+  double x = fma(dt, v, o);
   double sh = floor(x * G.inv_hc);
   if (!(fabs(sh) < 1e9)) sh = x > 0 ? 1e9 : -1e9;
   long long shift = (long long)sh;
-  x -= sh * G.hc;
+  x = fma(-sh, G.hc, x);
   // guard against rounding just outside [0, h_c)
   if (x < 0.0) x = 0.0;
   if (x >= G.hc) x = nextafter(G.hc, 0.0);
@@ -79,11 +80,11 @@ __device__ __forceinline__ void integrate_granule(const DGrid& G, const DParams<
                                                   T fa0, T fa1, T fa2, int32_t& c_out, pos_t<T>& p_out,
                                                   vec_t<T>& v_out, T& fe0, T& fe1, T& fe2, uint32_t& flags) {
   Masses<T> M = masses(P, radius_of(p));
-  T inv = T(1) / (M.m + M.ma);
-  T a0 = (fc0 + ff0 + M.m * P.g[0] + M.ma * fa0) * inv;
-  T a1 = (fc1 + ff1 + M.m * P.g[1] + M.ma * fa1) * inv;
-  T a2 = (fc2 + ff2 + M.m * P.g[2] + M.ma * fa2) * inv;
-  T v0 = v.x + P.dt * a0, v1 = v.y + P.dt * a1, v2 = v.z + P.dt * a2;
+  T inv = T(1) / M.sum;
+  T a0 = fma(M.ma, fa0, fma(M.m, P.g[0], fc0 + ff0)) * inv;
+  T a1 = fma(M.ma, fa1, fma(M.m, P.g[1], fc1 + ff1)) * inv;
+  T a2 = fma(M.ma, fa2, fma(M.m, P.g[2], fc2 + ff2)) * inv;
+  T v0 = fma(P.dt, a0, v.x), v1 = fma(P.dt, a1, v.y), v2 = fma(P.dt, a2, v.z);
   if (!isfinite(v0) || !isfinite(v1) || !isfinite(v2)) flags |= GIC_STATUS_NONFINITE;
   int c3[3] = {cell_x(c), cell_y(c), cell_z(c)};
   int cn[3];
@@ -93,9 +94,9 @@ __device__ __forceinline__ void integrate_granule(const DGrid& G, const DParams<
   advance_axis(G, P.dt, v2, p.z, c3[2], G.nc[2], p_out.z, cn[2], flags);
   c_out = pack_cell(cn[0], cn[1], cn[2]);
   v_out = make_vec<T>(v0, v1, v2);
-  fe0 = ff0 + M.ma * (fa0 - a0);
-  fe1 = ff1 + M.ma * (fa1 - a1);
-  fe2 = ff2 + M.ma * (fa2 - a2);
+  fe0 = fma(M.ma, fa0 - a0, ff0);
+  fe1 = fma(M.ma, fa1 - a1, ff1);
+  fe2 = fma(M.ma, fa2 - a2, ff2);
 }
 
 // Adjoint of integrate_granule: from the gradients gx, gv, gf of (x', v',
@@ -111,7 +112,7 @@ template <typename T>
 __device__ __forceinline__ IntegrateAdj<T> integrate_adj_granule(const DParams<T>& P, T r, const vec_t<T>& gx,
                                                                  const vec_t<T>& gv, const vec_t<T>& gf) {
   const Masses<T> M = masses(P, r);
-  const T inv = T(1) / (M.m + M.ma);
+  const T inv = T(1) / M.sum;
   IntegrateAdj<T> o;
   const T x[3] = {gx.x, gx.y, gx.z}, v[3] = {gv.x, gv.y, gv.z}, f[3] = {gf.x, gf.y, gf.z};
 #pragma unroll

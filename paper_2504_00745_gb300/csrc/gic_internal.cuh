@@ -43,7 +43,6 @@ struct alignas(32) d4 {
 // error reporting (thread-local text) and launch accounting
 int set_error(int code, const char* fmt, ...);
 void count_launches(int64_t k);
-void set_capturing(bool on);
 int wait_stream(cudaStream_t stream, int64_t timeout_ms, const char* what);
 uint32_t* status_word();  // device address of the sticky status word (current device)
 
@@ -118,15 +117,19 @@ int make_grid(const GicGrid* g, DGrid* out);
 template <typename T>
 int make_params(const GicParams* p, DParams<T>* out);
 int check_granules(const GicGranules* s, const char* what, bool need_id = false);
-// gic_sort gated by two device words (see gic_sort.cu)
-int sort_gated(const GicGrid* grid, const GicGranules* in, GicGranules* out, int32_t* perm, void* cell_table, void* ws,
-               size_t ws_bytes, const uint32_t* gate, cudaStream_t stream);
 // per-granule vectors are real[4n]: 16-byte (FP32) / 32-byte (FP64) aligned
 int check_vecs(int32_t precision, const char* what, std::initializer_list<const void*> ptrs);
 
 inline unsigned grid_blocks(int64_t n, int threads) { return (unsigned)((n + threads - 1) / threads); }
 
 // ----------------------------------------------------------------- device side
+
+// A product that is never contracted into a fused multiply-add with what
+// follows: kernels that share a formula (the fused substep and the
+// separate entry points) then round it the same way, whatever the compiler
+// sees around it.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
 __device__ __forceinline__ int cell_x(int32_t c) { return c & (kMaxCellsPerAxis - 1); }
 __device__ __forceinline__ int cell_y(int32_t c) { return (c >> kCellBits) & (kMaxCellsPerAxis - 1); }
@@ -268,11 +271,11 @@ __device__ __forceinline__ int mac_of(const DGrid& G, int c) { return (int)(((ui
 
 __device__ __forceinline__ float mac_frac(const DGrid& G, int c, int m, uint32_t q) {
   int sub = c - m * G.k;
-  return ((float)sub + (float)q * 0x1p-30f) * G.inv_k_f;
+  return mul_rn((float)sub + (float)q * 0x1p-30f, G.inv_k_f);
 }
 __device__ __forceinline__ double mac_frac(const DGrid& G, int c, int m, double o) {
   int sub = c - m * G.k;
-  return ((double)sub * G.hc + o) * G.inv_dx;
+  return mul_rn(fma((double)sub, G.hc, o), G.inv_dx);
 }
 // FP64 fraction from the fixed-point state (used where the volume fraction is
 // accumulated in FP64): exact integer numerator, one rounding.

@@ -95,7 +95,7 @@ __device__ __forceinline__ T interp(const Stencil3<T>& S, Load load, T inv_dx, T
         T wx = a ? S.w[0] : T(1) - S.w[0];
         T wy = b ? S.w[1] : T(1) - S.w[1];
         T wz = c ? S.w[2] : T(1) - S.w[2];
-        acc += wx * wy * wz * f;
+        acc = fma(wx * wy * wz, f, acc);
         if (grad) {
           g0 += (a ? T(1) : T(-1)) * wy * wz * f;
           g1 += wx * (b ? T(1) : T(-1)) * wz * f;

@@ -5,15 +5,13 @@
 // and the P2G scatter of F_s at the old positions and, when asked, of
 // alpha_s at the new ones.  The per-granule force arrays of the separate
 // entry points (F_c, F_fl, a_f, f_ex) never leave registers.
-#include <string.h>
-
-#include <mutex>
 #include <type_traits>
 
 #include "gic_capillary.cuh"
 #include "gic_contact.cuh"
 #include "gic_grid.cuh"
 #include "gic_integrate.cuh"
+#include "gic_tile.cuh"
 
 namespace gic {
 
@@ -21,21 +19,124 @@ constexpr int kSubstepThreads = 256;
 static_assert(kSubstepThreads == 32 * kSubWarps && kSubstepThreads + kSubstepThreads / 32 <= kSpreadStride,
               "the shared tile's warp arrays and the spread deposits are sized for CTAs of 256 threads");
 
-// kKeep: the kernel of gic_step's list-keeping branch without the capillary
-// force (its lists are valid by the branch's condition, so it carries neither
-// the build nor the bridge code: a smaller instruction footprint); otherwise
-// the general kernel, which reads from the list flags whether it rebuilds.
-// kNoAlpha: a call without alpha_s (the kernel then carries none of its code).
-template <typename T, bool kKeep, bool kNoAlpha = false>
-__global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2) k_substep(
-    DGrid G, DParams<T> P, int64_t n, const int32_t* __restrict__ cell, const pos_t<T>* __restrict__ pos,
-    const float4* __restrict__ posf, const vec_t<T>* __restrict__ vel, const int32_t* __restrict__ id, NbDev nb,
-    const uint4* __restrict__ table, T skin, Fields<T> Fd, int32_t* __restrict__ cell_out, pos_t<T>* __restrict__ pos_out,
-    vec_t<T>* __restrict__ vel_out, int32_t* __restrict__ id_out, float4* __restrict__ posf_out,
-    vec_t<T>* __restrict__ fex_out, double* __restrict__ alpha, T* __restrict__ Fs_u, T* __restrict__ Fs_v,
-    T* __restrict__ Fs_w, double* __restrict__ sums, uint32_t* status) {
-  __shared__ std::conditional_t<sizeof(T) == 4, SubTile, int> sh;  // FP32 path only
-  const bool rebuild = !kKeep && (nb.flags[kNbRebuild] | nb.flags[kNbSticky]) != 0u;  // uniform over the launch
+// The granule arrays a substep reads.
+template <typename T>
+struct StateIn {
+  const int32_t* cell;
+  const pos_t<T>* pos;
+  const float4* posf;
+  const vec_t<T>* vel;
+  const int32_t* id;
+};
+
+template <typename T>
+static StateIn<T> state_in(const GicGranules* s) {
+  return StateIn<T>{s->cell, (const pos_t<T>*)s->pos, sizeof(T) == 4 ? (const float4*)s->posf : nullptr,
+                    (const vec_t<T>*)s->vel, s->id};
+}
+
+// The shared memory of a substep CTA: the tile (FP32), and before it, in a
+// gic_step call that rebuilds, the staged neighbourhood of the list build.
+// Dynamic, so that the out-of-line build addresses it as shared memory.
+extern __shared__ __align__(16) unsigned char g_substep_smem[];
+constexpr size_t kBuildSmem = sizeof(TileShared<kSubstepThreads>);
+constexpr size_t kSubTileSmem = sizeof(SubTile) > kBuildSmem ? sizeof(SubTile) : kBuildSmem;
+static_assert(kSubTileSmem <= 48 * 1024, "more shared memory than a kernel has without asking");
+
+// Contact (and bridge) force of sorted granule i from the 27 cells, walls
+// excluded, into vel_out[i] (which the granule's own thread reads and then
+// overwrites): for a granule whose row overflowed.
+template <typename T, bool kCap>
+__device__ __forceinline__ void contact_walk(const DGrid& G, const DParams<T>& P, const StateIn<T>& S, const T* af,
+                                             const uint4* table, uint32_t epoch, int64_t i, vec_t<T>* vel_out,
+                                             uint32_t* status) {
+  const int32_t* cell = S.cell;
+  const pos_t<T>* pos = S.pos;
+  const vec_t<T>* vel = S.vel;
+  const int32_t ci = cell[i];
+  const int cx = cell_x(ci), cy = cell_y(ci), cz = cell_z(ci);
+  const pos_t<T> pi = pos[i];
+  const vec_t<T> vi = vel[i];
+  const T ri = radius_of(pi);
+  const T mi = granule_mass(P, ri);
+  T F0 = T(0), F1 = T(0), F2 = T(0);
+  bool coincident = false;
+  auto contact = [&](int64_t j, const PairGeom<T>& g) {
+    add_force(P, g, vi, ldg(&vel[j]), mi, radius_of(ldg(&pos[j])), F0, F1, F2, coincident);
+  };
+  if constexpr (kCap) {
+    const T sri = moisture_ratio_at(G, P, af, ci, pi, (T*)nullptr);
+    for_each_partner(G, table, epoch, i, cx, cy, cz, [&](int64_t j, int ox, int oy, int oz) {
+      const pos_t<T> pj = ldg(&pos[j]);
+      const T rj = radius_of(pj);
+      PairGeom<T> g;
+      if (!pair_within(G, pi, pj, ox, oy, oz, ri, rj, P.kappa * (ri + rj), g)) return;
+      if (g.overlap > T(0))
+        contact(j, g);
+      else
+        add_bridge(P, g, ri, rj, sri,
+                   moisture_ratio_at(G, P, af, pack_cell(cx + ox, cy + oy, cz + oz), pj, (T*)nullptr), F0, F1, F2);
+    });
+  } else {
+    for_each_contact<T>(G, table, epoch, i, cx, cy, cz, pi, ri, pos, S.posf, contact);
+  }
+  if (coincident) raise_status(status, GIC_STATUS_COINCIDENT);
+  vel_out[i] = make_vec<T>(F0, F1, F2);
+}
+
+// The CTA's share of a rebuild: the rows of its granules of the sorted state
+// (each is read only by its own granule's thread, so no CTA waits for
+// another's).  Out of line, at the kernel's start: it costs the calls that keep
+// their lists no registers, and no launch of its own (an idle launch of one CTA
+// per 128 granules costs 2.3 ns per CTA: 20 us of every call on 1M granules).
+// The references are to the kernel's parameters.
+template <typename T, bool kCap>
+static __device__ __noinline__ void step_build(const DGrid& G, const DParams<T>& P, const StateIn<T>& S,
+                                               const NbDev& nb, int64_t n, const T* af, const uint4* table, T skin,
+                                               vec_t<T>* vel_out, uint32_t* status) {
+  TileShared<kSubstepThreads>& sh = *reinterpret_cast<TileShared<kSubstepThreads>*>(g_substep_smem);
+  const uint32_t epoch = __ldg(&table[0].x);
+  const int64_t i = blockIdx.x * (int64_t)kSubstepThreads + threadIdx.x;
+  const bool valid = i < n;
+  const int32_t ci = valid ? __ldg(&S.cell[i]) : 0;
+  const FloatPos<T> fpos{S.cell, S.pos, S.posf, G.inv_hc};
+  const TileBox B = tile_stage<kSubstepThreads, T>(sh, G, table, epoch, fpos, valid, ci);
+  const bool over = build_row<kSubstepThreads, T, kCap, true>(sh, B, G, n, i, ci, fpos, S.id, table, epoch, nb,
+                                                              (float)skin, (float)(T(1) + P.kappa));
+  if (over) contact_walk<T, kCap>(G, P, S, af, table, epoch, i, vel_out, status);
+  __syncthreads();  // the shared memory is the tile's from here on
+}
+
+// kMode: kGeneral is gic_substep's kernel, which reads from the list flags
+// whether it rebuilds; kStep and kStepCap are gic_step's, without and with the
+// capillary force: in a call that rebuilds they read `sorted` and build its rows
+// first, out of line, so that the other calls' path carries no build code (a
+// smaller instruction footprint: 1317 -> 1286 us on the 16M sweep).  kNoAlpha: a call without alpha_s (the kernel then carries none of
+// its code).
+enum SubMode { kGeneral, kStep, kStepCap };
+
+template <typename T, int kMode, bool kNoAlpha = false>
+__global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2)
+    k_substep(const __grid_constant__ DGrid G, const __grid_constant__ DParams<T> P, int64_t n,
+              const __grid_constant__ StateIn<T> state, const __grid_constant__ StateIn<T> sorted,
+              const __grid_constant__ NbDev nb, const uint4* __restrict__ table, T skin, Fields<T> Fd,
+              int32_t* __restrict__ cell_out, pos_t<T>* __restrict__ pos_out, vec_t<T>* __restrict__ vel_out,
+              int32_t* __restrict__ id_out, float4* __restrict__ posf_out, vec_t<T>* __restrict__ fex_out,
+              double* __restrict__ alpha, T* __restrict__ Fs_u, T* __restrict__ Fs_v, T* __restrict__ Fs_w,
+              double* __restrict__ sums, uint32_t* status) {
+  // uniform over the launch
+  const bool resorted = kMode != kGeneral && step_rebuilds(nb.flags);
+  const bool rebuild = kMode == kGeneral && (nb.flags[kNbRebuild] | nb.flags[kNbSticky]) != 0u;
+  const StateIn<T> S = resorted ? sorted : state;
+  const int32_t* __restrict__ cell = S.cell;
+  const pos_t<T>* __restrict__ pos = S.pos;
+  const float4* __restrict__ posf = S.posf;
+  const vec_t<T>* __restrict__ vel = S.vel;
+  const int32_t* __restrict__ id = S.id;
+  if constexpr (kMode != kGeneral)
+    if (resorted)
+      step_build<T, kMode == kStepCap>(G, P, sorted, nb, n, Fd.af, table, skin, vel_out, status);
+  SubTile& sh = *reinterpret_cast<SubTile*>(g_substep_smem);  // FP32 path only
   const bool do_a = !kNoAlpha && alpha != nullptr, do_f = Fs_u != nullptr;
   const int64_t i = blockIdx.x * (int64_t)kSubstepThreads + threadIdx.x;
   const bool valid = i < n;
@@ -75,11 +176,16 @@ __global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2) k_sub
       const int cx = cell_x(ci), cy = cell_y(ci), cz = cell_z(ci);
       const bool has_f = sizeof(T) == 4 && posf != nullptr;
       const float4 fi = has_f ? __ldg(&posf[i]) : make_float4(0.f, 0.f, 0.f, 0.f);
-      if (!kKeep && P.cap) {  // with the capillary bridges (Sec. 5.4): contacts and bridge candidates
+      if (kMode != kGeneral && nb.count[i] < 0) {  // the row overflowed: step_build left the force here
+        const vec_t<T> Fc = vel_out[i];
+        F0 = Fc.x;
+        F1 = Fc.y;
+        F2 = Fc.z;
+      } else if (kMode == kStepCap || (kMode == kGeneral && P.cap)) {  // with the capillary bridges (Sec. 5.4): contacts and bridge candidates
         const T sri = moisture_ratio_at(G, P, Fd.af, ci, pi, (T*)nullptr);
         auto near = [&](int64_t j, int32_t cj, const pos_t<T>& pj, const PairGeom<T>& g) {
           if (g.overlap > T(0))
-            add_force(P, g, vi, ldg(&vel[j]), mi, granule_mass(P, radius_of(pj)), F0, F1, F2, coincident);
+            add_force(P, g, vi, ldg(&vel[j]), mi, radius_of(pj), F0, F1, F2, coincident);
           else
             add_bridge(P, g, ri, radius_of(pj), sri, moisture_ratio_at(G, P, Fd.af, cj, pj, (T*)nullptr), F0, F1,
                        F2);
@@ -122,8 +228,7 @@ __global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2) k_sub
     vel_out[i] = vo;
     if (id_out && id) id_out[i] = id[i];
     if constexpr (sizeof(T) == 4) {
-      if (posf_out)
-        posf_out[i] = posf_of(co, po);
+      if (posf_out) posf_out[i] = posf_of(co, po);
     }
     if (fex_out) fex_out[i] = make_vec<T>(fe[0], fe[1], fe[2]);
     // the next call's displacement test, on the positions just written
@@ -136,7 +241,8 @@ __global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2) k_sub
                       nb_lim2(nb, T(0)));
     }
   }
-  if (__any_sync(0xffffffffu, far) && lane_id() == 0) atomicOr(&nb.flags[kNbNext], 1u);
+  const bool cta_far = __any_sync(0xffffffffu, far) && lane_id() == 0;
+  if (kMode == kGeneral && cta_far) atomicOr(&nb.flags[kNbNext], 1u);
 
   // a5: P2G
   if constexpr (sizeof(T) == 4) {
@@ -168,7 +274,7 @@ __global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2) k_sub
     if (spread && inv_unit != 0.f) {
       spread_deposit(sh, B, G, Fs, inv_unit);
     } else if (kNoAlpha && valid && do_f) {  // inv_unit == 0 here: no tile for F_s
-      fs_deposit_global(G, Fs_u, Fs_v, Fs_w, ci, pi, fc[0], fc[1], fc[2]);
+      fs_deposit_global(G, Fs[0], Fs[1], Fs[2], ci, pi, fc[0], fc[1], fc[2]);
     } else if (valid && do_f) {
       int m[3];
       float t[3];
@@ -228,7 +334,10 @@ __global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2) k_sub
       if (threadIdx.x == 0) atomicAdd(&sums[1], s);
     }
   }
-  verlet_call_done(nb, rebuild);
+  if constexpr (kMode == kGeneral)
+    verlet_call_done(nb, rebuild);
+  else
+    step_call_done(nb, resorted, cta_far);
 }
 
 constexpr int kSubstepAdjThreads = 128;
@@ -280,9 +389,8 @@ __global__ void __launch_bounds__(kSubstepAdjThreads, sizeof(T) == 4 ? 6 : 3) k_
       const T rj = radius_of(ldg(&pos[j]));
       const IntegrateAdj<T> oj =
           integrate_adj_granule(P, rj, ldg(&gxo[j]), ldg(&gvo[j]), gfe ? ldg(&gfe[j]) : zero);
-      const T mj = granule_mass(P, rj);
       gm += pair_force_adj(P, g.x0, g.x1, g.x2, g.d, g.overlap, vi.x - vj.x, vi.y - vj.y, vi.z - vj.z,
-                           mi * mj / (mi + mj), l0 - oj.gFc[0], l1 - oj.gFc[1], l2 - oj.gFc[2], l0, l1, l2, gx[0],
+                           pair_mass(P, mi, rj), l0 - oj.gFc[0], l1 - oj.gFc[1], l2 - oj.gFc[2], l0, l1, l2, gx[0],
                            gx[1], gx[2], gv[0], gv[1], gv[2]);
     };
     const int cx = cell_x(ci), cy = cell_y(ci), cz = cell_z(ci);
@@ -364,48 +472,45 @@ using namespace gic;
 
 namespace gic {
 
-// [zero alpha_s] -> k_substep (sorted -> next) -> [alpha_s out]; counts its
-// launches into *launches.
-static int substep_launch(const DGrid& G, const GicParams* params, const GicGranules* s, const void* cell_table,
-                          const GicNeighbors* nb, const NbDev& d, const void* u, const void* v, const void* w,
-                          const void* p, const void* alpha_f, GicGranules* next, void* f_ex, double* alpha_s,
-                          void* Fs_u, void* Fs_v, void* Fs_w, double* sums2, cudaStream_t stream, int* launches,
-                          bool keep = false, void* scratch = nullptr) {
+// [zero alpha_s] -> k_substep -> [alpha_s out].  sorted: null for gic_substep
+// (the substep of s); else gic_step's, which reads `sorted` in a call that
+// rebuilt and s otherwise.
+static int substep_launch(const DGrid& G, const GicParams* params, const GicGranules* s, const GicGranules* sorted,
+                          const void* cell_table, const GicNeighbors* nb, const NbDev& d, const void* u, const void* v,
+                          const void* w, const void* p, const void* alpha_f, GicGranules* next, void* f_ex,
+                          double* alpha_s, void* Fs_u, void* Fs_v, void* Fs_w, double* sums2, cudaStream_t stream,
+                          void* scratch = nullptr) {
   int rc;
   const int64_t ncell = (int64_t)G.nx * G.ny * G.nz;
-  if (alpha_s) {
-    alpha_begin(alpha_s, ncell, sums2, stream, scratch);
-    ++*launches;
-  }
+  if (alpha_s && (rc = alpha_begin(alpha_s, ncell, sums2, stream, scratch))) return rc;
   if (s->n > 0) {
     const unsigned blocks = grid_blocks(s->n, kSubstepThreads);
+    auto go = [&](auto t, auto* kern, const DParams<decltype(t)>& P, size_t smem) {
+      using T = decltype(t);
+      kern<<<blocks, kSubstepThreads, smem, stream>>>(
+          G, P, s->n, state_in<T>(s), state_in<T>(sorted ? sorted : s), d, (const uint4*)cell_table, (T)nb->skin,
+          fields<T>(u, v, w, p, alpha_f), next->cell, (pos_t<T>*)next->pos, (vec_t<T>*)next->vel, next->id,
+          sizeof(T) == 4 ? (float4*)next->posf : nullptr, (vec_t<T>*)f_ex, alpha_s, (T*)Fs_u, (T*)Fs_v, (T*)Fs_w,
+          sums2, status_word());
+    };
     if (s->precision == GIC_FP32) {
       DParams<float> P;
       if ((rc = make_params(params, &P))) return rc;
-      auto kern = !(keep && !P.cap) ? k_substep<float, false>
-                  : alpha_s             ? k_substep<float, true>
-                                        : k_substep<float, true, true>;
-      kern<<<blocks, kSubstepThreads, 0, stream>>>(
-          G, P, s->n, s->cell, (const uint4*)s->pos, (const float4*)s->posf, (const float4*)s->vel, s->id, d,
-          (const uint4*)cell_table, (float)nb->skin, fields<float>(u, v, w, p, alpha_f), next->cell,
-          (uint4*)next->pos, (float4*)next->vel, next->id, (float4*)next->posf, (float4*)f_ex, alpha_s,
-          (float*)Fs_u, (float*)Fs_v, (float*)Fs_w, sums2, status_word());
+      go(0.f,
+         !sorted   ? k_substep<float, kGeneral>
+         : P.cap   ? k_substep<float, kStepCap>
+         : alpha_s ? k_substep<float, kStep>
+                   : k_substep<float, kStep, true>,
+         P, kSubTileSmem);
     } else {
       DParams<double> P;
       if ((rc = make_params(params, &P))) return rc;
-      auto kern = keep && !P.cap ? k_substep<double, true> : k_substep<double, false>;
-      kern<<<blocks, kSubstepThreads, 0, stream>>>(
-          G, P, s->n, s->cell, (const d4*)s->pos, nullptr, (const d4*)s->vel, s->id, d, (const uint4*)cell_table,
-          nb->skin, fields<double>(u, v, w, p, alpha_f), next->cell, (d4*)next->pos, (d4*)next->vel, next->id,
-          nullptr, (d4*)f_ex, alpha_s, (double*)Fs_u, (double*)Fs_v, (double*)Fs_w, sums2, status_word());
+      go(0.0, !sorted ? k_substep<double, kGeneral> : P.cap ? k_substep<double, kStepCap> : k_substep<double, kStep>, P,
+         sorted ? kBuildSmem : 0);
     }
     count_launches(1);
-    ++*launches;
   }
-  if (alpha_s) {
-    alpha_end(G, s->precision, alpha_s, ncell, sums2, stream, scratch);
-    ++*launches;
-  }
+  if (alpha_s && (rc = alpha_end(G, s->precision, alpha_s, ncell, sums2, stream, scratch))) return rc;
   return GIC_OK;
 }
 
@@ -436,172 +541,12 @@ extern "C" int gic_substep(const GicGrid* grid, const GicParams* params, const G
   if ((rc = check_vecs(s->precision, "gic_substep", {f_ex}))) return rc;
   NbDev d;
   if ((rc = verlet_prelude(G, params, s, cell_table, nb, nullptr, stream, "gic_substep", &d, false))) return rc;
-  int launches = 0;
-  if ((rc = substep_launch(G, params, s, cell_table, nb, d, u, v, w, p, alpha_f, next, f_ex, alpha_s, Fs_u, Fs_v, Fs_w,
-                           sums2, (cudaStream_t)stream, &launches)))
+  if ((rc = substep_launch(G, params, s, nullptr, cell_table, nb, d, u, v, w, p, alpha_f, next, f_ex, alpha_s, Fs_u,
+                           Fs_v, Fs_w, sums2, (cudaStream_t)stream)))
     return rc;
   GIC_CHECK_LAUNCH("gic_substep");
   return GIC_OK;
 }
-
-namespace gic {
-
-// gic_step's decision: this call rebuilds the lists (and sorts) when the
-// previous call's k_substep left a granule beyond skin / 2 of its reference,
-// or a rebuild was requested.  Sets the two branches' conditionals.
-__global__ void k_step_decide(uint32_t* flags, cudaGraphConditionalHandle rebuild, cudaGraphConditionalHandle keep) {
-  const unsigned r = (flags[kNbNext] | flags[kNbSticky]) != 0u ? 1u : 0u;
-  flags[kNbRebuild] = r;
-  flags[kNbNext] = 0u;
-  cudaGraphSetConditional(rebuild, r);
-  cudaGraphSetConditional(keep, 1u - r);
-}
-
-// Everything a gic_step graph depends on; a call with the same bytes reuses
-// the instantiated graph.
-struct StepKey {
-  GicGrid grid;
-  GicParams params;
-  GicGranules state, next, sorted;
-  GicNeighbors nb;
-  const void* ptr[13];
-  size_t ws_bytes;
-};
-
-struct StepGraph {
-  bool used = false;
-  uint64_t last = 0;
-  StepKey key;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  int launches = 0;  // kernels every launch runs (the sort's are not counted)
-};
-
-constexpr int kStepGraphs = 8;
-static StepGraph g_step_graphs[kStepGraphs];
-static uint64_t g_step_clock = 0;
-static std::mutex g_step_mu;
-
-static bool same_key(const StepKey& a, const StepKey& b) { return memcmp(&a, &b, sizeof(StepKey)) == 0; }
-
-static void store_key(StepKey& k, const GicGrid* grid, const GicParams* params, const GicGranules* state,
-                      const GicGranules* next, const GicGranules* sorted, const GicNeighbors* nb,
-                      const void* const ptr[13], size_t ws_bytes) {
-  memset(&k, 0, sizeof(k));  // padding bytes take part in the comparison
-  memcpy(&k.grid, grid, sizeof(GicGrid));
-  memcpy(&k.params, params, sizeof(GicParams));
-  memcpy(&k.state, state, sizeof(GicGranules));
-  memcpy(&k.next, next, sizeof(GicGranules));
-  memcpy(&k.sorted, sorted, sizeof(GicGranules));
-  memcpy(&k.nb, nb, sizeof(GicNeighbors));
-  for (int i = 0; i < 13; ++i) k.ptr[i] = ptr[i];
-  k.ws_bytes = ws_bytes;
-}
-
-// Adds an IF node on `dep` with handle h and captures fill(stream) into its body.
-template <typename Fill>
-static int add_branch(cudaGraph_t g, cudaGraphNode_t dep, cudaGraphConditionalHandle h, cudaStream_t cs, Fill&& fill) {
-  cudaGraphNodeParams cp = {};
-  cp.type = cudaGraphNodeTypeConditional;
-  cp.conditional.handle = h;
-  cp.conditional.type = cudaGraphCondTypeIf;
-  cp.conditional.size = 1;
-  cudaGraphNode_t cond;
-  if (cudaGraphAddNode(&cond, g, &dep, nullptr, 1, &cp) != cudaSuccess)
-    return set_error(GIC_ERR_CUDA, "gic_step: conditional node failed");
-  cudaGraph_t body = cp.conditional.phGraph_out[0];
-  cudaGraph_t got = nullptr;
-  if (cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) != cudaSuccess)
-    return set_error(GIC_ERR_CUDA, "gic_step: graph capture failed");
-  int rc = fill(cs);
-  if (cudaStreamEndCapture(cs, &got) != cudaSuccess && rc == GIC_OK)
-    rc = set_error(GIC_ERR_CUDA, "gic_step: graph capture failed");
-  return rc;
-}
-
-// Builds the graph of one gic_step configuration:
-//   decide -> IF rebuild: sort (state -> sorted) -> [zero alpha] -> k_substep (sorted -> next) -> [alpha out]
-//          -> IF keep:    [zero alpha] -> k_substep (state -> next) -> [alpha out]
-static int build_step_graph(StepGraph& sg, const DGrid& G, const GicGrid* grid, const GicParams* params,
-                            const GicGranules* state, GicGranules* next, GicGranules* sorted, int32_t* perm,
-                            void* cell_table, void* ws, size_t ws_bytes, const GicNeighbors* nb, const NbDev& d,
-                            const void* u, const void* v, const void* w, const void* p, const void* alpha_f,
-                            double* alpha_s, void* Fs_u, void* Fs_v, void* Fs_w, double* sums2) {
-  int rc = GIC_OK;
-  cudaGraph_t g = nullptr;
-  cudaGraphExec_t ex = nullptr;
-  cudaStream_t cs = nullptr;
-  cudaGraph_t got = nullptr;
-  cudaGraphConditionalHandle h_rebuild, h_keep;
-  int launches = 0;
-  status_word();  // resolve the device address before capturing
-  if ((rc = alpha_prepare())) return rc;
-  if (cudaGraphCreate(&g, 0) != cudaSuccess) return set_error(GIC_ERR_CUDA, "gic_step: cudaGraphCreate failed");
-  if (cudaGraphConditionalHandleCreate(&h_rebuild, g, 0, cudaGraphCondAssignDefault) != cudaSuccess ||
-      cudaGraphConditionalHandleCreate(&h_keep, g, 0, cudaGraphCondAssignDefault) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
-    cudaGetLastError();
-    cudaGraphDestroy(g);
-    return set_error(GIC_ERR_CUDA, "gic_step: graph setup failed");
-  }
-  set_capturing(true);
-  do {
-    // 1. the decision
-    if (cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
-      rc = set_error(GIC_ERR_CUDA, "gic_step: graph capture failed");
-      break;
-    }
-    k_step_decide<<<1, 1, 0, cs>>>(nb->flags, h_rebuild, h_keep);
-    if (cudaStreamEndCapture(cs, &got) != cudaSuccess) {
-      rc = set_error(GIC_ERR_CUDA, "gic_step: graph capture failed");
-      break;
-    }
-    launches += 1;
-    size_t nn = 0;
-    cudaGraphNode_t decide = nullptr;
-    if (cudaGraphGetNodes(g, nullptr, &nn) != cudaSuccess || nn != 1 || cudaGraphGetNodes(g, &decide, &nn) != cudaSuccess) {
-      rc = set_error(GIC_ERR_CUDA, "gic_step: unexpected graph");
-      break;
-    }
-    // 2. the branch that rebuilds: sort, then the substep from the sorted state (its launches not counted)
-    int uncounted = 0;
-    rc = add_branch(g, decide, h_rebuild, cs, [&](cudaStream_t st) {
-      int r = sort_gated(grid, state, sorted, perm, cell_table, ws, ws_bytes, nullptr, st);
-      // FP32 with float copies and the contact law alone: the rows are built on
-      // the staged neighbourhood first, and the substep walks them
-      if (r == GIC_OK && state->precision == GIC_FP32 && sorted->posf && params->sigma == 0.0)
-        r = launch_build_tile(G, sorted, cell_table, d, nb->skin, st);
-      if (r == GIC_OK)
-        r = substep_launch(G, params, sorted, cell_table, nb, d, u, v, w, p, alpha_f, next, nullptr, alpha_s, Fs_u,
-                           Fs_v, Fs_w, sums2, st, &uncounted, false, ws);
-      return r;
-    });
-    if (rc) break;
-    // 3. the branch that keeps the lists: the substep straight from the state
-    rc = add_branch(g, decide, h_keep, cs, [&](cudaStream_t st) {
-      return substep_launch(G, params, state, cell_table, nb, d, u, v, w, p, alpha_f, next, nullptr, alpha_s, Fs_u,
-                            Fs_v, Fs_w, sums2, st, &launches, true, ws);
-    });
-    if (rc) break;
-    if (cudaGraphInstantiate(&ex, g, 0) != cudaSuccess) {
-      rc = set_error(GIC_ERR_CUDA, "gic_step: graph instantiation failed");
-      break;
-    }
-  } while (false);
-  set_capturing(false);
-  cudaStreamDestroy(cs);
-  if (rc) {
-    cudaGetLastError();
-    if (g) cudaGraphDestroy(g);
-    return rc;
-  }
-  sg.graph = g;
-  sg.exec = ex;
-  sg.launches = launches;
-  return GIC_OK;
-}
-
-}  // namespace gic
 
 static bool share_array(const GicGranules* a, const GicGranules* b) {
   return a->cell == b->cell || a->pos == b->pos || a->vel == b->vel || a->id == b->id ||
@@ -639,45 +584,19 @@ extern "C" int gic_step(const GicGrid* grid, const GicParams* params, const GicG
   NbDev d;
   if ((rc = verlet_view(G, state, cell_table, nb, "gic_step", true, &d))) return rc;
   if (state->n == 0) return GIC_OK;
-  {  // arguments of the sort, checked before they are baked into a graph
+  {  // the sort's workspace
     size_t need = 0;
     if ((rc = gic_workspace_size(grid, state->n, state->precision, &need))) return rc;
     if (!ws || ws_bytes < need)
       return set_error(GIC_ERR_WORKSPACE, "gic_step: workspace of %zu bytes needed, %zu given", need, ws_bytes);
     if ((uintptr_t)ws % 256) return set_error(GIC_ERR_ALIGN, "gic_step: workspace must be 256-byte aligned");
   }
-  const void* ptr[13] = {perm, cell_table, ws, u, v, w, p, alpha_f, alpha_s, Fs_u, Fs_v, Fs_w, sums2};
-  StepKey key;
-  store_key(key, grid, params, state, next, sorted, nb, ptr, ws_bytes);
-  std::lock_guard<std::mutex> lock(g_step_mu);
-  StepGraph* hit = nullptr;
-  for (auto& sg : g_step_graphs)
-    if (sg.used && same_key(sg.key, key)) hit = &sg;
-  if (!hit) {
-    StepGraph* slot = &g_step_graphs[0];
-    for (auto& sg : g_step_graphs) {
-      if (!sg.used) {
-        slot = &sg;
-        break;
-      }
-      if (sg.last < slot->last) slot = &sg;
-    }
-    if (slot->used) {
-      cudaGraphExecDestroy(slot->exec);
-      cudaGraphDestroy(slot->graph);
-      slot->used = false;
-    }
-    if ((rc = build_step_graph(*slot, G, grid, params, state, next, sorted, perm, cell_table, ws, ws_bytes, nb, d, u,
-                               v, w, p, alpha_f, alpha_s, Fs_u, Fs_v, Fs_w, sums2)))
-      return rc;
-    memcpy(&slot->key, &key, sizeof(StepKey));
-    slot->used = true;
-    hit = slot;
-  }
-  hit->last = ++g_step_clock;
-  cudaError_t e = cudaGraphLaunch(hit->exec, (cudaStream_t)stream);
-  if (e != cudaSuccess) return set_error(GIC_ERR_CUDA, "gic_step: cudaGraphLaunch: %s", cudaGetErrorString(e));
-  count_launches(hit->launches);
+  const cudaStream_t st = (cudaStream_t)stream;
+  if ((rc = launch_step_sort(G, state, sorted, perm, cell_table, ws, d.flags, st))) return rc;
+  if ((rc = substep_launch(G, params, state, sorted, cell_table, nb, d, u, v, w, p, alpha_f, next, nullptr, alpha_s,
+                           Fs_u, Fs_v, Fs_w, sums2, st, ws)))
+    return rc;
+  GIC_CHECK_LAUNCH("gic_step");
   return GIC_OK;
 }
 

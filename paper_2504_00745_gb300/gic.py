@@ -24,6 +24,7 @@ STATUS_RADIUS = 8
 STATUS_BAD_CELL = 16
 STATUS_FAST = 32
 STATUS_DEBUG_INDEX = 64  # set only by the GIC_DEBUG build
+STATUS_STALL = 128  # a wait inside a kernel ran out of its limit
 
 
 class GicError(RuntimeError):
