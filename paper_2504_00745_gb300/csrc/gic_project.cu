@@ -14,8 +14,8 @@
 // refinement: the solution p and each residual b - A p are FP64 (one FP64
 // stencil pass per refinement step), and each correction A e = r comes from
 // an FP32 conjugate-gradient run, preconditioned by a geometric multigrid
-// V-cycle, to a modest reduction.  The CG iterations run as CUDA graphs of a
-// few iterations between host reads of the stop flag.
+// V-cycle, to a modest reduction.  The CG iterations are queued a few at a time
+// between host reads of the stop flag.
 // Reductions are deterministic: every block writes a partial sum, and the
 // block that finishes last (an atomic ticket, no waiting) adds the partials
 // in index order and writes the scalar that the next kernels read.
@@ -80,12 +80,32 @@ __device__ __forceinline__ bool reduce_last(const double (&v)[NV], double* __res
 struct KahanF {
   float s = 0.f, c = 0.f;
   __device__ __forceinline__ void add(float x) {
-    const float y = x - c;
-    const float t = s + y;
-    c = (t - s) - y;
+    const float y = __fsub_rn(x, c);
+    const float t = __fadd_rn(s, y);
+    c = __fsub_rn(__fsub_rn(t, s), y);
     s = t;
   }
 };
+
+// Sum of the CTA's compensated partials, in double, valid in thread 0: the warps
+// add (hi, lo) float pairs with TwoSum, and only one value per warp takes the
+// FP64 pipe (a tree of double shuffles in every warp cost 3 us of a pass at
+// 128^3).  smem: one double per warp.
+__device__ __forceinline__ double block_sum(const KahanF& k, double* smem) {
+  float h = k.s, l = -k.c;
+  for (int off = 16; off > 0; off >>= 1) {
+    const float h2 = __shfl_down_sync(0xffffffffu, h, off), l2 = __shfl_down_sync(0xffffffffu, l, off);
+    const float t = __fadd_rn(h, h2), b = __fsub_rn(t, h);
+    l = __fadd_rn(__fadd_rn(l, l2), __fadd_rn(__fsub_rn(h, __fsub_rn(t, b)), __fsub_rn(h2, b)));
+    h = t;
+  }
+  if (lane_id() == 0) smem[threadIdx.x >> 5] = (double)h + (double)l;
+  __syncthreads();
+  double r = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += smem[w];
+  return r;
+}
 
 // alpha_f' = 1 - min(alpha_s, alpha_s_max); a NaN alpha_s stays NaN (and is reported)
 __device__ __forceinline__ double target_fraction(double alpha_s, double amax) {
@@ -142,37 +162,28 @@ __global__ void __launch_bounds__(kProjThreads) k_proj_faces64(PGrid g, unsigned
   }
 }
 
-// FP64 residual r = b - A p of system `which` (1: velocity, 2: density);
-// starts the FP32 correction run: r32 = r, e = 0, and arms its stop test.
-// Scalars: ||r||^2 (FP64) and ||b||^2.
-__global__ void __launch_bounds__(kProjThreads) k_proj_residual(
+// Right-hand side b of system `which` (1: velocity, 2: density) in FP64, kept for
+// the solve's later residuals: with p = 0 it is the first residual.  Starts the
+// FP32 correction run: r32 = b, e = 0, and arms its stop test.  Scalars: ||b||^2
+// as ||r||^2 and ||b||^2.
+__global__ void __launch_bounds__(kProjThreads) k_proj_rhs(
     PGrid g, int which, ProjScales S, const double* __restrict__ alpha_s, const float* __restrict__ alpha_star,
     const float* __restrict__ u, const float* __restrict__ v, const float* __restrict__ w,
     const double* __restrict__ fx, const double* __restrict__ fy, const double* __restrict__ fz,
-    const double* __restrict__ p, float* __restrict__ r32, float* __restrict__ e32, double inner_tol2,
+    double* __restrict__ b64, float* __restrict__ r32, float* __restrict__ e32, double inner_tol2,
     double* __restrict__ P, ProjRed* red, uint32_t* status) {
   __shared__ double smem[64];
-  double rr = 0.0, bb = 0.0;
-  const unsigned n = (unsigned)g.n, nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
+  double bb = 0.0;
+  const unsigned n = (unsigned)g.n, nx = g.nx, ny = g.ny, nxy = nx * ny;
   for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-    const unsigned k = c / nxy, rem = c - k * nxy, j = rem / nx, i = rem - j * nx;
-    const unsigned fu = i + (nx + 1) * (j + ny * k), fv = i + nx * (j + (ny + 1) * k);
-    // the six face weights: low and high x, y, z (0 on solid sides)
-    const double w0 = fx[fu], w1 = fx[fu + 1], w2 = fy[fv], w3 = fy[fv + nx], w4 = fz[c], w5 = fz[c + nxy];
-    const double pc = p[c];
-    // (A p)_c as differences (a neighbour beyond an open side is 0)
-    double Ap = 0.0;
-    Ap = fma(w0, i > 0 ? pc - p[c - 1] : pc, Ap);
-    Ap = fma(w1, i + 1 < nx ? pc - p[c + 1] : pc, Ap);
-    Ap = fma(w2, j > 0 ? pc - p[c - nx] : pc, Ap);
-    Ap = fma(w3, j + 1 < ny ? pc - p[c + nx] : pc, Ap);
-    Ap = fma(w4, k > 0 ? pc - p[c - nxy] : pc, Ap);
-    Ap = fma(w5, k + 1 < nz ? pc - p[c + nxy] : pc, Ap);
     double b;
     if (which == 1) {
+      const unsigned k = c / nxy, rem = c - k * nxy, j = rem / nx, i = rem - j * nx;
+      const unsigned fu = i + (nx + 1) * (j + ny * k), fv = i + nx * (j + (ny + 1) * k);
       // b1 = (rho h / dt) (sum over low faces - sum over high faces) of beta v*
-      const double flux = (w0 * (double)u[fu] - w1 * (double)u[fu + 1]) + (w2 * (double)v[fv] - w3 * (double)v[fv + nx]) +
-                          (w4 * (double)w[c] - w5 * (double)w[c + nxy]);
+      const double flux = (fx[fu] * (double)u[fu] - fx[fu + 1] * (double)u[fu + 1]) +
+                          (fy[fv] * (double)v[fv] - fy[fv + nx] * (double)v[fv + nx]) +
+                          (fz[c] * (double)w[c] - fz[c + nxy] * (double)w[c + nxy]);
       b = S.vel * flux;
     } else {
       const double ac = target_fraction(alpha_s[c], S.amax);
@@ -180,17 +191,54 @@ __global__ void __launch_bounds__(kProjThreads) k_proj_residual(
       const double ratio = q < S.rmin ? S.rmin : (q > S.rmax ? S.rmax : q);  // NaN stays NaN
       b = S.den * ac * (1.0 - ratio);
     }
-    const double r = b - Ap;
+    if (!isfinite(b)) raise_status(status, GIC_STATUS_NONFINITE);
+    b64[c] = b;
+    r32[c] = (float)b;
+    e32[c] = 0.f;
+    bb += b * b;
+  }
+  bb = block_sum(bb, smem);
+  const double vals[2] = {bb, bb};
+  double* const outs[2] = {&red->rr64, &red->bb};
+  if (reduce_last<2>(vals, P, red, outs) && threadIdx.x == 0) {  // arm the CG run on this residual
+    red->rr_stop = inner_tol2 * red->rr64;
+    red->done = 0;
+    red->iters = 0;
+  }
+}
+
+// FP64 residual r = b - A p; starts the next FP32 correction run as k_proj_rhs
+// does.  Bound by the FP64 pipe (15 operations per cell; with b formed again in
+// every pass 30): 72 us at 128^3, 140 before.
+__global__ void __launch_bounds__(kProjThreads) k_proj_residual(
+    PGrid g, const double* __restrict__ b64, const double* __restrict__ fx, const double* __restrict__ fy,
+    const double* __restrict__ fz, const double* __restrict__ p, float* __restrict__ r32, float* __restrict__ e32,
+    double inner_tol2, double* __restrict__ P, ProjRed* red, uint32_t* status) {
+  __shared__ double smem[32];
+  double rr = 0.0;
+  const unsigned n = (unsigned)g.n, nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
+  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
+    const unsigned k = c / nxy, rem = c - k * nxy, j = rem / nx, i = rem - j * nx;
+    const unsigned fu = i + (nx + 1) * (j + ny * k), fv = i + nx * (j + (ny + 1) * k);
+    const double pc = p[c];
+    // (A p)_c as differences (a neighbour beyond an open side is 0; solid sides have weight 0)
+    double Ap = 0.0;
+    Ap = fma(fx[fu], i > 0 ? pc - p[c - 1] : pc, Ap);
+    Ap = fma(fx[fu + 1], i + 1 < nx ? pc - p[c + 1] : pc, Ap);
+    Ap = fma(fy[fv], j > 0 ? pc - p[c - nx] : pc, Ap);
+    Ap = fma(fy[fv + nx], j + 1 < ny ? pc - p[c + nx] : pc, Ap);
+    Ap = fma(fz[c], k > 0 ? pc - p[c - nxy] : pc, Ap);
+    Ap = fma(fz[c + nxy], k + 1 < nz ? pc - p[c + nxy] : pc, Ap);
+    const double r = b64[c] - Ap;
     if (!isfinite(r)) raise_status(status, GIC_STATUS_NONFINITE);
     r32[c] = (float)r;
     e32[c] = 0.f;
     rr += r * r;
-    bb += b * b;
   }
-  block_sum2(rr, bb, smem);
-  const double vals[2] = {rr, bb};
-  double* const outs[2] = {&red->rr64, &red->bb};
-  if (reduce_last<2>(vals, P, red, outs) && threadIdx.x == 0) {  // arm the CG run on this residual
+  rr = block_sum(rr, smem);
+  const double vals[1] = {rr};
+  double* const outs[1] = {&red->rr64};
+  if (reduce_last<1>(vals, P, red, outs) && threadIdx.x == 0) {  // arm the CG run on this residual
     red->rr_stop = inner_tol2 * red->rr64;
     red->done = 0;
     red->iters = 0;
@@ -214,6 +262,21 @@ __global__ void __launch_bounds__(kProjThreads) k_proj_residual(
 // positive definite and halves the CG iterations against 1.0), and runs the
 // small levels, down to the coarsest (every axis <= 4 cells, solved by a
 // palindromic sequence of Gauss-Seidel sweeps), in one CTA.
+//
+// A level takes four passes instead of a pass per half sweep and transfer.
+// Down: the red half sweep from x = 0 is invd b, which the black cells form for
+// their neighbours themselves (mg_down); the black cells' residuals then vanish,
+// so the restriction reads the red children alone (mg_restrict).  Up: the black
+// half sweep adds the coarse correction to its red neighbours as it reads them,
+// and its own old value and the red cells' do not outlive the two half sweeps,
+// so the interpolation is never stored (mg_up_black, mg_up_red).  A thread takes
+// the two cells of a pair along x, one of each colour, so that no lane idles on
+// the other colour.  128^3, per CG iteration: level 0 12 + 10 + 10 + 17 us (the
+// last with r . z), the levels below 27 us, the tail 16 us, the CG passes 38 us;
+// bound by the traffic between L2 and L1 (each array about 2.4 times through the
+// halos of 64 x 8 x 4 cells).  Before, with a pass per half sweep and transfer,
+// 230 us in 26 launches (now 16).  Runs of four cells per thread with 16-byte
+// loads measured the same.
 constexpr float kMgOmega = 1.6f;
 constexpr int kMgCoarsePairs = 8;  // (black, red) sweep pairs after the first red sweep on the coarsest level
 constexpr int kMgMaxLevels = 16;
@@ -222,6 +285,8 @@ struct MgLevel {
   int nx, ny, nz;
   float *bx, *by, *bz;  // face weights: (nx+1) ny nz, nx (ny+1) nz, nx ny (nz+1)
   float* invd;          // 1 / (sum of the cell's six face weights)
+  const float* ap;      // level 0: alpha_f', from which its passes form the face weights again
+  unsigned open;        // level 0: the open sides
   float *x, *b;         // correction and right-hand side
 };
 
@@ -235,27 +300,7 @@ __device__ __forceinline__ void level_ijk(const MgLevel& L, unsigned c, unsigned
   i = r - j * nx;
 }
 
-// sum over the cell's interior faces of beta_f x_nb, and the sum of all six
-// face weights
-__device__ __forceinline__ void level_gather(const MgLevel& L, unsigned c, unsigned i, unsigned j, unsigned k,
-                                             const float* __restrict__ x, float& s, float& diag) {
-  const unsigned nx = (unsigned)L.nx, ny = (unsigned)L.ny, nz = (unsigned)L.nz, nxy = nx * ny;
-  const unsigned fx = i + (nx + 1) * (j + ny * k);
-  const unsigned fy = i + nx * (j + (ny + 1) * k);
-  const float wxl = L.bx[fx], wxh = L.bx[fx + 1];
-  const float wyl = L.by[fy], wyh = L.by[fy + nx];
-  const float wzl = L.bz[c], wzh = L.bz[c + nxy];
-  diag = ((wxl + wxh) + (wyl + wyh)) + (wzl + wzh);
-  float t = 0.f;
-  if (i > 0) t = fmaf(wxl, x[c - 1], t);
-  if (i + 1 < nx) t = fmaf(wxh, x[c + 1], t);
-  if (j > 0) t = fmaf(wyl, x[c - nx], t);
-  if (j + 1 < ny) t = fmaf(wyh, x[c + nx], t);
-  if (k > 0) t = fmaf(wzl, x[c - nxy], t);
-  if (k + 1 < nz) t = fmaf(wzh, x[c + nxy], t);
-  s = t;
-}
-
+// sum of the cell's six face weights
 __device__ __forceinline__ float level_diag(const MgLevel& L, unsigned c, unsigned i, unsigned j, unsigned k) {
   const unsigned nx = (unsigned)L.nx, ny = (unsigned)L.ny, nxy = nx * ny;
   const unsigned fx = i + (nx + 1) * (j + ny * k);
@@ -336,113 +381,326 @@ __global__ void __launch_bounds__(kProjThreads) k_mg_diag(MgLevel L) {
   }
 }
 
-// The V-cycle's passes over the cells t0, t0 + stride, ... of a level: the
-// kernels below run them grid-wide, k_mg_tail within one CTA.
+// Pair p of cells along x on a level: cells i0 = 2 p and i0 + 1 of row (j, k),
+// one red ((i + j + k) even) and one black.
+struct MgPair {
+  unsigned j, k, ir, ib;   // x of the red and of the black cell
+  unsigned row;            // index of cell (0, j, k)
+  bool red, black;         // the cell exists (the last pair of an odd row has one)
+};
+__device__ __forceinline__ MgPair mg_pair(const MgLevel& L, unsigned p, unsigned j, unsigned k) {
+  MgPair q;
+  const unsigned odd = (j + k) & 1u;
+  q.j = j;
+  q.k = k;
+  q.ir = 2 * p + odd;
+  q.ib = 2 * p + 1 - odd;
+  q.row = (unsigned)L.nx * (j + (unsigned)L.ny * k);
+  q.red = q.ir < (unsigned)L.nx;
+  q.black = q.ib < (unsigned)L.nx;
+  return q;
+}
 
-// One Gauss-Seidel half sweep: the cells with (i + j + k) % 2 == color get
-// x_c = (b_c + sum beta_f x_nb) / diag_c.  init: x is taken as 0 (the other
-// color is written 0).
-__device__ __forceinline__ void mg_smooth_range(const MgLevel& L, unsigned color, int init, unsigned t0,
-                                                unsigned stride) {
-  const unsigned n = (unsigned)L.nx * L.ny * L.nz;
-  for (unsigned c = t0; c < n; c += stride) {
-    unsigned i, j, k;
-    level_ijk(L, c, i, j, k);
-    if (((i + j + k) & 1u) != color) {
-      if (init) L.x[c] = 0.f;
-      continue;
+// The six face weights of cell (i, j, k): low and high x, y, z.  kAp (level 0):
+// from alpha_f' of the cell and its neighbours, the values k_mg_faces0 stores:
+// 8 MB at 128^3 instead of 25, so that a CG iteration's arrays (67 MB) fit L2.
+// Outside the grid the cell itself stands in (its index q), so that no load
+// waits on a branch.
+struct MgFaces {
+  float w[6];
+};
+struct MgNear {
+  unsigned q[6];  // indices of the six neighbours, the cell's own beyond a side
+  bool in[6];
+};
+__device__ __forceinline__ MgNear mg_near(const MgLevel& L, unsigned c, unsigned i, unsigned j, unsigned k) {
+  const unsigned nx = (unsigned)L.nx, nxy = nx * (unsigned)L.ny;
+  MgNear m;
+  m.in[0] = i > 0, m.in[1] = i + 1 < nx, m.in[2] = j > 0, m.in[3] = j + 1 < (unsigned)L.ny, m.in[4] = k > 0,
+  m.in[5] = k + 1 < (unsigned)L.nz;
+  m.q[0] = m.in[0] ? c - 1 : c, m.q[1] = m.in[1] ? c + 1 : c;
+  m.q[2] = m.in[2] ? c - nx : c, m.q[3] = m.in[3] ? c + nx : c;
+  m.q[4] = m.in[4] ? c - nxy : c, m.q[5] = m.in[5] ? c + nxy : c;
+  return m;
+}
+template <bool kAp>
+__device__ __forceinline__ MgFaces mg_faces(const MgLevel& L, const MgNear& m, unsigned c, unsigned i, unsigned j,
+                                            unsigned k) {
+  MgFaces F;
+  if constexpr (kAp) {
+    const float own = L.ap[c];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+      const float w = 0.5f * (a & 1 ? L.ap[m.q[a]] + own : own + L.ap[m.q[a]]);  // high side + low side
+      F.w[a] = m.in[a] ? w : ((L.open >> a) & 1u ? own : 0.f);
     }
-    float s = 0.f, diag;
-    if (!init) level_gather(L, c, i, j, k, L.x, s, diag);
-    L.x[c] = L.invd[c] * (L.b[c] + s);
+  } else {
+    const unsigned nx = (unsigned)L.nx, ny = (unsigned)L.ny, nxy = nx * ny;
+    const unsigned fx = i + (nx + 1) * (j + ny * k);
+    const unsigned fy = i + nx * (j + (ny + 1) * k);
+    F.w[0] = L.bx[fx], F.w[1] = L.bx[fx + 1], F.w[2] = L.by[fy], F.w[3] = L.by[fy + nx], F.w[4] = L.bz[c],
+    F.w[5] = L.bz[c + nxy];
+  }
+  return F;
+}
+
+// sum over the interior faces of cell (i, j, k) of beta_f f(neighbour), f given
+// the neighbour's index and coordinates.  All loads are in flight together
+// (behind tests of the sides they took 27 cycles per instruction).
+template <bool kAp, typename F>
+__device__ __forceinline__ float mg_gather(const MgLevel& L, unsigned c, unsigned i, unsigned j, unsigned k, F&& f) {
+  const MgNear m = mg_near(L, c, i, j, k);
+  const MgFaces w = mg_faces<kAp>(L, m, c, i, j, k);
+  float v[6];
+#pragma unroll
+  for (int a = 0; a < 6; ++a) {
+    const unsigned d = m.in[a];
+    v[a] = f(m.q[a], a == 0 ? i - d : (a == 1 ? i + d : i), a == 2 ? j - d : (a == 3 ? j + d : j),
+             a == 4 ? k - d : (a == 5 ? k + d : k));
+  }
+  float t = 0.f;
+#pragma unroll
+  for (int a = 0; a < 6; ++a) t = fmaf(m.in[a] ? w.w[a] : 0.f, v[a], t);
+  return t;
+}
+
+// Down: x of both colours from x = 0 (red invd b, black with those).
+template <bool kAp>
+__device__ __forceinline__ void mg_down(const MgLevel& L, const MgPair& q) {
+  if (q.red) L.x[q.row + q.ir] = L.invd[q.row + q.ir] * L.b[q.row + q.ir];
+  if (!q.black) return;
+  const unsigned c = q.row + q.ib;
+  const float s = mg_gather<kAp>(L, c, q.ib, q.j, q.k,
+                            [&](unsigned d, unsigned, unsigned, unsigned) { return L.invd[d] * L.b[d]; });
+  L.x[c] = L.invd[c] * (L.b[c] + s);
+}
+
+// Residual b - A x of the red child in pair (I, j, k) of level F after mg_down:
+// its own row was solved in the red half sweep (with the black cells 0), so
+// what is left is the black neighbours' part.  (The black cells' residuals
+// vanish after theirs.)
+template <bool kAp>
+__device__ __forceinline__ float mg_residual(const MgLevel& F, unsigned I, unsigned j, unsigned k) {
+  if (j >= (unsigned)F.ny || k >= (unsigned)F.nz) return 0.f;
+  const MgPair q = mg_pair(F, I, j, k);
+  if (!q.red) return 0.f;
+  return mg_gather<kAp>(F, q.row + q.ir, q.ir, j, k, [&](unsigned d, unsigned, unsigned, unsigned) { return F.x[d]; });
+}
+
+// Coarse right-hand side of cell (I, J, K), the sum of its children's residuals:
+// four lanes per cell, lane m (of the aligned four) the child row 2 J + (m & 1)
+// of layer 2 K + (m >> 1).
+template <bool kAp>
+__device__ __forceinline__ void mg_restrict(const MgLevel& F, const MgLevel& C, unsigned I, unsigned m, unsigned J,
+                                            unsigned K) {
+  float r = mg_residual<kAp>(F, I, 2 * J + (m & 1u), 2 * K + (m >> 1));
+  const unsigned quad = 0xfu << (lane_id() & 28);
+  r += __shfl_xor_sync(quad, r, 1);
+  r += __shfl_xor_sync(quad, r, 2);
+  if (m == 0) C.b[I + (unsigned)C.nx * (J + (unsigned)C.ny * K)] = r;
+}
+
+// Up, black cells: x_c = invd (b + sum beta_f (x_nb + omega x_coarse(nb's parent))).
+template <bool kAp>
+__device__ __forceinline__ void mg_up_black(const MgLevel& L, const MgLevel& C, const MgPair& q) {
+  if (!q.black) return;
+  const unsigned c = q.row + q.ib;
+  const float s = mg_gather<kAp>(L, c, q.ib, q.j, q.k, [&](unsigned d, unsigned i, unsigned j, unsigned k) {
+    return fmaf(kMgOmega, C.x[(i >> 1) + (unsigned)C.nx * ((j >> 1) + (unsigned)C.ny * (k >> 1))], L.x[d]);
+  });
+  L.x[c] = L.invd[c] * (L.b[c] + s);
+}
+
+// One colour's half sweep at cell (i, j, k).
+template <bool kAp>
+__device__ __forceinline__ float mg_sweep(const MgLevel& L, unsigned c, unsigned i, unsigned j, unsigned k) {
+  const float s = mg_gather<kAp>(L, c, i, j, k, [&](unsigned d, unsigned, unsigned, unsigned) { return L.x[d]; });
+  const float x = L.invd[c] * (L.b[c] + s);
+  L.x[c] = x;
+  return x;
+}
+
+// The passes grid-wide: a CTA takes tiles of 2^lx pairs x (256 >> lx) rows x kc
+// layers, tile blockIdx.x, + gridDim.x, ... (two divisions per tile, none per
+// cell).  f(p, j, k) for every pair (or coarse cell) p < np.
+struct MgTiles {
+  unsigned np, ny, nz;       // extent
+  unsigned lx, kc;           // tile shape
+  unsigned tx, ty, tiles;    // tiles along x, y; in all
+};
+template <typename F>
+__device__ __forceinline__ void mg_tiles(const MgTiles& T, F&& f) {
+  const unsigned px = threadIdx.x & ((1u << T.lx) - 1u), py = threadIdx.x >> T.lx;
+  for (unsigned t = blockIdx.x; t < T.tiles; t += gridDim.x) {
+    const unsigned txy = T.tx * T.ty, tz = t / txy, r = t - tz * txy, y = r / T.tx, x = r - y * T.tx;
+    const unsigned p = (x << T.lx) + px, j = y * ((unsigned)kProjThreads >> T.lx) + py;
+    if (p >= T.np || j >= T.ny) continue;
+    const unsigned k1 = min((tz + 1) * T.kc, T.nz);
+#pragma unroll 2
+    for (unsigned k = tz * T.kc; k < k1; ++k) f(p, j, k);
   }
 }
 
-// Coarse right-hand side: the sum of the children's residuals b - A x.
-__device__ __forceinline__ void mg_restrict_range(const MgLevel& F, const MgLevel& C, unsigned t0, unsigned stride) {
-  const unsigned n = (unsigned)C.nx * C.ny * C.nz;
-  const unsigned fnx = F.nx, fny = F.ny, fnz = F.nz;
-  for (unsigned q = t0; q < n; q += stride) {
-    unsigned I, J, K;
-    level_ijk(C, q, I, J, K);
-    float acc = 0.f;
-    for (unsigned k = 2 * K; k < min(2 * K + 2, fnz); ++k)
-      for (unsigned j = 2 * J; j < min(2 * J + 2, fny); ++j)
-        for (unsigned i = 2 * I; i < min(2 * I + 2, fnx); ++i) {
-          const unsigned c = i + fnx * (j + fny * k);
-          float s, diag;
-          level_gather(F, c, i, j, k, F.x, s, diag);
-          acc += F.b[c] - (diag * F.x[c] - s);
-        }
-    C.b[q] = acc;
-  }
-}
-
-// x_fine += kMgOmega x_coarse(parent)
-__device__ __forceinline__ void mg_prolong_range(const MgLevel& C, const MgLevel& F, unsigned t0, unsigned stride) {
-  const unsigned n = (unsigned)F.nx * F.ny * F.nz;
-  for (unsigned c = t0; c < n; c += stride) {
-    unsigned i, j, k;
-    level_ijk(F, c, i, j, k);
-    F.x[c] = fmaf(kMgOmega, C.x[(i >> 1) + (unsigned)C.nx * ((j >> 1) + (unsigned)C.ny * (k >> 1))], F.x[c]);
-  }
-}
-
-__global__ void __launch_bounds__(kProjThreads) k_mg_smooth(MgLevel L, unsigned color, int init,
-                                                            const ProjRed* red) {
+template <bool kAp>
+__global__ void __launch_bounds__(kProjThreads, 4) k_mg_down(MgLevel L, MgTiles T, const ProjRed* red) {
   if (stopped(red)) return;
-  mg_smooth_range(L, color, init, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  mg_tiles(T, [&](unsigned p, unsigned j, unsigned k) { mg_down<kAp>(L, mg_pair(L, p, j, k)); });
 }
 
-__global__ void __launch_bounds__(kProjThreads) k_mg_restrict(MgLevel F, MgLevel C, const ProjRed* red) {
+template <bool kAp>
+__global__ void __launch_bounds__(kProjThreads, 4) k_mg_restrict(MgLevel F, MgLevel C, MgTiles T, const ProjRed* red) {
   if (stopped(red)) return;
-  mg_restrict_range(F, C, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  mg_tiles(T, [&](unsigned p, unsigned J, unsigned K) { mg_restrict<kAp>(F, C, p >> 2, p & 3u, J, K); });
 }
 
-__global__ void __launch_bounds__(kProjThreads) k_mg_prolong(MgLevel C, MgLevel F, const ProjRed* red) {
+template <bool kAp>
+__global__ void __launch_bounds__(kProjThreads, 4) k_mg_up_black(MgLevel L, MgLevel C, MgTiles T, const ProjRed* red) {
   if (stopped(red)) return;
-  mg_prolong_range(C, F, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+  mg_tiles(T, [&](unsigned p, unsigned j, unsigned k) { mg_up_black<kAp>(L, C, mg_pair(L, p, j, k)); });
+}
+
+__global__ void __launch_bounds__(kProjThreads, 4) k_mg_up_red(MgLevel L, MgTiles T, const ProjRed* red) {
+  if (stopped(red)) return;
+  mg_tiles(T, [&](unsigned p, unsigned j, unsigned k) {
+    const MgPair q = mg_pair(L, p, j, k);
+    if (q.red) mg_sweep<false>(L, q.row + q.ir, q.ir, j, k);
+  });
+}
+
+// The same on level 0, where x = z = M^-1 r is complete after it, with rho =
+// r . z into red->rz[cur] (b is r): a thread has both cells of its pair at hand.
+__global__ void __launch_bounds__(kProjThreads, 4) k_mg_up_red_dot(MgLevel L, MgTiles T, int cur,
+                                                                   double* __restrict__ P, ProjRed* red) {
+  __shared__ double smem[32];
+  if (stopped(red)) return;
+  KahanF sum;
+  mg_tiles(T, [&](unsigned p, unsigned j, unsigned k) {
+    const MgPair q = mg_pair(L, p, j, k);
+    if (q.red) sum.add(L.b[q.row + q.ir] * mg_sweep<true>(L, q.row + q.ir, q.ir, j, k));
+    if (q.black) sum.add(L.b[q.row + q.ib] * L.x[q.row + q.ib]);
+  });
+  const double rz = block_sum(sum, smem);
+  const double vals[1] = {rz};
+  double* const outs[1] = {&red->rz[cur]};
+  reduce_last<1>(vals, P, red, outs);
 }
 
 // The levels from `first` (at most kMgTailCells cells) down to the coarsest
-// in one CTA, with a barrier between passes (their launches would cost more
-// than their work): the same passes as the grid-wide V-cycle, and on the
-// coarsest level (every axis <= 4 cells) red from x = 0, then kMgCoarsePairs
-// (black, red) sweep pairs.  Same-color cells do not touch, so a half sweep
-// reads only values no thread of the pass writes.
+// in one CTA: their weights, invd and the right-hand side of `first` are copied
+// to shared memory (all copies in flight together), and every pass runs there with a barrier after it (16^3
+// and below: 16 us; with the levels in global memory, a barrier and an L2 round
+// trip per pass, 29 us).  On the coarsest level (every axis <= 4 cells, so
+// at most 32 pairs: one warp) red from x = 0, then kMgCoarsePairs (black, red)
+// sweep pairs.  Same-colour cells do not touch, so a half sweep reads only
+// values no thread of the pass writes.
 constexpr int kMgTailThreads = 1024;
 constexpr int kMgTailCells = 4096;
+constexpr size_t kMgTailSmem = 200 * 1024;
 struct MgLevels {
   MgLevel l[kMgMaxLevels];
 };
+// Floats of one level in the tail's shared memory; its arrays start at multiples
+// of four floats.
+__host__ __device__ inline unsigned mg_pad(unsigned n) { return (n + 3u) & ~3u; }
+__host__ __device__ inline unsigned mg_level_floats(unsigned nx, unsigned ny, unsigned nz) {
+  return mg_pad((nx + 1) * ny * nz) + mg_pad(nx * (ny + 1) * nz) + mg_pad(nx * ny * (nz + 1)) + 3 * mg_pad(nx * ny * nz);
+}
+
+extern __shared__ __align__(16) float g_mg_smem[];
+
+// Level L's arrays at `base` floats in shared memory.
+__device__ __forceinline__ MgLevel mg_shared(const MgLevel& L, unsigned base) {
+  const unsigned nx = L.nx, ny = L.ny, nz = L.nz, n = mg_pad(nx * ny * nz);
+  MgLevel S = L;
+  float* q = g_mg_smem + base;
+  S.bx = q;
+  q += mg_pad((nx + 1) * ny * nz);
+  S.by = q;
+  q += mg_pad(nx * (ny + 1) * nz);
+  S.bz = q;
+  q += mg_pad(nx * ny * (nz + 1));
+  S.invd = q;
+  S.x = q + n;
+  S.b = q + 2 * n;
+  return S;
+}
+
+// n floats to shared memory, not waited for (both sides 16-byte aligned).
+__device__ __forceinline__ void mg_copy(float* dst, const float* src, unsigned n) {
+  const unsigned to = (unsigned)__cvta_generic_to_shared(dst);
+  for (unsigned q = threadIdx.x; q < n / 4; q += kMgTailThreads)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(to + 16 * q), "l"(src + 4 * q) : "memory");
+  const unsigned q = (n & ~3u) + threadIdx.x;
+  if (q < n) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to + 4 * q), "l"(src + q) : "memory");
+}
+
+// f(p, j, k) for the np x ny x nz pairs (or cells) by the whole CTA
+template <typename F>
+__device__ __forceinline__ void mg_cta(unsigned np, unsigned ny, unsigned nz, F&& f) {
+  for (unsigned t = threadIdx.x; t < np * ny * nz; t += kMgTailThreads) {
+    const unsigned k = t / (np * ny), r = t - k * np * ny, j = r / np;
+    f(r - j * np, j, k);
+  }
+  __syncthreads();
+}
 
 __global__ void __launch_bounds__(kMgTailThreads) k_mg_tail(MgLevels Ls, int first, int top, const ProjRed* red) {
   if (stopped(red)) return;
-  const unsigned t0 = threadIdx.x, st = blockDim.x;
-  for (int l = first; l < top; ++l) {
-    mg_smooth_range(Ls.l[l], 0u, 1, t0, st);
-    __syncthreads();
-    mg_smooth_range(Ls.l[l], 1u, 0, t0, st);
-    __syncthreads();
-    mg_restrict_range(Ls.l[l], Ls.l[l + 1], t0, st);
-    __syncthreads();
+  unsigned base = 0;
+  for (int l = first; l <= top; ++l) {
+    const MgLevel G = Ls.l[l], S = mg_shared(G, base);
+    const unsigned nx = G.nx, ny = G.ny, nz = G.nz, n = nx * ny * nz;
+    mg_copy(S.bx, G.bx, (nx + 1) * ny * nz);
+    mg_copy(S.by, G.by, nx * (ny + 1) * nz);
+    mg_copy(S.bz, G.bz, nx * ny * (nz + 1));
+    mg_copy(S.invd, G.invd, n);
+    if (l == first) mg_copy(S.b, G.b, n);
+    base += mg_level_floats(G.nx, G.ny, G.nz);
   }
-  mg_smooth_range(Ls.l[top], 0u, 1, t0, st);
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  for (int p = 0; p < kMgCoarsePairs; ++p) {
-    mg_smooth_range(Ls.l[top], 1u, 0, t0, st);
-    __syncthreads();
-    mg_smooth_range(Ls.l[top], 0u, 0, t0, st);
+  base = 0;
+  for (int l = first; l < top; ++l) {
+    const MgLevel S = mg_shared(Ls.l[l], base);
+    base += mg_level_floats(S.nx, S.ny, S.nz);
+    const MgLevel C = mg_shared(Ls.l[l + 1], base);
+    mg_cta((S.nx + 1) / 2, S.ny, S.nz, [&](unsigned p, unsigned j, unsigned k) { mg_down<false>(S, mg_pair(S, p, j, k)); });
+    mg_cta(4 * C.nx, C.ny, C.nz, [&](unsigned p, unsigned J, unsigned K) { mg_restrict<false>(S, C, p >> 2, p & 3u, J, K); });
+  }
+  {
+    const MgLevel S = mg_shared(Ls.l[top], base);
+    const unsigned np = (S.nx + 1) / 2, t = threadIdx.x;
+    if (t < 32) {
+      const bool any = t < np * S.ny * S.nz;
+      const unsigned k = t / (np * S.ny), r = t - k * np * S.ny, j = r / np;
+      const MgPair q = mg_pair(S, r - j * np, j, k);
+      if (any) mg_down<false>(S, q);  // red from x = 0, then black
+      __syncwarp();
+      if (any && q.red) mg_sweep<false>(S, q.row + q.ir, q.ir, j, k);
+      __syncwarp();
+      for (int m = 1; m < kMgCoarsePairs; ++m) {
+        if (any && q.black) mg_sweep<false>(S, q.row + q.ib, q.ib, j, k);
+        __syncwarp();
+        if (any && q.red) mg_sweep<false>(S, q.row + q.ir, q.ir, j, k);
+        __syncwarp();
+      }
+    }
     __syncthreads();
   }
   for (int l = top - 1; l >= first; --l) {
-    mg_prolong_range(Ls.l[l + 1], Ls.l[l], t0, st);
-    __syncthreads();
-    mg_smooth_range(Ls.l[l], 1u, 0, t0, st);
-    __syncthreads();
-    mg_smooth_range(Ls.l[l], 0u, 0, t0, st);
-    __syncthreads();
+    const MgLevel C = mg_shared(Ls.l[l + 1], base);
+    base -= mg_level_floats(Ls.l[l].nx, Ls.l[l].ny, Ls.l[l].nz);
+    const MgLevel S = mg_shared(Ls.l[l], base);
+    const unsigned np = (S.nx + 1) / 2;
+    mg_cta(np, S.ny, S.nz, [&](unsigned p, unsigned j, unsigned k) { mg_up_black<false>(S, C, mg_pair(S, p, j, k)); });
+    mg_cta(np, S.ny, S.nz, [&](unsigned p, unsigned j, unsigned k) {
+      const MgPair q = mg_pair(S, p, j, k);
+      if (q.red) mg_sweep<false>(S, q.row + q.ir, q.ir, j, k);
+    });
   }
+  const MgLevel S = mg_shared(Ls.l[first], 0);
+  float* x = Ls.l[first].x;
+  for (unsigned c = threadIdx.x; c < (unsigned)(S.nx * S.ny * S.nz); c += kMgTailThreads) x[c] = S.x[c];
 }
 
 // ---- conjugate gradients on A e = r with the multigrid preconditioner ----
@@ -456,7 +714,7 @@ __global__ void __launch_bounds__(kProjThreads) k_cg_dot(int64_t n64, int cur, c
   const unsigned n = (unsigned)n64;
   KahanF k;
   for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) k.add(r[c] * z[c]);
-  const double rz = block_sum((double)k.s, smem);
+  const double rz = block_sum(k, smem);
   const double vals[1] = {rz};
   double* const outs[1] = {&red->rz[cur]};
   reduce_last<1>(vals, P, red, outs);
@@ -465,38 +723,35 @@ __global__ void __launch_bounds__(kProjThreads) k_cg_dot(int64_t n64, int cur, c
 // d_new = z + beta d_old (beta = rho / rho_prev; 0 on a run's first
 // iteration), y = A d_new and d_new . y into red->dy.  d_old and d_new are
 // different buffers: neighbours' d_new is formed from their z and d_old.
-__global__ void __launch_bounds__(kProjThreads) k_cg_dir_apply(MgLevel L, int cur, const float* __restrict__ z,
-                                                               const float* __restrict__ d_old,
-                                                               float* __restrict__ d_new, float* __restrict__ y,
-                                                               double* __restrict__ P, ProjRed* red) {
+// The face weights are formed again from alpha_f' (mg_faces).
+__global__ void __launch_bounds__(kProjThreads, 4) k_cg_dir_apply(MgLevel L, MgTiles T, int cur,
+                                                                  const float* __restrict__ z,
+                                                                  const float* __restrict__ d_old,
+                                                                  float* __restrict__ d_new, float* __restrict__ y,
+                                                                  double* __restrict__ P, ProjRed* red) {
   __shared__ double smem[32];
   if (stopped(red)) return;
   // beta in FP32 (a double divide per thread would occupy GB300's slow FP64 pipe)
   const float be = red->iters == 0 ? 0.f : (float)red->rz[cur] / (float)red->rz[cur ^ 1];
-  const unsigned nx = L.nx, ny = L.ny, nz = L.nz, nxy = nx * ny, n = nxy * nz;
   KahanF dyk;
-  for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x) {
-    unsigned i, j, k;
-    level_ijk(L, c, i, j, k);
-    // beta = 0 takes z alone (the old direction is not read into the sum)
-    auto dn = [&](unsigned q) { return be != 0.f ? fmaf(be, d_old[q], z[q]) : z[q]; };
+  // beta = 0 takes z alone (the old direction is not read into the sum)
+  auto dn = [&](unsigned q) { return be != 0.f ? fmaf(be, d_old[q], z[q]) : z[q]; };
+  mg_tiles(T, [&](unsigned i, unsigned j, unsigned k) {
+    const unsigned c = i + (unsigned)L.nx * (j + (unsigned)L.ny * k);
+    const MgNear m = mg_near(L, c, i, j, k);
+    const MgFaces w = mg_faces<true>(L, m, c, i, j, k);
+    float v[6];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) v[a] = dn(m.q[a]);
     const float dc = dn(c);
-    const unsigned fx = i + (nx + 1) * (j + ny * k);
-    const unsigned fy = i + nx * (j + (ny + 1) * k);
-    const float wxl = L.bx[fx], wxh = L.bx[fx + 1], wyl = L.by[fy], wyh = L.by[fy + nx], wzl = L.bz[c],
-                wzh = L.bz[c + nxy];
-    float acc = (((wxl + wxh) + (wyl + wyh)) + (wzl + wzh)) * dc;
-    if (i > 0) acc = fmaf(-wxl, dn(c - 1), acc);
-    if (i + 1 < nx) acc = fmaf(-wxh, dn(c + 1), acc);
-    if (j > 0) acc = fmaf(-wyl, dn(c - nx), acc);
-    if (j + 1 < ny) acc = fmaf(-wyh, dn(c + nx), acc);
-    if (k > 0) acc = fmaf(-wzl, dn(c - nxy), acc);
-    if (k + 1 < nz) acc = fmaf(-wzh, dn(c + nxy), acc);
+    float acc = (((w.w[0] + w.w[1]) + (w.w[2] + w.w[3])) + (w.w[4] + w.w[5])) * dc;
+#pragma unroll
+    for (int a = 0; a < 6; ++a) acc = fmaf(m.in[a] ? -w.w[a] : 0.f, v[a], acc);
     d_new[c] = dc;
     y[c] = acc;
     dyk.add(dc * acc);
-  }
-  const double dy = block_sum((double)dyk.s, smem);
+  });
+  const double dy = block_sum(dyk, smem);
   const double vals[1] = {dy};
   double* const outs[1] = {&red->dy};
   reduce_last<1>(vals, P, red, outs);
@@ -543,7 +798,7 @@ __global__ void __launch_bounds__(kProjThreads) k_cg_update(int64_t n64, int cur
     r[c] = rc;
     rrk.add(rc * rc);
   }
-  const double rr = block_sum((double)rrk.s, smem);
+  const double rr = block_sum(rrk, smem);
   const double vals[1] = {rr};
   double* const outs[1] = {&red->rr};
   if (reduce_last<1>(vals, P, red, outs) && threadIdx.x == 0) {
@@ -617,6 +872,7 @@ __global__ void __launch_bounds__(kProjThreads) k_proj_faces(
 
 struct ProjWs {
   double *fx, *fy, *fz;                // FP64 face weights (the residual's operator)
+  double* b64;                         // right-hand side of the solve
   float *ap32, *r, *z, *d[2], *y, *e;  // d: the CG direction, double-buffered
   double* P;                           // 2 * nblk partial sums
   ProjRed* red;
@@ -649,6 +905,7 @@ static size_t proj_layout(const PGrid& g, int nblk, char* base, ProjWs* W) {
   w.fx = (double*)take(8 * (size_t)(g.nx + 1) * g.ny * g.nz);
   w.fy = (double*)take(8 * (size_t)g.nx * (g.ny + 1) * g.nz);
   w.fz = (double*)take(8 * (size_t)g.nx * g.ny * (g.nz + 1));
+  w.b64 = (double*)take(8 * n);
   w.ap32 = (float*)take(4 * n);
   w.r = (float*)take(4 * n);
   w.z = (float*)take(4 * n);
@@ -761,6 +1018,9 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
   cudaStream_t st = (cudaStream_t)stream_;
   ProjWs W;
   proj_layout(g, nblk, (char*)ws, &W);
+  for (int l = 0; l < W.levels; ++l) W.lev[l].ap = nullptr, W.lev[l].open = 0u;
+  W.lev[0].ap = W.ap32;
+  W.lev[0].open = open_bits;
   if (W.levels == kMgMaxLevels && !(W.lev[kMgMaxLevels - 1].nx <= 4 && W.lev[kMgMaxLevels - 1].ny <= 4 &&
                                     W.lev[kMgMaxLevels - 1].nz <= 4))
     return set_error(GIC_ERR_INVALID, "gic_project: grid too large for the multigrid hierarchy");
@@ -798,56 +1058,67 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
     k_mg_diag<<<lblocks(W.lev[l]), kProjThreads, 0, st>>>(W.lev[l]);
     launches += 2;
   }
-  // the levels from `first` on run in one CTA (k_mg_tail)
+  // the levels from `first` on run in one CTA (k_mg_tail): the largest that has
+  // few cells and fits its shared memory with those below it
   MgLevels levels;
   for (int l = 0; l < W.levels; ++l) levels.l[l] = W.lev[l];
-  int first = 0;
-  while (first < W.levels - 1 && (int64_t)W.lev[first].nx * W.lev[first].ny * W.lev[first].nz > kMgTailCells) ++first;
+  const int top = W.levels - 1;
+  int first = top;
+  size_t tail_bytes = 4 * (size_t)mg_level_floats(W.lev[top].nx, W.lev[top].ny, W.lev[top].nz);
+  while (first > 0) {
+    const MgLevel& L = W.lev[first - 1];
+    if ((int64_t)L.nx * L.ny * L.nz > kMgTailCells) break;
+    const size_t more = 4 * (size_t)mg_level_floats(L.nx, L.ny, L.nz);
+    if (tail_bytes + more > kMgTailSmem) break;
+    tail_bytes += more;
+    --first;
+  }
+  if (tail_bytes > 48 * 1024 &&
+      cudaFuncSetAttribute(k_mg_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMgTailSmem) != cudaSuccess)
+    return set_error(GIC_ERR_CUDA, "gic_project: shared memory of the coarse levels refused");
+  // tiles of a pass over np x ny x nz pairs (or cells): wide enough for the rows, and
+  // up to four layers per tile where that still leaves a tile for every CTA
+  auto tiles = [&](unsigned np, unsigned ny, unsigned nz) {
+    MgTiles T;
+    T.np = np, T.ny = ny, T.nz = nz;
+    T.lx = 0;
+    while (T.lx < 5 && (1u << T.lx) < np) ++T.lx;
+    const unsigned rows = (unsigned)kProjThreads >> T.lx;
+    T.tx = (np + (1u << T.lx) - 1) >> T.lx;
+    T.ty = (ny + rows - 1) / rows;
+    T.kc = 1;
+    while (T.kc < 4 && (uint64_t)T.tx * T.ty * ((nz + 2 * T.kc - 1) / (2 * T.kc)) >= 608) T.kc *= 2;
+    T.tiles = T.tx * T.ty * ((nz + T.kc - 1) / T.kc);
+    return T;
+  };
+  auto pairs = [&](const MgLevel& L) { return tiles((unsigned)(L.nx + 1) / 2, L.ny, L.nz); };
+  auto quads = [&](const MgLevel& L) { return tiles(4 * (unsigned)L.nx, L.ny, L.nz); };  // four lanes per cell
+  auto ctas = [&](const MgTiles& T) { return (int)(T.tiles < (unsigned)nblk ? T.tiles : (unsigned)nblk); };
   // one preconditioned CG iteration: z = V-cycle(r), rho = r . z, the new
   // direction with y = A d, the updates; all arguments but the parity are
   // fixed for the call
-  int per_iter = 0;
-  auto cg_iteration = [&](int cur, cudaStream_t s_) {
-    const int top = W.levels - 1;
+  auto cg_iteration = [&](int cur) {
     for (int l = 0; l < first; ++l) {
-      k_mg_smooth<<<lblocks(W.lev[l]), kProjThreads, 0, s_>>>(W.lev[l], 0u, 1, W.red);
-      k_mg_smooth<<<lblocks(W.lev[l]), kProjThreads, 0, s_>>>(W.lev[l], 1u, 0, W.red);
-      k_mg_restrict<<<lblocks(W.lev[l + 1]), kProjThreads, 0, s_>>>(W.lev[l], W.lev[l + 1], W.red);
+      const MgLevel &L = W.lev[l], &C = W.lev[l + 1];
+      const MgTiles T = pairs(L), Q = quads(C);
+      (l == 0 ? k_mg_down<true> : k_mg_down<false>)<<<ctas(T), kProjThreads, 0, st>>>(L, T, W.red);
+      (l == 0 ? k_mg_restrict<true> : k_mg_restrict<false>)<<<ctas(Q), kProjThreads, 0, st>>>(L, C, Q, W.red);
     }
-    k_mg_tail<<<1, kMgTailThreads, 0, s_>>>(levels, first, top, W.red);
+    k_mg_tail<<<1, kMgTailThreads, tail_bytes, st>>>(levels, first, top, W.red);
     for (int l = first - 1; l >= 0; --l) {
-      k_mg_prolong<<<lblocks(W.lev[l]), kProjThreads, 0, s_>>>(W.lev[l + 1], W.lev[l], W.red);
-      k_mg_smooth<<<lblocks(W.lev[l]), kProjThreads, 0, s_>>>(W.lev[l], 1u, 0, W.red);
-      k_mg_smooth<<<lblocks(W.lev[l]), kProjThreads, 0, s_>>>(W.lev[l], 0u, 0, W.red);
+      const MgLevel &L = W.lev[l], &C = W.lev[l + 1];
+      const MgTiles T = pairs(L);
+      (l == 0 ? k_mg_up_black<true> : k_mg_up_black<false>)<<<ctas(T), kProjThreads, 0, st>>>(L, C, T, W.red);
+      if (l > 0)
+        k_mg_up_red<<<ctas(T), kProjThreads, 0, st>>>(L, T, W.red);
+      else
+        k_mg_up_red_dot<<<ctas(T), kProjThreads, 0, st>>>(L, T, cur, W.P, W.red);
     }
-    k_cg_dot<<<nblk, kProjThreads, 0, s_>>>(g.n, cur, W.r, W.z, W.P, W.red);
-    k_cg_dir_apply<<<nblk, kProjThreads, 0, s_>>>(W.lev[0], cur, W.z, W.d[cur ^ 1], W.d[cur], W.y, W.P, W.red);
-    k_cg_update<<<nblk, kProjThreads, 0, s_>>>(g.n, cur, W.d[cur], W.y, W.e, W.r, W.P, W.red);
-    per_iter = 6 * first + 4;
-  };
-  // kChunk iterations as one CUDA graph (kChunk even: the parities repeat),
-  // built when the first CG run needs it
-  constexpr int kChunk = 4;
-  cudaGraphExec_t chunk = nullptr;
-  auto build_chunk = [&]() -> int {
-    cudaStream_t cs = nullptr;
-    cudaGraph_t gr = nullptr;
-    bool ok = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-    if (ok) {
-      for (int q = 0; q < kChunk; ++q) cg_iteration(q & 1, cs);
-      ok = cudaStreamEndCapture(cs, &gr) == cudaSuccess && gr != nullptr;
-    }
-    ok = ok && cudaGraphInstantiate(&chunk, gr, 0) == cudaSuccess;
-    if (gr) cudaGraphDestroy(gr);
-    if (cs) cudaStreamDestroy(cs);
-    if (!ok) {
-      cudaGetLastError();
-      if (chunk) cudaGraphExecDestroy(chunk);
-      chunk = nullptr;
-      return set_error(GIC_ERR_CUDA, "gic_project: building the CG graph failed");
-    }
-    return GIC_OK;
+    if (first == 0) k_cg_dot<<<nblk, kProjThreads, 0, st>>>(g.n, cur, W.r, W.z, W.P, W.red);
+    const MgTiles T = tiles(g.nx, g.ny, g.nz);
+    k_cg_dir_apply<<<ctas(T), kProjThreads, 0, st>>>(W.lev[0], T, cur, W.z, W.d[cur ^ 1], W.d[cur], W.y, W.P, W.red);
+    k_cg_update<<<nblk, kProjThreads, 0, st>>>(g.n, cur, W.d[cur], W.y, W.e, W.r, W.P, W.red);
+    launches += 4 * first + (first == 0 ? 4 : 3);
   };
 
   for (int which = 1; which <= 2 && rc2 == GIC_OK; ++which) {
@@ -857,9 +1128,15 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
       rc2 = set_error(GIC_ERR_CUDA, "gic_project: clearing p failed");
       break;
     }
+    int last_iters = 4;  // of the previous CG run
     for (int outer = 0;; ++outer) {
-      k_proj_residual<<<nblk, kProjThreads, 0, st>>>(g, which, S, alpha_s, alpha_star, u, v, w, W.fx, W.fy, W.fz, p,
-                                                     W.r, W.e, P->inner_tol * P->inner_tol, W.P, W.red, status);
+      const double tol2 = P->inner_tol * P->inner_tol;
+      if (outer == 0)  // p = 0
+        k_proj_rhs<<<nblk, kProjThreads, 0, st>>>(g, which, S, alpha_s, alpha_star, u, v, w, W.fx, W.fy, W.fz, W.b64,
+                                                  W.r, W.e, tol2, W.P, W.red, status);
+      else
+        k_proj_residual<<<nblk, kProjThreads, 0, st>>>(g, W.b64, W.fx, W.fy, W.fz, p, W.r, W.e, tol2, W.P, W.red,
+                                                       status);
       ++launches;
       if ((rc2 = read_red(W.red, &hr, st))) break;
       if (!isfinite(hr.rr64) || !isfinite(hr.bb)) {
@@ -874,24 +1151,12 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
       }
       if (outer >= P->max_outer) break;
       // the FP32 preconditioned CG on A e = r to a reduction of inner_tol (of
-      // the FP32 copy's r . r): graph launches of kChunk iterations, the stop
-      // flag read after each
-      int it = 0;
+      // the FP32 copy's r . r): as many iterations as the previous run took,
+      // less one, are queued before the stop flag is read, then two at a time
+      // (iterations queued past the stop return at once)
+      int it = 0, want = last_iters > 2 ? last_iters - 1 : 2;
       for (;;) {
-        if (P->max_inner - it >= kChunk) {
-          if (!chunk && (rc2 = build_chunk())) break;
-          if (cudaGraphLaunch(chunk, st) != cudaSuccess) {
-            rc2 = set_error(GIC_ERR_CUDA, "gic_project: graph launch failed");
-            break;
-          }
-          it += kChunk;
-          launches += (int64_t)per_iter * kChunk;
-        } else {
-          for (; it < P->max_inner; ++it) {
-            cg_iteration(it & 1, st);
-            launches += per_iter;
-          }
-        }
+        for (int q = 0; q < want && it < P->max_inner; ++q, ++it) cg_iteration(it & 1);
         cudaError_t le = cudaGetLastError();
         if (le != cudaSuccess) {
           rc2 = set_error(GIC_ERR_CUDA, "gic_project: %s", cudaGetErrorString(le));
@@ -899,7 +1164,9 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
         }
         if ((rc2 = read_red(W.red, &hr, st))) break;
         if (hr.done || it >= P->max_inner) break;
+        want = 2;
       }
+      last_iters = hr.iters;
       if (rc2) break;
       inf.inner[sys] += hr.iters;
       k_proj_add<<<nblk, kProjThreads, 0, st>>>(g.n, p, W.e);
@@ -914,7 +1181,6 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
                                               u_out, v_out, w_out, dx_u, dx_v, dx_w);
     ++launches;
   }
-  if (chunk) cudaGraphExecDestroy(chunk);
   count_launches(launches);
   if (rc2) return rc2;
   GIC_CHECK_LAUNCH("gic_project");
