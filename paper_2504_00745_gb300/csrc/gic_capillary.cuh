@@ -143,6 +143,7 @@ __device__ __forceinline__ bool pair_within(const DGrid& G, const uint4& pi, con
 }
 __device__ __forceinline__ bool pair_within(const DGrid& G, const d4& pi, const d4& pj, int ox, int oy, int oz,
                                             double ri, double rj, double reach, PairGeom<double>& g) {
+  if (!may_reach(G, pi, pj, ox, oy, oz, abs_trunc_f(ri) + abs_trunc_f(rj) + abs_trunc_f(reach))) return false;
   double x0, x1, x2;
   rel_ij(G, pi, pj, ox, oy, oz, x0, x1, x2);
   const double d2 = x0 * x0 + x1 * x1 + x2 * x2;

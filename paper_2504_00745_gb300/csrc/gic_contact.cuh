@@ -194,6 +194,23 @@ __device__ __forceinline__ bool pair_geom(const DGrid& G, const d4& pi, const d4
   return true;
 }
 
+// FP64 candidates, in float and with integer conversions: whether granule j at
+// cell offset o may be within `reach` (metres) of i.  The offsets are below h_c
+// and truncated by less than 2^-23 of themselves, the sums rounded to float:
+// each component is off by less than 2^-20 h_c, which the margin of 2^-13 h_c
+// covers.
+__device__ __forceinline__ bool may_reach(const DGrid& G, const d4& pi, const d4& pj, int ox, int oy, int oz,
+                                          float reach) {
+  const float rx = (trunc_f(pi.x) - trunc_f(pj.x)) - (float)ox * G.hc_f;
+  const float ry = (trunc_f(pi.y) - trunc_f(pj.y)) - (float)oy * G.hc_f;
+  const float rz = (trunc_f(pi.z) - trunc_f(pj.z)) - (float)oz * G.hc_f;
+  const float R = fmaf(G.hc_f, 1.0f / 8192.0f, reach);
+  return fmaf(rx, rx, fmaf(ry, ry, rz * rz)) < R * R;
+}
+__device__ __forceinline__ bool may_reach(const DGrid&, const uint4&, const uint4&, int, int, int, float) {
+  return true;  // the FP32 path has its own float pre-tests
+}
+
 // Wall geometry: the granule's gap to the lower (side 0) or upper wall of
 // axis a when it sits in the first / last contact cell.  FP32: the gap is the
 // exact integer q (or 2^30 - q) and the overlap r 2^30/h_c - gap is formed
@@ -320,6 +337,8 @@ __device__ __forceinline__ void for_each_contact(const DGrid& G, const uint4* __
   }
   for_each_partner(G, table, epoch, i, cx, cy, cz, [&](int64_t j, int ox, int oy, int oz) {
     pos_t<T> pj = ldg(&pos[j]);
+    if constexpr (sizeof(T) == 8)
+      if (!may_reach(G, pi, pj, ox, oy, oz, abs_trunc_f(ri) + abs_trunc_f(radius_of(pj)))) return;
     PairGeom<T> g;
     if (pair_geom(G, pi, pj, ox, oy, oz, ri, radius_of(pj), g)) f(j, g);
   });
@@ -391,10 +410,16 @@ __device__ __forceinline__ bool moved_far(const DGrid&, int32_t c, const uint4& 
 }
 __device__ __forceinline__ bool moved_far(const DGrid& G, int32_t c, const d4& p, int32_t cr, const d4& pr,
                                           double lim2) {
-  double dx = (double)(cell_x(c) - cell_x(cr)) * G.hc + (p.x - pr.x);
-  double dy = (double)(cell_y(c) - cell_y(cr)) * G.hc + (p.y - pr.y);
-  double dz = (double)(cell_z(c) - cell_z(cr)) * G.hc + (p.z - pr.z);
-  return dx * dx + dy * dy + dz * dz > lim2;
+  if (c != cr) {
+    double dx = (double)(cell_x(c) - cell_x(cr)) * G.hc + (p.x - pr.x);
+    double dy = (double)(cell_y(c) - cell_y(cr)) * G.hc + (p.y - pr.y);
+    double dz = (double)(cell_z(c) - cell_z(cr)) * G.hc + (p.z - pr.z);
+    return dx * dx + dy * dy + dz * dz > lim2;
+  }
+  // same cell: the squares in float, with a margin past their rounding (a
+  // rebuild a little early changes no contact)
+  const float dx = abs_trunc_f(p.x - pr.x), dy = abs_trunc_f(p.y - pr.y), dz = abs_trunc_f(p.z - pr.z);
+  return fmaf(dx, dx, fmaf(dy, dy, dz * dz)) > abs_trunc_f(lim2) * (1.0f - 1e-5f);
 }
 
 template <typename T>
@@ -452,6 +477,8 @@ __device__ __forceinline__ void verlet_pair(const DGrid& G, const d4& pi, double
                                             const float4&, const d4* __restrict__ pos, int64_t j, int ox, int oy, int oz,
                                             double skin, bool& near, bool& touch, PairGeom<double>& g) {
   d4 pj = ldg(&pos[j]);
+  near = touch = false;
+  if (!may_reach(G, pi, pj, ox, oy, oz, abs_trunc_f(ri) + abs_trunc_f(pj.w) + abs_trunc_f(skin))) return;
   double x0, x1, x2;
   rel_ij(G, pi, pj, ox, oy, oz, x0, x1, x2);
   double d2 = x0 * x0 + x1 * x1 + x2 * x2;

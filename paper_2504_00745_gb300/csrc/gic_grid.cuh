@@ -41,26 +41,13 @@ __device__ __forceinline__ GradPLoad<T> gradp_loader(const DGrid& G, const T* p,
   return L;
 }
 
-// G2P coupling of one granule at (cell, p) with velocity v (Sec. 3.3 Eqs. 5a,
-// 5b; Sec. 5.2 Eq. momentum4): F_fl = c_drag pi r^2 rho_f |u_f - v| (u_f - v)
-// - V grad p and a_f = g - grad p / rho_f.  Returns |u_f - v|.  face(comp)
-// and gradp(comp) give the samplers of the face velocities and of the face
-// pressure gradients (global memory or a staged tile: the same values).
-template <typename T, typename Face, typename GradP>
-__device__ __forceinline__ T g2p_granule_with(const DGrid& G, const DParams<T>& P, int32_t cell, const pos_t<T>& pi,
-                                              const vec_t<T>& vi, Face face, GradP gradp, T F[3], T a[3]) {
-  int m[3];
-  T t[3];
-  granule_mac<T>(G, cell, pi, m, t);
-  T uf[3], gp[3];
-  T inv_dx = grid_inv_dx<T>(G);
-#pragma unroll
-  for (int comp = 0; comp < 3; ++comp) {
-    Stencil3<T> S = make_stencil<T>(G, m, t, comp);
-    uf[comp] = interp<T>(S, face(comp), inv_dx, nullptr);
-    gp[comp] = interp<T>(S, gradp(comp), inv_dx, nullptr);
-  }
-  T r = radius_of(pi);
+// F_fl = c_drag pi r^2 rho_f |u_f - v| (u_f - v) - V grad p and a_f = g - grad p /
+// rho_f of a granule of radius r and velocity v from the fluid velocity uf and
+// the pressure gradient gp at it (Sec. 3.3 Eqs. 5a, 5b; Sec. 5.2 Eq. momentum4).
+// Returns |u_f - v|.
+template <typename T>
+__device__ __forceinline__ T coupling_forces(const DParams<T>& P, T r, const vec_t<T>& vi, const T uf[3], const T gp[3],
+                                             T F[3], T a[3]) {
   T V = T(4.0 / 3.0 * kPi) * r * r * r;
   T d0 = uf[0] - vi.x, d1 = uf[1] - vi.y, d2 = uf[2] - vi.z;
   T sp = sqrt(fma(d2, d2, fma(d0, d0, d1 * d1)));
@@ -78,6 +65,26 @@ __device__ __forceinline__ T g2p_granule_with(const DGrid& G, const DParams<T>& 
     a[2] = P.g[2];
   }
   return sp;
+}
+
+// G2P coupling of one granule at (cell, p) with velocity v.  face(comp) and
+// gradp(comp) give the samplers of the face velocities and of the face
+// pressure gradients (global memory or a staged tile: the same values).
+template <typename T, typename Face, typename GradP>
+__device__ __forceinline__ T g2p_granule_with(const DGrid& G, const DParams<T>& P, int32_t cell, const pos_t<T>& pi,
+                                              const vec_t<T>& vi, Face face, GradP gradp, T F[3], T a[3]) {
+  int m[3];
+  T t[3];
+  granule_mac<T>(G, cell, pi, m, t);
+  T uf[3], gp[3];
+  T inv_dx = grid_inv_dx<T>(G);
+#pragma unroll
+  for (int comp = 0; comp < 3; ++comp) {
+    Stencil3<T> S = make_stencil<T>(G, m, t, comp);
+    uf[comp] = interp_value<T>(S, face(comp), inv_dx);
+    gp[comp] = interp_value<T>(S, gradp(comp), inv_dx);
+  }
+  return coupling_forces<T>(P, radius_of(pi), vi, uf, gp, F, a);
 }
 
 template <typename T>
@@ -479,11 +486,12 @@ struct TileLoad {
   }
 };
 
-// CTA-wide (every thread calls it): the box of the granules' MAC cells, the
-// staged fields and the zeroed accumulators.  valid: this thread has a
-// granule in contact cell c.
-__device__ __forceinline__ SubBox sub_tile_begin(SubTile& sh, const DGrid& G, const Fields<float>& Fd, bool valid,
-                                                 int32_t c, bool do_a, bool do_f) {
+// CTA-wide (every thread calls it; one barrier): the box of samples m - 1 .. m + 1
+// per axis around the MAC cells of the CTA's granules, used as a tile when it
+// holds at most `most` of them.  valid: this thread has a granule in contact
+// cell c.
+__device__ __forceinline__ SubBox sub_box(int (&wlo)[3][kSubWarps], int (&whi)[3][kSubWarps], const DGrid& G,
+                                          bool valid, int32_t c, int most) {
   const int warp = threadIdx.x >> 5;
   const int c3[3] = {cell_x(c), cell_y(c), cell_z(c)};
 #pragma unroll
@@ -492,8 +500,8 @@ __device__ __forceinline__ SubBox sub_tile_begin(SubTile& sh, const DGrid& G, co
     const int l = __reduce_min_sync(0xffffffffu, valid ? m : INT_MAX);
     const int h = __reduce_max_sync(0xffffffffu, valid ? m : INT_MIN);
     if (lane_id() == 0) {
-      sh.wlo[a][warp] = l;
-      sh.whi[a][warp] = h;
+      wlo[a][warp] = l;
+      whi[a][warp] = h;
     }
   }
   __syncthreads();
@@ -503,8 +511,8 @@ __device__ __forceinline__ SubBox sub_tile_begin(SubTile& sh, const DGrid& G, co
     lo[a] = INT_MAX;
     hi[a] = INT_MIN;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      lo[a] = min(lo[a], sh.wlo[a][w]);
-      hi[a] = max(hi[a], sh.whi[a][w]);
+      lo[a] = min(lo[a], wlo[a][w]);
+      hi[a] = max(hi[a], whi[a][w]);
     }
   }
   SubBox B;
@@ -515,10 +523,18 @@ __device__ __forceinline__ SubBox sub_tile_begin(SubTile& sh, const DGrid& G, co
   B.ex = any ? hi[0] + 1 - B.b[0] + 1 : 1;
   B.ey = any ? hi[1] + 1 - B.b[1] + 1 : 1;
   B.ez = any ? hi[2] + 1 - B.b[2] + 1 : 1;
-  B.tile = any && (int64_t)B.ex * B.ey * B.ez <= kSubTile;
+  B.tile = any && (int64_t)B.ex * B.ey * B.ez <= most;
   B.sy = B.ex;
   B.sz = B.ex * B.ey;
   B.vol = B.tile ? B.ex * B.ey * B.ez : 0;
+  return B;
+}
+
+// CTA-wide (every thread calls it): the box, the staged fields and the zeroed
+// accumulators.
+__device__ __forceinline__ SubBox sub_tile_begin(SubTile& sh, const DGrid& G, const Fields<float>& Fd, bool valid,
+                                                 int32_t c, bool do_a, bool do_f) {
+  const SubBox B = sub_box(sh.wlo, sh.whi, G, valid, c, kSubTile);
   const float rx = 1.f / (float)B.ex, rxy = 1.f / (float)max(B.sz, 1);
   for (int e = threadIdx.x; e < B.vol; e += blockDim.x) {
     // e = lx + ex (ly + ey lz); (e + 1/2) / d stays >= 1/(2 d) from an integer
@@ -540,6 +556,94 @@ __device__ __forceinline__ SubBox sub_tile_begin(SubTile& sh, const DGrid& G, co
   }
   __syncthreads();
   return B;
+}
+
+// ---- FP64 substep: the CTA's tile of fluid samples ----
+//
+// As the FP32 tile, for G2P alone: the face velocities and face pressure
+// gradients of the box, each with its difference to the next sample along x, so
+// that a granule's six interpolations take 66 FP64 operations instead of 141
+// and the gradients' differences are formed once per sample.  The values and
+// their order are interp_value's: the same bits as from global memory.
+// (F_s in the tile as fixed-point limbs: 1% faster, and its unit, tied to the CTA's
+// largest force, cost two bits of the sums.  It stays with global atomics.)
+template <int NT>
+struct SubTile64 {
+  static constexpr int kSamples = NT == 64 ? 512 : 768;  // 48 KB / 72 KB
+  double f[6][kSamples], d[6][kSamples];
+  int wlo[3][kSubWarps], whi[3][kSubWarps];
+};
+
+template <int NT>
+__device__ __forceinline__ SubBox sub_tile64_begin(SubTile64<NT>& sh, const DGrid& G, const Fields<double>& Fd,
+                                                   bool valid, int32_t c) {
+  const SubBox B = sub_box(sh.wlo, sh.whi, G, valid, c, SubTile64<NT>::kSamples);
+  const float rx = 1.f / (float)B.ex, rxy = 1.f / (float)max(B.sz, 1);
+  for (int e = threadIdx.x; e < B.vol; e += NT) {
+    // e = lx + ex (ly + ey lz); (e + 1/2) / d stays >= 1/(2 d) from an integer
+    const int lz = (int)(((float)e + 0.5f) * rxy);
+    const int r = e - lz * B.sz;
+    const int ly = (int)(((float)r + 0.5f) * rx);
+    const int i = B.b[0] + r - ly * B.ex, j = B.b[1] + ly, k = B.b[2] + lz;
+    const bool cx = i < G.nx, cy = j < G.ny, cz = k < G.nz;     // a cell-centred index
+    const bool fx = i <= G.nx, fy = j <= G.ny, fz = k <= G.nz;  // a face index
+    sh.f[0][e] = (fx && cy && cz) ? face_loader<double>(G, Fd.u, 0)(i, j, k) : 0.0;
+    sh.f[1][e] = (cx && fy && cz) ? face_loader<double>(G, Fd.v, 1)(i, j, k) : 0.0;
+    sh.f[2][e] = (cx && cy && fz) ? face_loader<double>(G, Fd.w, 2)(i, j, k) : 0.0;
+    sh.f[3][e] = (fx && cy && cz) ? gradp_loader<double>(G, Fd.p, 0)(i, j, k) : 0.0;
+    sh.f[4][e] = (cx && fy && cz) ? gradp_loader<double>(G, Fd.p, 1)(i, j, k) : 0.0;
+    sh.f[5][e] = (cx && cy && fz) ? gradp_loader<double>(G, Fd.p, 2)(i, j, k) : 0.0;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < B.vol; e += NT) {
+    const int q = min(e + 1, B.vol - 1);  // the last sample of a row has no use for its difference
+#pragma unroll
+    for (int a = 0; a < 6; ++a) sh.d[a][e] = sh.f[a][q] - sh.f[a][e];
+  }
+  __syncthreads();
+  return B;
+}
+
+template <int NT>
+__device__ __forceinline__ double sub_g2p64(const SubTile64<NT>& sh, const SubBox& B, const DGrid& G,
+                                            const DParams<double>& P, const Fields<double>& Fd, int32_t c, const d4& pi,
+                                            const d4& vi, double F[3], double a[3]) {
+  if (!B.tile) return g2p_granule<double>(G, P, Fd, c, pi, vi, F, a);
+  int m[3];
+  double t[3], uf[3], gp[3];
+  granule_mac<double>(G, c, pi, m, t);
+#pragma unroll
+  for (int comp = 0; comp < 3; ++comp) {
+    const Stencil3<double> S = make_stencil<double>(G, m, t, comp);
+    const int e0 = B.index(S.i0[0], S.i0[1], S.i0[2]);
+    uf[comp] = gp[comp] = 0.0;
+    if (!GIC_DBG_OK(G.dbg, e0 >= 0 && e0 + 1 + B.sy + B.sz < B.vol)) continue;
+#pragma unroll
+    for (int cc = 0; cc < 2; ++cc)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const int e = e0 + b * B.sy + cc * B.sz;
+        const double w = (b ? S.w[1] : 1.0 - S.w[1]) * (cc ? S.w[2] : 1.0 - S.w[2]);
+        uf[comp] = fma(w, fma(S.w[0], sh.d[comp][e], sh.f[comp][e]), uf[comp]);
+        gp[comp] = fma(w, fma(S.w[0], sh.d[3 + comp][e], sh.f[3 + comp][e]), gp[comp]);
+      }
+  }
+  return coupling_forces<double>(P, radius_of(pi), vi, uf, gp, F, a);
+}
+
+// F_s deposits of one granule with double atomics: a row's deposit a is split
+// into w a and a - w a.
+__device__ __forceinline__ void add_face64(const DGrid& G, double* Fs, const Stencil3<double>& St, double fc) {
+#pragma unroll
+  for (int c = 0; c < 2; ++c)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const double a = (b ? St.w[1] : 1.0 - St.w[1]) * (c ? St.w[2] : 1.0 - St.w[2]) * fc;
+      const double hi = mul_rn(St.w[0], a);
+      const int64_t row = sample_index(St.ns[0], St.ns[1], St.i0[0], St.i0[1] + b, St.i0[2] + c);
+      atomicAdd(&Fs[row], a - hi);
+      atomicAdd(&Fs[row + 1], hi);
+    }
 }
 
 // G2P of one granule from global memory, out of line: the path of a CTA whose

@@ -50,6 +50,13 @@ __device__ __forceinline__ void advance_axis(const DGrid& G, float dt, float v, 
 __device__ __forceinline__ void advance_axis(const DGrid& G, double dt, double v, double o, int c, int nc,
                                              double& o_out, int& c_out, uint32_t& flags) {
   double x = fma(dt, v, o);
+  // still in the cell: 0 <= x < h_c, compared as integers (a negative or NaN x is
+  // above every such value), without the floor and its conversions
+  if ((unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(G.hc)) {
+    o_out = x;
+    c_out = c;
+    return;
+  }
   double sh = floor(x * G.inv_hc);
   if (!(fabs(sh) < 1e9)) sh = x > 0 ? 1e9 : -1e9;
   long long shift = (long long)sh;
@@ -85,7 +92,7 @@ __device__ __forceinline__ void integrate_granule(const DGrid& G, const DParams<
   T a1 = fma(M.ma, fa1, fma(M.m, P.g[1], fc1 + ff1)) * inv;
   T a2 = fma(M.ma, fa2, fma(M.m, P.g[2], fc2 + ff2)) * inv;
   T v0 = fma(P.dt, a0, v.x), v1 = fma(P.dt, a1, v.y), v2 = fma(P.dt, a2, v.z);
-  if (!isfinite(v0) || !isfinite(v1) || !isfinite(v2)) flags |= GIC_STATUS_NONFINITE;
+  if (!finite_bits(v0) || !finite_bits(v1) || !finite_bits(v2)) flags |= GIC_STATUS_NONFINITE;
   int c3[3] = {cell_x(c), cell_y(c), cell_z(c)};
   int cn[3];
   p_out = p;

@@ -131,6 +131,25 @@ inline unsigned grid_blocks(int64_t n, int threads) { return (unsigned)((n + thr
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 
+// Finite, from the exponent bits: a floating compare would occupy the FP64 pipe
+// (a 1 / 64 of the FP32 rate on this GPU).
+__device__ __forceinline__ bool finite_bits(float x) { return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u; }
+__device__ __forceinline__ bool finite_bits(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
+}
+
+// |x| as a float, truncated (relative error < 2^-23; 0 below 2^-126, large values
+// saturate at 2^127), with integer instructions: for pre-tests of FP64 values
+// off the FP64 pipe, which also converts.
+__device__ __forceinline__ float abs_trunc_f(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x) & 0x7fffffffu, lo = (uint32_t)__double2loint(x);
+  const uint32_t e = min(max(hi, 897u << 20), (1150u << 20)) - (896u << 20);  // rebias the exponent
+  return hi < (897u << 20) ? 0.f : __uint_as_float((e << 3) | (lo >> 29));
+}
+__device__ __forceinline__ float trunc_f(double x) {
+  return __uint_as_float(__float_as_uint(abs_trunc_f(x)) | ((uint32_t)__double2hiint(x) & 0x80000000u));
+}
+
 __device__ __forceinline__ int cell_x(int32_t c) { return c & (kMaxCellsPerAxis - 1); }
 __device__ __forceinline__ int cell_y(int32_t c) { return (c >> kCellBits) & (kMaxCellsPerAxis - 1); }
 __device__ __forceinline__ int cell_z(int32_t c) { return (c >> (2 * kCellBits)) & (kMaxCellsPerAxis - 1); }

@@ -15,7 +15,15 @@
 
 namespace gic {
 
+// CTAs of 256 threads; a small FP64 state takes CTAs of 64, at most four per SM, so
+// that it is spread over the chip: 8,000 granules in 32 CTAs kept 32 SMs busy and
+// 120 idle, and FP64 instructions issue at 1.8 lanes per clock and SM.  The 10-substep
+// window of 8,000 granules with one rebuild: 552 us in CTAs of 256, 433 in these.
+// (FP32 stays at 256: 467 against 446 us at 7,000 granules, and two partners'
+// opposite deposits cancel exactly inside one CTA's integer tile only.)
 constexpr int kSubstepThreads = 256;
+constexpr int kSmallThreads = 64;
+constexpr int64_t kSmallGranules = 4 * 152 * kSmallThreads;
 static_assert(kSubstepThreads == 32 * kSubWarps && kSubstepThreads + kSubstepThreads / 32 <= kSpreadStride,
               "the shared tile's warp arrays and the spread deposits are sized for CTAs of 256 threads");
 
@@ -39,9 +47,12 @@ static StateIn<T> state_in(const GicGranules* s) {
 // gic_step call that rebuilds, the staged neighbourhood of the list build.
 // Dynamic, so that the out-of-line build addresses it as shared memory.
 extern __shared__ __align__(16) unsigned char g_substep_smem[];
-constexpr size_t kBuildSmem = sizeof(TileShared<kSubstepThreads>);
-constexpr size_t kSubTileSmem = sizeof(SubTile) > kBuildSmem ? sizeof(SubTile) : kBuildSmem;
-static_assert(kSubTileSmem <= 48 * 1024, "more shared memory than a kernel has without asking");
+template <typename T, int NT>
+using SubShared = std::conditional_t<sizeof(T) == 4, SubTile, SubTile64<NT>>;
+template <typename T, int NT>
+constexpr size_t kSubSmem = sizeof(SubShared<T, NT>) > sizeof(TileShared<NT>) ? sizeof(SubShared<T, NT>)
+                                                                             : sizeof(TileShared<NT>);
+static_assert(kSubSmem<float, kSubstepThreads> <= 48 * 1024, "more shared memory than a kernel has without asking");
 
 // Contact (and bridge) force of sorted granule i from the 27 cells, walls
 // excluded, into vel_out[i] (which the granule's own thread reads and then
@@ -90,18 +101,18 @@ __device__ __forceinline__ void contact_walk(const DGrid& G, const DParams<T>& P
 // their lists no registers, and no launch of its own (an idle launch of one CTA
 // per 128 granules costs 2.3 ns per CTA: 20 us of every call on 1M granules).
 // The references are to the kernel's parameters.
-template <typename T, bool kCap>
+template <typename T, int NT, bool kCap>
 static __device__ __noinline__ void step_build(const DGrid& G, const DParams<T>& P, const StateIn<T>& S,
                                                const NbDev& nb, int64_t n, const T* af, const uint4* table, T skin,
                                                vec_t<T>* vel_out, uint32_t* status) {
-  TileShared<kSubstepThreads>& sh = *reinterpret_cast<TileShared<kSubstepThreads>*>(g_substep_smem);
+  TileShared<NT>& sh = *reinterpret_cast<TileShared<NT>*>(g_substep_smem);
   const uint32_t epoch = __ldg(&table[0].x);
-  const int64_t i = blockIdx.x * (int64_t)kSubstepThreads + threadIdx.x;
+  const int64_t i = blockIdx.x * (int64_t)NT + threadIdx.x;
   const bool valid = i < n;
   const int32_t ci = valid ? __ldg(&S.cell[i]) : 0;
   const FloatPos<T> fpos{S.cell, S.pos, S.posf, G.inv_hc};
-  const TileBox B = tile_stage<kSubstepThreads, T>(sh, G, table, epoch, fpos, valid, ci);
-  const bool over = build_row<kSubstepThreads, T, kCap, true>(sh, B, G, n, i, ci, fpos, S.id, table, epoch, nb,
+  const TileBox B = tile_stage<NT, T>(sh, G, table, epoch, fpos, valid, ci);
+  const bool over = build_row<NT, T, kCap, true>(sh, B, G, n, i, ci, fpos, S.id, table, epoch, nb,
                                                               (float)skin, (float)(T(1) + P.kappa));
   if (over) contact_walk<T, kCap>(G, P, S, af, table, epoch, i, vel_out, status);
   __syncthreads();  // the shared memory is the tile's from here on
@@ -115,8 +126,8 @@ static __device__ __noinline__ void step_build(const DGrid& G, const DParams<T>&
 // its code).
 enum SubMode { kGeneral, kStep, kStepCap };
 
-template <typename T, int kMode, bool kNoAlpha = false>
-__global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2)
+template <typename T, int kMode, bool kNoAlpha = false, int NT = kSubstepThreads>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 : 2)
     k_substep(const __grid_constant__ DGrid G, const __grid_constant__ DParams<T> P, int64_t n,
               const __grid_constant__ StateIn<T> state, const __grid_constant__ StateIn<T> sorted,
               const __grid_constant__ NbDev nb, const uint4* __restrict__ table, T skin, Fields<T> Fd,
@@ -135,10 +146,10 @@ __global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2)
   const int32_t* __restrict__ id = S.id;
   if constexpr (kMode != kGeneral)
     if (resorted)
-      step_build<T, kMode == kStepCap>(G, P, sorted, nb, n, Fd.af, table, skin, vel_out, status);
-  SubTile& sh = *reinterpret_cast<SubTile*>(g_substep_smem);  // FP32 path only
+      step_build<T, NT, kMode == kStepCap>(G, P, sorted, nb, n, Fd.af, table, skin, vel_out, status);
+  SubShared<T, NT>& sh = *reinterpret_cast<SubShared<T, NT>*>(g_substep_smem);
   const bool do_a = !kNoAlpha && alpha != nullptr, do_f = Fs_u != nullptr;
-  const int64_t i = blockIdx.x * (int64_t)kSubstepThreads + threadIdx.x;
+  const int64_t i = blockIdx.x * (int64_t)NT + threadIdx.x;
   const bool valid = i < n;
   const int32_t ci = valid ? cell[i] : 0;
   // the granule's own records, prefetched into L2 before the CTA's tile
@@ -154,9 +165,12 @@ __global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2)
       prefetch_l2(reinterpret_cast<const pos_t<T>*>(nb.ref_pos) + sl);
     }
   }
-  // FP32: the CTA's tile (fields staged for G2P, F_s / alpha_s accumulators)
-  SubBox B{};
-  if constexpr (sizeof(T) == 4) B = sub_tile_begin(sh, G, Fd, valid, ci, do_a, do_f);
+  // the CTA's tile: the fields staged for G2P, and (FP32) F_s / alpha_s accumulators
+  SubBox B;
+  if constexpr (sizeof(T) == 4)
+    B = sub_tile_begin(sh, G, Fd, valid, ci, do_a, do_f);
+  else
+    B = sub_tile64_begin<NT>(sh, G, Fd, valid, ci);
 
   int32_t co = 0;
   pos_t<T> pi{}, po{};
@@ -208,7 +222,7 @@ __global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2)
           add_walls(G, P, pi, ri, mi, vi, cx, cy, cz, F0, F1, F2, status);
       }
       if (coincident) flags |= GIC_STATUS_COINCIDENT;
-      if (!isfinite(F0) || !isfinite(F1) || !isfinite(F2)) flags |= GIC_STATUS_NONFINITE;
+      if (!finite_bits(F0) || !finite_bits(F1) || !finite_bits(F2)) flags |= GIC_STATUS_NONFINITE;
     }
     // a3: G2P coupling
     T Ffl[3], af[3];
@@ -216,8 +230,8 @@ __global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2)
     if constexpr (sizeof(T) == 4)
       sp = sub_g2p(sh, B, G, P, Fd, ci, pi, vi, Ffl, af);
     else
-      sp = g2p_granule(G, P, Fd, ci, pi, vi, Ffl, af);
-    if (!isfinite(sp)) flags |= GIC_STATUS_NONFINITE;
+      sp = sub_g2p64<NT>(sh, B, G, P, Fd, ci, pi, vi, Ffl, af);
+    if (!finite_bits(sp)) flags |= GIC_STATUS_NONFINITE;
     // a4: integrate into the next state
     vec_t<T> vo;
     integrate_granule(G, P, ci, pi, vi, F0, F1, F2, Ffl[0], Ffl[1], Ffl[2], af[0], af[1], af[2], co, po, vo, fe[0],
@@ -314,20 +328,8 @@ __global__ void __launch_bounds__(kSubstepThreads, sizeof(T) == 4 ? 4 : 2)
       granule_mac<T>(G, ci, pi, m, t);
       T* Fs[3] = {Fs_u, Fs_v, Fs_w};
 #pragma unroll
-      for (int comp = 0; comp < 3; ++comp) {
-        Stencil3<T> St = make_stencil<T>(G, m, t, comp);
-        const T fv = P.exch * fe[comp];
-        const int nsx = St.ns[0], nsy = St.ns[1];
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-          for (int b = 0; b < 2; ++b) {
-            T wyz = (b ? St.w[1] : T(1) - St.w[1]) * (c ? St.w[2] : T(1) - St.w[2]) * fv;
-            int64_t row = sample_index(nsx, nsy, St.i0[0], St.i0[1] + b, St.i0[2] + c);
-            atomicAdd(&Fs[comp][row], (T(1) - St.w[0]) * wyz);
-            atomicAdd(&Fs[comp][row + 1], St.w[0] * wyz);
-          }
-      }
+      for (int comp = 0; comp < 3; ++comp)
+        add_face64(G, Fs[comp], make_stencil<T>(G, m, t, comp), P.exch * fe[comp]);
     }
     if (sums) {
       double s = block_sum(Vi, s_red);
@@ -484,30 +486,45 @@ static int substep_launch(const DGrid& G, const GicParams* params, const GicGran
   const int64_t ncell = (int64_t)G.nx * G.ny * G.nz;
   if (alpha_s && (rc = alpha_begin(alpha_s, ncell, sums2, stream, scratch))) return rc;
   if (s->n > 0) {
-    const unsigned blocks = grid_blocks(s->n, kSubstepThreads);
-    auto go = [&](auto t, auto* kern, const DParams<decltype(t)>& P, size_t smem) {
+    auto go = [&](auto t, auto nt, auto* kern, const DParams<decltype(t)>& P) -> int {
       using T = decltype(t);
-      kern<<<blocks, kSubstepThreads, smem, stream>>>(
+      constexpr int NT = decltype(nt)::value;
+      constexpr size_t smem = kSubSmem<T, NT>;
+      if (smem > 48 * 1024 &&
+          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return set_error(GIC_ERR_CUDA, "substep: %zu bytes of shared memory refused", smem);
+      kern<<<grid_blocks(s->n, NT), NT, smem, stream>>>(
           G, P, s->n, state_in<T>(s), state_in<T>(sorted ? sorted : s), d, (const uint4*)cell_table, (T)nb->skin,
           fields<T>(u, v, w, p, alpha_f), next->cell, (pos_t<T>*)next->pos, (vec_t<T>*)next->vel, next->id,
           sizeof(T) == 4 ? (float4*)next->posf : nullptr, (vec_t<T>*)f_ex, alpha_s, (T*)Fs_u, (T*)Fs_v, (T*)Fs_w,
           sums2, status_word());
+      return GIC_OK;
     };
+    constexpr std::integral_constant<int, kSubstepThreads> kWhole{};
+    constexpr std::integral_constant<int, kSmallThreads> kSmall{};
     if (s->precision == GIC_FP32) {
       DParams<float> P;
       if ((rc = make_params(params, &P))) return rc;
-      go(0.f,
-         !sorted   ? k_substep<float, kGeneral>
-         : P.cap   ? k_substep<float, kStepCap>
-         : alpha_s ? k_substep<float, kStep>
-                   : k_substep<float, kStep, true>,
-         P, kSubTileSmem);
+      rc = go(0.f, kWhole,
+              !sorted   ? k_substep<float, kGeneral>
+              : P.cap   ? k_substep<float, kStepCap>
+              : alpha_s ? k_substep<float, kStep>
+                        : k_substep<float, kStep, true>,
+              P);
     } else {
       DParams<double> P;
       if ((rc = make_params(params, &P))) return rc;
-      go(0.0, !sorted ? k_substep<double, kGeneral> : P.cap ? k_substep<double, kStepCap> : k_substep<double, kStep>, P,
-         sorted ? kBuildSmem : 0);
+      if (sorted && s->n <= kSmallGranules)
+        rc = go(0.0, kSmall,
+                P.cap ? k_substep<double, kStepCap, false, kSmallThreads>
+                      : k_substep<double, kStep, false, kSmallThreads>,
+                P);
+      else
+        rc = go(0.0, kWhole,
+                !sorted ? k_substep<double, kGeneral> : P.cap ? k_substep<double, kStepCap> : k_substep<double, kStep>,
+                P);
     }
+    if (rc) return rc;
     count_launches(1);
   }
   if (alpha_s && (rc = alpha_end(G, s->precision, alpha_s, ncell, sums2, stream, scratch))) return rc;

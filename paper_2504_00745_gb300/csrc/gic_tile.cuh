@@ -49,8 +49,8 @@ constexpr int kTileThreads = 128;
 // The CTA's staged neighbourhood in shared memory.
 template <int NT>
 struct TileShared {
-  static constexpr int kCells = NT == 128 ? 512 : 768;
-  static constexpr int kGranules = NT == 128 ? 1152 : 2304;
+  static constexpr int kCells = NT <= 128 ? 512 : 768;
+  static constexpr int kGranules = NT <= 128 ? 1152 : 2304;
   int lo[3], hi[3];
   uint32_t start[kCells];
   uint32_t off[kCells + 1];  // first slot of each cell; at first its granule count
