@@ -450,13 +450,22 @@ __device__ __forceinline__ void p2g_sums(double* sums, long long v) {
 // gives the same bits) and zeroes its F_s (and alpha_s) accumulators; F_s is
 // then scattered into the same box (fixed point as in the P2G kernel), and
 // alpha_s, at the new positions, into it where the stencil fits.  A box
-// beyond kSubTile entries falls back to global memory.
+// beyond kSubTile entries falls back to global memory (1 to 3% of the CTAs, where
+// the Morton order jumps).
+//
+// Instruction issue and the latency of the first loads bound it (2.2 of 4
+// instructions per clock and SM, DRAM at a quarter of its rate), so the tile's
+// arithmetic is kept short: velocity and gradient of a sample in one 8-byte
+// entry, one index and seven loads per interior sample, the stencils formed once
+// for G2P and F_s, deposits rounded by the multiply-add that forms them.
+// 1702 -> 1400 instructions per warp on the 16M sweep; a gic_step call that
+// keeps its lists 1180 -> 1020 us there, 78 -> 67 us on the 1M dam break.
 constexpr int kSubTile = 960;  // 46 KB of static shared memory
-constexpr int kSubWarps = 8;  // CTA of 256 threads
+constexpr int kSubThreads = 256;
+constexpr int kSubWarps = kSubThreads / 32;
 
 struct SubTile {
-  float u[kSubTile], v[kSubTile], w[kSubTile];
-  float gp[3][kSubTile];
+  float2 ug[3][kSubTile];  // face velocity and face pressure gradient of each axis
   int32_t f[3][kSubTile];
   uint32_t a[3][kSubTile];
   int wlo[3][kSubWarps], whi[3][kSubWarps];
@@ -474,29 +483,19 @@ struct SubBox {
   }
 };
 
-// Sampler of a staged field: the same values as the global sampler.
-struct TileLoad {
-  const float* s;
-  SubBox B;
-  uint32_t* dbg;
-  __device__ __forceinline__ float operator()(int i, int j, int k) const {
-    const int e = B.index(i, j, k);
-    if (!GIC_DBG_OK(dbg, e >= 0 && e < B.vol)) return 0.f;
-    return s[e];
-  }
-};
-
 // CTA-wide (every thread calls it; one barrier): the box of samples m - 1 .. m + 1
 // per axis around the MAC cells of the CTA's granules, used as a tile when it
 // holds at most `most` of them.  valid: this thread has a granule in contact
 // cell c.
+template <int NT>
 __device__ __forceinline__ SubBox sub_box(int (&wlo)[3][kSubWarps], int (&whi)[3][kSubWarps], const DGrid& G,
                                           bool valid, int32_t c, int most) {
+  static_assert(NT % 32 == 0 && (NT & (NT - 1)) == 0 && NT / 32 <= kSubWarps, "lanes read the warps' extents in turn");
   const int warp = threadIdx.x >> 5;
   const int c3[3] = {cell_x(c), cell_y(c), cell_z(c)};
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    const int m = valid ? mac_of(G, c3[a]) : 0;
+    const int m = mac_of(G, c3[a]);
     const int l = __reduce_min_sync(0xffffffffu, valid ? m : INT_MAX);
     const int h = __reduce_max_sync(0xffffffffu, valid ? m : INT_MIN);
     if (lane_id() == 0) {
@@ -507,16 +506,13 @@ __device__ __forceinline__ SubBox sub_box(int (&wlo)[3][kSubWarps], int (&whi)[3
   __syncthreads();
   int lo[3], hi[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    lo[a] = INT_MAX;
-    hi[a] = INT_MIN;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      lo[a] = min(lo[a], wlo[a][w]);
-      hi[a] = max(hi[a], whi[a][w]);
-    }
+  for (int a = 0; a < 3; ++a) {  // one load and one reduction per bound instead of a loop over the warps
+    const int w = lane_id() & (NT / 32 - 1);
+    lo[a] = __reduce_min_sync(0xffffffffu, wlo[a][w]);
+    hi[a] = __reduce_max_sync(0xffffffffu, whi[a][w]);
   }
   SubBox B;
-  const bool any = lo[0] <= hi[0];  // a CTA without granules has lo > hi
+  const bool any = lo[0] <= hi[0];  // a CTA without granules has lo > hi: a box of one sample, no tile
   B.b[0] = any ? max(lo[0] - 1, 0) : 0;
   B.b[1] = any ? max(lo[1] - 1, 0) : 0;
   B.b[2] = any ? max(lo[2] - 1, 0) : 0;
@@ -530,27 +526,67 @@ __device__ __forceinline__ SubBox sub_box(int (&wlo)[3][kSubWarps], int (&whi)[3
   return B;
 }
 
+// The staged values of a sample at an end of the grid, or of none of the grids, out
+// of line (a few samples of the CTAs there).
+struct SubSample {
+  float2 s[3];
+};
+static __device__ __noinline__ SubSample sub_edge_sample(const DGrid& G, const Fields<float>& Fd, int i, int j,
+                                                         int k) {
+  const bool cx = i < G.nx, cy = j < G.ny, cz = k < G.nz;     // a cell-centred index
+  const bool fx = i <= G.nx, fy = j <= G.ny, fz = k <= G.nz;  // a face index
+  const bool in[3] = {fx && cy && cz, cx && fy && cz, cx && cy && fz};
+  const float* uvw[3] = {Fd.u, Fd.v, Fd.w};
+  SubSample S;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+    S.s[a] = in[a] ? make_float2(face_loader<float>(G, uvw[a], a)(i, j, k), gradp_loader<float>(G, Fd.p, a)(i, j, k))
+                   : make_float2(0.f, 0.f);
+  return S;
+}
+
+// e = lx + ex (ly + ey lz) of a box entry, by approximate reciprocals: (e + 1/2) / d
+// stays >= 1 / (2 d) from an integer, far beyond their error for e <= 1024.
+struct BoxSplit {
+  float rx, rxy;
+  __device__ __forceinline__ BoxSplit(const SubBox& B) {
+    rx = __fdividef(1.f, (float)B.sy);
+    rxy = __fdividef(1.f, (float)B.sz);
+  }
+  __device__ __forceinline__ void operator()(const SubBox& B, int e, int& i, int& j, int& k) const {
+    const int lz = (int)(((float)e + 0.5f) * rxy);
+    const int r = e - lz * B.sz;
+    const int ly = (int)(((float)r + 0.5f) * rx);
+    i = B.b[0] + r - ly * B.sy;
+    j = B.b[1] + ly;
+    k = B.b[2] + lz;
+  }
+};
+
 // CTA-wide (every thread calls it): the box, the staged fields and the zeroed
 // accumulators.
 __device__ __forceinline__ SubBox sub_tile_begin(SubTile& sh, const DGrid& G, const Fields<float>& Fd, bool valid,
                                                  int32_t c, bool do_a, bool do_f) {
-  const SubBox B = sub_box(sh.wlo, sh.whi, G, valid, c, kSubTile);
-  const float rx = 1.f / (float)B.ex, rxy = 1.f / (float)max(B.sz, 1);
-  for (int e = threadIdx.x; e < B.vol; e += blockDim.x) {
-    // e = lx + ex (ly + ey lz); (e + 1/2) / d stays >= 1/(2 d) from an integer
-    const int lz = (int)(((float)e + 0.5f) * rxy);
-    const int r = e - lz * B.sz;
-    const int ly = (int)(((float)r + 0.5f) * rx);
-    const int lx = r - ly * B.ex;
-    const int i = B.b[0] + lx, j = B.b[1] + ly, k = B.b[2] + lz;
-    const bool cx = i < G.nx, cy = j < G.ny, cz = k < G.nz;  // a cell-centred index
-    const bool fx = i <= G.nx, fy = j <= G.ny, fz = k <= G.nz;  // a face index
-    sh.u[e] = (fx && cy && cz) ? face_loader<float>(G, Fd.u, 0)(i, j, k) : 0.f;
-    sh.v[e] = (cx && fy && cz) ? face_loader<float>(G, Fd.v, 1)(i, j, k) : 0.f;
-    sh.w[e] = (cx && cy && fz) ? face_loader<float>(G, Fd.w, 2)(i, j, k) : 0.f;
-    sh.gp[0][e] = (fx && cy && cz) ? gradp_loader<float>(G, Fd.p, 0)(i, j, k) : 0.f;
-    sh.gp[1][e] = (cx && fy && cz) ? gradp_loader<float>(G, Fd.p, 1)(i, j, k) : 0.f;
-    sh.gp[2][e] = (cx && cy && fz) ? gradp_loader<float>(G, Fd.p, 2)(i, j, k) : 0.f;
+  const SubBox B = sub_box<kSubThreads>(sh.wlo, sh.whi, G, valid, c, kSubTile);
+  const BoxSplit split(B);
+  for (int e = threadIdx.x; e < B.vol; e += kSubThreads) {
+    int i, j, k;
+    split(B, e, i, j, k);
+    if (i >= 1 && i < G.nx && j >= 1 && j < G.ny && k >= 1 && k < G.nz) {
+      // inside: one index (below 2^31: cells have 30 bits) and the loaders' values,
+      // the three pressure differences sharing their upper sample
+      const int row = j + G.ny * k, q = i + G.nx * row;
+      const float u = __ldg(&Fd.u[q + row]), v = __ldg(&Fd.v[q + G.nx * k]), w = __ldg(&Fd.w[q]);
+      const float p = __ldg(&Fd.p[q]), px = __ldg(&Fd.p[q - 1]), py = __ldg(&Fd.p[q - G.nx]),
+                  pz = __ldg(&Fd.p[q - G.nx * G.ny]);
+      sh.ug[0][e] = make_float2(u, (p - px) * G.inv_dx_f);
+      sh.ug[1][e] = make_float2(v, (p - py) * G.inv_dx_f);
+      sh.ug[2][e] = make_float2(w, (p - pz) * G.inv_dx_f);
+    } else {
+      const SubSample S = sub_edge_sample(G, Fd, i, j, k);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) sh.ug[a][e] = S.s[a];
+    }
     if (do_f) sh.f[0][e] = sh.f[1][e] = sh.f[2][e] = 0;
     if (do_a) sh.a[0][e] = sh.a[1][e] = sh.a[2][e] = 0u;
   }
@@ -577,14 +613,11 @@ struct SubTile64 {
 template <int NT>
 __device__ __forceinline__ SubBox sub_tile64_begin(SubTile64<NT>& sh, const DGrid& G, const Fields<double>& Fd,
                                                    bool valid, int32_t c) {
-  const SubBox B = sub_box(sh.wlo, sh.whi, G, valid, c, SubTile64<NT>::kSamples);
-  const float rx = 1.f / (float)B.ex, rxy = 1.f / (float)max(B.sz, 1);
+  const SubBox B = sub_box<NT>(sh.wlo, sh.whi, G, valid, c, SubTile64<NT>::kSamples);
+  const BoxSplit split(B);
   for (int e = threadIdx.x; e < B.vol; e += NT) {
-    // e = lx + ex (ly + ey lz); (e + 1/2) / d stays >= 1/(2 d) from an integer
-    const int lz = (int)(((float)e + 0.5f) * rxy);
-    const int r = e - lz * B.sz;
-    const int ly = (int)(((float)r + 0.5f) * rx);
-    const int i = B.b[0] + r - ly * B.ex, j = B.b[1] + ly, k = B.b[2] + lz;
+    int i, j, k;
+    split(B, e, i, j, k);
     const bool cx = i < G.nx, cy = j < G.ny, cz = k < G.nz;     // a cell-centred index
     const bool fx = i <= G.nx, fy = j <= G.ny, fz = k <= G.nz;  // a face index
     sh.f[0][e] = (fx && cy && cz) ? face_loader<double>(G, Fd.u, 0)(i, j, k) : 0.0;
@@ -658,43 +691,78 @@ static __device__ __noinline__ G2POut g2p_global_f32(const DGrid G, const DParam
   return o;
 }
 
-// G2P of one granule from the staged tile (B.tile) or global memory.
-__device__ __forceinline__ float sub_g2p(const SubTile& sh, const SubBox& B, const DGrid& G, const DParams<float>& P,
-                                         const Fields<float>& Fd, int32_t c, const uint4& pi, const float4& vi,
-                                         float F[3], float a[3]) {
-  if (!B.tile) {
-    const G2POut o = g2p_global_f32(G, P, Fd, c, pi, vi);
+// A granule's stencils in the box: the weights of the upper sample per axis on
+// the face grid normal to it (wf) and on the others (wc), and the box index of
+// each face grid's base sample.  The values are make_stencil's.
+struct SubStencil {
+  float wf[3], wc[3];
+  int e0[3];
+};
+
+__device__ __forceinline__ SubStencil sub_stencil(const SubBox& B, const DGrid& G, int32_t c, const uint4& pi) {
+  SubStencil S;
+  int m[3];
+  granule_mac<float>(G, c, pi, m, S.wf);
+  const int n[3] = {G.nx, G.ny, G.nz}, str[3] = {1, B.sy, B.sz};
+  int up[3], sum = 0;
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      F[d] = o.F[d];
-      a[d] = o.a[d];
+  for (int a = 0; a < 3; ++a) {
+    const float t = S.wf[a];
+    const bool hi = t >= 0.5f;
+    int i0 = hi ? m[a] : m[a] - 1;
+    float w = hi ? t - 0.5f : t + 0.5f;
+    if (i0 < 0) {
+      i0 = 0;
+      w = 0.f;
+    } else if (i0 > n[a] - 2) {
+      i0 = n[a] - 2;
+      w = 1.f;
     }
-    return o.sp;
+    S.wc[a] = w;
+    sum += (i0 - B.b[a]) * str[a];
+    up[a] = (m[a] - i0) * str[a];
   }
-  const float* uvw[3] = {sh.u, sh.v, sh.w};
-  return g2p_granule_with<float>(
-      G, P, c, pi, vi, [&](int comp) { return TileLoad{uvw[comp], B, G.dbg}; },
-      [&](int comp) { return TileLoad{sh.gp[comp], B, G.dbg}; }, F, a);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) S.e0[a] = sum + up[a];
+  return S;
 }
 
-// CTA-wide: the F_s fixed-point unit from the largest |exch f_ex| component
-// of the CTA (M); returns 2^b / M (0 if F_s cannot use the tile).
+// G2P of one granule from the staged tile: interp's products and order.
+__device__ __forceinline__ float sub_g2p(const SubTile& sh, const SubBox& B, const SubStencil& S, const DGrid& G,
+                                         const DParams<float>& P, const uint4& pi, const float4& vi, float F[3],
+                                         float a[3]) {
+  float uf[3], gp[3];
+#pragma unroll
+  for (int comp = 0; comp < 3; ++comp) {
+    uf[comp] = gp[comp] = 0.f;
+    const float wx = comp == 0 ? S.wf[0] : S.wc[0], wy = comp == 1 ? S.wf[1] : S.wc[1],
+                wz = comp == 2 ? S.wf[2] : S.wc[2];
+    if (!GIC_DBG_OK(G.dbg, S.e0[comp] >= 0 && S.e0[comp] + 1 + B.sy + B.sz < B.vol)) continue;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float2 s = sh.ug[comp][S.e0[comp] + (k & 1) + ((k >> 1) & 1) * B.sy + (k >> 2) * B.sz];
+      const float w = mul_rn(mul_rn((k & 1) ? wx : 1.f - wx, (k & 2) ? wy : 1.f - wy), (k & 4) ? wz : 1.f - wz);
+      uf[comp] = fmaf(w, s.x, uf[comp]);
+      gp[comp] = fmaf(w, s.y, gp[comp]);
+    }
+  }
+  return coupling_forces<float>(P, radius_of(pi), vi, uf, gp, F, a);
+}
+
+// CTA-wide: the F_s fixed-point unit M 2^-b from the largest |exch f_ex|
+// component of the CTA (M); returns 2^b / M (0 if F_s cannot use the tile).
 __device__ __forceinline__ float sub_fs_scale(SubTile& sh, const SubBox& B, float Mthread, float& unit) {
-  const int warp = threadIdx.x >> 5;
   const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(Mthread));  // non-negative floats
-  if (lane_id() == 0) sh.wM[warp] = mb;
+  if (lane_id() == 0) sh.wM[threadIdx.x >> 5] = mb;
   __syncthreads();
-  unsigned M = 0u;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) M = max(M, sh.wM[w]);
-  const float Mc = __uint_as_float(M);
-  const int bits = 30 - (32 - __clz((int)blockDim.x - 1));  // 22 for 256 threads
+  const float Mc = __uint_as_float(__reduce_max_sync(0xffffffffu, sh.wM[lane_id() & (kSubWarps - 1)]));
+  constexpr float kScale = 4194304.f;  // 2^b, b = 30 - log2(threads)
+  static_assert(kSubThreads * 4194304ll == 1ll << 30, "one deposit per granule and entry sums below 2^30 units");
   const bool ok = B.tile && Mc >= 1e-30f && Mc <= 3.0e38f;
-  unit = ldexpf(Mc, -bits);
-  return ok ? ldexpf(1.0f, bits) / Mc : 0.f;
+  unit = Mc * (1.f / kScale);
+  return ok ? kScale / Mc : 0.f;
 }
 
-// F_s deposit of one granule on face grid comp (its stencil lies in the box
-// whenever the tile is used; inv_unit = 0: global atomics).
 // F_s deposit of one granule on face grid comp straight to global memory
 // (float atomics).
 __device__ __forceinline__ void add_face_global(const DGrid& G, float* Fs, int comp, const Stencil3<float>& St,
@@ -712,21 +780,22 @@ __device__ __forceinline__ void add_face_global(const DGrid& G, float* Fs, int c
   }
 }
 
-__device__ __forceinline__ void sub_add_face(SubTile& sh, const SubBox& B, const DGrid& G, float* Fs, int comp,
-                                             const Stencil3<float>& St, float fc, float inv_unit) {
-  if (inv_unit == 0.f) {
-    add_face_global(G, Fs, comp, St, fc);
-    return;
-  }
-  const float wx = St.w[0], wy = St.w[1], wz = St.w[2];
-  const float fx0 = (1.f - wx) * fc, fx1 = wx * fc;
-  const float wyz[4] = {(1.f - wy) * (1.f - wz), wy * (1.f - wz), (1.f - wy) * wz, wy * wz};
-  const int e0 = B.index(St.i0[0], St.i0[1], St.i0[2]);
+// F_s deposit of one granule on a face grid into the tile; wx, wy, wz the upper
+// weights, e0 the base sample and fcs the exchange force in units (|fcs| <= 2^22,
+// rounded).  Adding 1.5 2^23 in the multiply-add that forms a deposit leaves its
+// rounded value in the low bits: no conversion instruction, which issues at a
+// quarter of the rate.
+__device__ __forceinline__ void sub_add_face(int32_t* f, const SubBox& B, const DGrid& G, int e0, float wx, float wy,
+                                             float wz, float fcs) {
+  constexpr float kMagic = 12582912.f;
+  constexpr int kMagicBits = 0x4B400000;
   if (!GIC_DBG_OK(G.dbg, e0 >= 0 && e0 + 1 + B.sy + B.sz < B.vol)) return;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int q = __float2int_rn(((k & 1) ? fx1 : fx0) * wyz[k >> 1] * inv_unit);
-    atomicAdd(&sh.f[comp][e0 + (k & 1) + ((k >> 1) & 1) * B.sy + (k >> 2) * B.sz], q);
+  for (int r = 0; r < 4; ++r) {
+    const float a = (((r & 1) ? wy : 1.f - wy) * ((r & 2) ? wz : 1.f - wz)) * fcs;
+    int32_t* row = f + e0 + (r & 1) * B.sy + (r >> 1) * B.sz;
+    atomicAdd(row, __float_as_int(fmaf(1.f - wx, a, kMagic)) - kMagicBits);
+    atomicAdd(row + 1, __float_as_int(fmaf(wx, a, kMagic)) - kMagicBits);
   }
 }
 
@@ -746,42 +815,49 @@ static __device__ __noinline__ void fs_deposit_global(const DGrid G, float* Fs_u
 // stencil samples, and a shared-memory atomic takes one pass per lane on the
 // same address, so granule g's deposits are made by lane g / W of warp g % W
 // (W warps): the lanes of a warp then hold granules W apart, mostly in other
-// cells.  Each thread first parks its granule's inputs (packed MAC cell,
-// in-cell fractions, exchange force) in the alpha_s limbs' space, which a
-// call without alpha_s leaves unused; a CTA barrier separates the two sides.
-// The tile receives the same integer deposits as from the granules' own
-// threads.
-constexpr int kSpreadWords = 7;
-constexpr int kSpreadStride = 256 + 8;  // 256 granules, bank-skewed
+// cells.  Each thread parks its granule's stencils (packed box indices, weights)
+// when it forms them for G2P, and its exchange force later, in the alpha_s limbs'
+// space, which a call without alpha_s leaves unused; a CTA barrier separates the
+// two sides.  The tile receives the same integer deposits as from the
+// granules' own threads.
+constexpr int kSpreadWords = 10;
+constexpr int kSpreadStride = kSubThreads + kSubThreads / 32;  // bank-skewed
 static_assert(kSpreadWords * kSpreadStride <= 3 * kSubTile, "spread inputs exceed the alpha_s limbs");
+static_assert(kSubTile <= 1024, "three box indices in a word");
 __device__ __forceinline__ int spread_slot(int g) { return g + (g >> 5); }
 
-__device__ __forceinline__ void spread_put(SubTile& sh, bool valid, const int m[3], const float t[3],
-                                           const float fc[3]) {
-  float* s = reinterpret_cast<float*>(&sh.a[0][0]);
-  const int k = spread_slot(threadIdx.x);
-  s[k] = __int_as_float(valid ? (m[0] | (m[1] << 10) | (m[2] << 20)) : -1);
+// (before the granule's forces are known; a thread without a granule parks -1)
+__device__ __forceinline__ void spread_put_stencil(SubTile& sh, bool valid, const SubStencil& S) {
+  float* s = reinterpret_cast<float*>(&sh.a[0][0]) + spread_slot(threadIdx.x);
+  s[0] = __int_as_float(valid ? (S.e0[0] | (S.e0[1] << 10) | (S.e0[2] << 20)) : -1);
+  if (!valid) return;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    s[(1 + a) * kSpreadStride + k] = t[a];
-    s[(4 + a) * kSpreadStride + k] = fc[a];
+    s[(1 + a) * kSpreadStride] = S.wf[a];
+    s[(4 + a) * kSpreadStride] = S.wc[a];
   }
 }
+__device__ __forceinline__ void spread_put_force(SubTile& sh, const float fc[3]) {
+  float* s = reinterpret_cast<float*>(&sh.a[0][0]) + spread_slot(threadIdx.x);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) s[(7 + a) * kSpreadStride] = fc[a];
+}
 
-__device__ __forceinline__ void spread_deposit(SubTile& sh, const SubBox& B, const DGrid& G, float* const Fs[3],
-                                               float inv_unit) {
-  const int W = blockDim.x >> 5;
-  const int g = lane_id() * W + (threadIdx.x >> 5);
-  const float* s = reinterpret_cast<const float*>(&sh.a[0][0]);
-  const int k = spread_slot(g);
-  const int pm = __float_as_int(s[k]);
-  if (pm < 0) return;
-  const int m[3] = {pm & 1023, (pm >> 10) & 1023, pm >> 20};
-  const float t[3] = {s[kSpreadStride + k], s[2 * kSpreadStride + k], s[3 * kSpreadStride + k]};
+__device__ __forceinline__ void spread_deposit(SubTile& sh, const SubBox& B, const DGrid& G, float inv_unit) {
+  const int g = lane_id() * kSubWarps + (threadIdx.x >> 5);
+  const float* s = reinterpret_cast<const float*>(&sh.a[0][0]) + spread_slot(g);
+  const int e = __float_as_int(s[0]);
+  if (e < 0) return;
+  float wf[3], wc[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    wf[a] = s[(1 + a) * kSpreadStride];
+    wc[a] = s[(4 + a) * kSpreadStride];
+  }
 #pragma unroll
   for (int comp = 0; comp < 3; ++comp)
-    sub_add_face(sh, B, G, Fs[comp], comp, make_stencil<float>(G, m, t, comp), s[(4 + comp) * kSpreadStride + k],
-                 inv_unit);
+    sub_add_face(sh.f[comp], B, G, (e >> (10 * comp)) & 1023, comp == 0 ? wf[0] : wc[0], comp == 1 ? wf[1] : wc[1],
+                 comp == 2 ? wf[2] : wc[2], s[(7 + comp) * kSpreadStride] * inv_unit);
 }
 
 // alpha_s deposits of one granule at its new position: into the tile when
@@ -813,13 +889,10 @@ __device__ __forceinline__ void sub_tile_flush(SubTile& sh, const SubBox& B, con
                                                float* const Fs[3], bool do_a, bool fs_tile, float unit) {
   if (!B.tile || (!do_a && !fs_tile)) return;
   __syncthreads();
-  const float rx = 1.f / (float)B.ex, rxy = 1.f / (float)B.sz;
-  for (int e = threadIdx.x; e < B.vol; e += blockDim.x) {
-    const int lz = (int)(((float)e + 0.5f) * rxy);
-    const int r = e - lz * B.sz;
-    const int ly = (int)(((float)r + 0.5f) * rx);
-    const int lx = r - ly * B.ex;
-    const int gx = B.b[0] + lx, gy = B.b[1] + ly, gz = B.b[2] + lz;
+  const BoxSplit split(B);
+  for (int e = threadIdx.x; e < B.vol; e += kSubThreads) {
+    int gx, gy, gz;
+    split(B, e, gx, gy, gz);
     if (do_a) {  // non-zero only at samples of alpha_s
       const unsigned long long a = (unsigned long long)sh.a[0][e] + ((unsigned long long)sh.a[1][e] << 18) +
                                    ((unsigned long long)sh.a[2][e] << 36);

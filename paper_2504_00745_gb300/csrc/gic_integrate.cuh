@@ -25,12 +25,19 @@ __device__ __forceinline__ Masses<T> masses(const DParams<T>& P, T r) {
 __device__ __forceinline__ void advance_axis(const DGrid& G, float dt, float v, uint32_t q, int c, int nc,
                                              uint32_t& q_out, int& c_out, uint32_t& flags) {
   float inc_f = dt * v * G.inv_unit_f;
+  // a move of less than a cell that stays in the domain: 32-bit integers
+  if (fabsf(inc_f) < 0x1p30f && q <= kFracMask) {
+    const int s = (int)q + __float2int_rn(inc_f);
+    const int cn = c + (s >> kFracBits);  // floor division by 2^30
+    if (cn >= 0 && cn < nc) {
+      q_out = (uint32_t)s & kFracMask;
+      c_out = cn;
+      return;
+    }
+  }
   // clamp far beyond one cell so the integer conversion is defined
   inc_f = fminf(fmaxf(inc_f, -0x1p40f), 0x1p40f);
-  // the same rounding either way; the 64-bit conversion runs on the FP64
-  // pipe, so it is kept for moves of a cell or more (flagged as fast)
-  long long inc = fabsf(inc_f) < 0x1p30f ? (long long)__float2int_rn(inc_f) : __float2ll_rn(inc_f);
-  long long s = (long long)q + inc;
+  long long s = (long long)q + __float2ll_rn(inc_f);
   long long shift = s >> kFracBits;  // floor division by 2^30
   q_out = (uint32_t)(s & (long long)kFracMask);
   long long cn = (long long)c + shift;

@@ -21,11 +21,9 @@ namespace gic {
 // window of 8,000 granules with one rebuild: 552 us in CTAs of 256, 433 in these.
 // (FP32 stays at 256: 467 against 446 us at 7,000 granules, and two partners'
 // opposite deposits cancel exactly inside one CTA's integer tile only.)
-constexpr int kSubstepThreads = 256;
+constexpr int kSubstepThreads = kSubThreads;
 constexpr int kSmallThreads = 64;
 constexpr int64_t kSmallGranules = 4 * 152 * kSmallThreads;
-static_assert(kSubstepThreads == 32 * kSubWarps && kSubstepThreads + kSubstepThreads / 32 <= kSpreadStride,
-              "the shared tile's warp arrays and the spread deposits are sized for CTAs of 256 threads");
 
 // The granule arrays a substep reads.
 template <typename T>
@@ -122,19 +120,19 @@ static __device__ __noinline__ void step_build(const DGrid& G, const DParams<T>&
 // whether it rebuilds; kStep and kStepCap are gic_step's, without and with the
 // capillary force: in a call that rebuilds they read `sorted` and build its rows
 // first, out of line, so that the other calls' path carries no build code (a
-// smaller instruction footprint: 1317 -> 1286 us on the 16M sweep).  kNoAlpha: a call without alpha_s (the kernel then carries none of
-// its code).
+// smaller instruction footprint: 2% on the 16M sweep).  kNoAlpha: a call without
+// alpha_s (the kernel then carries none of its code).
 enum SubMode { kGeneral, kStep, kStepCap };
 
 template <typename T, int kMode, bool kNoAlpha = false, int NT = kSubstepThreads>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 : 2)
     k_substep(const __grid_constant__ DGrid G, const __grid_constant__ DParams<T> P, int64_t n,
               const __grid_constant__ StateIn<T> state, const __grid_constant__ StateIn<T> sorted,
-              const __grid_constant__ NbDev nb, const uint4* __restrict__ table, T skin, Fields<T> Fd,
-              int32_t* __restrict__ cell_out, pos_t<T>* __restrict__ pos_out, vec_t<T>* __restrict__ vel_out,
-              int32_t* __restrict__ id_out, float4* __restrict__ posf_out, vec_t<T>* __restrict__ fex_out,
-              double* __restrict__ alpha, T* __restrict__ Fs_u, T* __restrict__ Fs_v, T* __restrict__ Fs_w,
-              double* __restrict__ sums, uint32_t* status) {
+              const __grid_constant__ NbDev nb, const uint4* __restrict__ table, T skin,
+              const __grid_constant__ Fields<T> Fd, int32_t* __restrict__ cell_out, pos_t<T>* __restrict__ pos_out,
+              vec_t<T>* __restrict__ vel_out, int32_t* __restrict__ id_out, float4* __restrict__ posf_out,
+              vec_t<T>* __restrict__ fex_out, double* __restrict__ alpha, T* __restrict__ Fs_u,
+              T* __restrict__ Fs_v, T* __restrict__ Fs_w, double* __restrict__ sums, uint32_t* status) {
   // uniform over the launch
   const bool resorted = kMode != kGeneral && step_rebuilds(nb.flags);
   const bool rebuild = kMode == kGeneral && (nb.flags[kNbRebuild] | nb.flags[kNbSticky]) != 0u;
@@ -154,10 +152,13 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
   const int32_t ci = valid ? cell[i] : 0;
   // the granule's own records, prefetched into L2 before the CTA's tile
   // barriers (the loads themselves come after them; no register is held)
+  pos_t<T> pi{}, po{};
+  vec_t<T> vi{};
+  int32_t idi = 0;
   if (valid) {
     prefetch_l2(&pos[i]);
     prefetch_l2(&vel[i]);
-    if (posf) prefetch_l2(&posf[i]);
+    if (id_out && id) prefetch_l2(&id[i]);
     if (!rebuild) {
       const int32_t sl = nb.ident ? (int32_t)i : nb.at[i];
       prefetch_l2(&nb.count[sl]);  // (not the row: a whole line for a few entries)
@@ -173,12 +174,15 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
     B = sub_tile64_begin<NT>(sh, G, Fd, valid, ci);
 
   int32_t co = 0;
-  pos_t<T> pi{}, po{};
   T fe[3] = {T(0), T(0), T(0)};
   bool far = false;
+  const bool spread = sizeof(T) == 4 && do_f && !do_a && B.tile;  // uniform over the CTA
+  if constexpr (sizeof(T) == 4)
+    if (spread && !valid) spread_put_stencil(sh, false, SubStencil{});
   if (valid) {
     pi = pos[i];
-    const vec_t<T> vi = vel[i];
+    vi = vel[i];
+    if (id_out && id) idi = id[i];
     const T ri = radius_of(pi);
     const T mi = granule_mass(P, ri);
     uint32_t flags = 0;
@@ -189,7 +193,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
     {
       const int cx = cell_x(ci), cy = cell_y(ci), cz = cell_z(ci);
       const bool has_f = sizeof(T) == 4 && posf != nullptr;
-      const float4 fi = has_f ? __ldg(&posf[i]) : make_float4(0.f, 0.f, 0.f, 0.f);
+      float4 fi = make_float4(0.f, 0.f, 0.f, 0.f);
+      if constexpr (sizeof(T) == 4) fi = posf_of(ci, pi);  // its record in posf
       if (kMode != kGeneral && nb.count[i] < 0) {  // the row overflowed: step_build left the force here
         const vec_t<T> Fc = vel_out[i];
         F0 = Fc.x;
@@ -227,11 +232,32 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
     // a3: G2P coupling
     T Ffl[3], af[3];
     T sp;
-    if constexpr (sizeof(T) == 4)
-      sp = sub_g2p(sh, B, G, P, Fd, ci, pi, vi, Ffl, af);
-    else
+    if constexpr (sizeof(T) == 4) {
+      if (B.tile) {
+        const SubStencil St = sub_stencil(B, G, ci, pi);
+        if (spread) spread_put_stencil(sh, true, St);
+        sp = sub_g2p(sh, B, St, G, P, pi, vi, Ffl, af);
+      } else {
+        const G2POut o = g2p_global_f32(G, P, Fd, ci, pi, vi);
+        sp = o.sp;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          Ffl[d] = o.F[d];
+          af[d] = o.a[d];
+        }
+      }
+    } else
       sp = sub_g2p64<NT>(sh, B, G, P, Fd, ci, pi, vi, Ffl, af);
     if (!finite_bits(sp)) flags |= GIC_STATUS_NONFINITE;
+    // the record of the last build for the displacement test below, loaded before
+    // the stores (which may not be moved past)
+    int32_t rc = ci;
+    pos_t<T> rp = pi;  // (after a build this call's positions are the reference)
+    if (!rebuild) {
+      const int32_t sl = nb.ident ? (int32_t)i : nb.at[i];
+      rc = nb.ref_cell[sl];
+      rp = reinterpret_cast<const pos_t<T>*>(nb.ref_pos)[sl];
+    }
     // a4: integrate into the next state
     vec_t<T> vo;
     integrate_granule(G, P, ci, pi, vi, F0, F1, F2, Ffl[0], Ffl[1], Ffl[2], af[0], af[1], af[2], co, po, vo, fe[0],
@@ -240,20 +266,13 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
     cell_out[i] = co;
     pos_out[i] = po;
     vel_out[i] = vo;
-    if (id_out && id) id_out[i] = id[i];
+    if (id_out && id) id_out[i] = idi;
     if constexpr (sizeof(T) == 4) {
       if (posf_out) posf_out[i] = posf_of(co, po);
     }
     if (fex_out) fex_out[i] = make_vec<T>(fe[0], fe[1], fe[2]);
     // the next call's displacement test, on the positions just written
-    // (after a build this call's positions are the reference)
-    if (rebuild) {
-      far = moved_far(G, co, po, ci, pi, nb_lim2(nb, T(0)));
-    } else {
-      const int32_t sl = nb.ident ? (int32_t)i : nb.at[i];
-      far = moved_far(G, co, po, nb.ref_cell[sl], reinterpret_cast<const pos_t<T>*>(nb.ref_pos)[sl],
-                      nb_lim2(nb, T(0)));
-    }
+    far = moved_far(G, co, po, rc, rp, nb_lim2(nb, T(0)));
   }
   const bool cta_far = __any_sync(0xffffffffu, far) && lane_id() == 0;
   if (kMode == kGeneral && cta_far) atomicOr(&nb.flags[kNbNext], 1u);
@@ -262,19 +281,13 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
   if constexpr (sizeof(T) == 4) {
     const float fc[3] = {P.exch * fe[0], P.exch * fe[1], P.exch * fe[2]};
     float unit = 0.f, inv_unit = 0.f;
-    const bool spread = do_f && !do_a && B.tile;  // uniform over the CTA
     if (do_f) {  // the CTA's fixed-point unit
       float Mt = 0.f;
       if (valid) {
         const float m = fmaxf(fabsf(fc[0]), fmaxf(fabsf(fc[1]), fabsf(fc[2])));
         Mt = m <= 3.0e38f ? m : INFINITY;  // NaN or inf: no fixed point for this CTA
       }
-      if (spread) {  // park the deposit's inputs before the barrier in sub_fs_scale
-        int m[3] = {0, 0, 0};
-        float t[3] = {0.f, 0.f, 0.f};
-        if (valid) granule_mac<float>(G, ci, pi, m, t);
-        spread_put(sh, valid, m, t, fc);
-      }
+      if (spread && valid) spread_put_force(sh, fc);  // before the barrier in sub_fs_scale
       inv_unit = sub_fs_scale(sh, B, Mt, unit);
     }
     float* Fs[3] = {Fs_u, Fs_v, Fs_w};
@@ -285,17 +298,16 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
       alpha_deposits(G, co, po, ia, va, S);
       sub_add_alpha(sh, B, G, (unsigned long long*)alpha, ia, va);
     }
-    if (spread && inv_unit != 0.f) {
-      spread_deposit(sh, B, G, Fs, inv_unit);
-    } else if (kNoAlpha && valid && do_f) {  // inv_unit == 0 here: no tile for F_s
-      fs_deposit_global(G, Fs[0], Fs[1], Fs[2], ci, pi, fc[0], fc[1], fc[2]);
-    } else if (valid && do_f) {
-      int m[3];
-      float t[3];
-      granule_mac<float>(G, ci, pi, m, t);
+    if (inv_unit == 0.f) {  // (uniform) no tile for F_s
+      if (valid && do_f) fs_deposit_global(G, Fs[0], Fs[1], Fs[2], ci, pi, fc[0], fc[1], fc[2]);
+    } else if (spread) {
+      spread_deposit(sh, B, G, inv_unit);
+    } else if (!kNoAlpha && valid) {
+      const SubStencil St = sub_stencil(B, G, ci, pi);
 #pragma unroll
       for (int comp = 0; comp < 3; ++comp)
-        sub_add_face(sh, B, G, Fs[comp], comp, make_stencil<float>(G, m, t, comp), fc[comp], inv_unit);
+        sub_add_face(sh.f[comp], B, G, St.e0[comp], comp == 0 ? St.wf[0] : St.wc[0], comp == 1 ? St.wf[1] : St.wc[1],
+                     comp == 2 ? St.wf[2] : St.wc[2], fc[comp] * inv_unit);
     }
     sub_tile_flush(sh, B, G, (unsigned long long*)alpha, Fs, do_a, inv_unit != 0.f, unit);
     if (sums) p2g_sums(sums, (long long)S);
