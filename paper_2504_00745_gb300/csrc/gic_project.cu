@@ -589,13 +589,15 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_mg_up_red_dot(MgLevel L, Mg
 // in one CTA: their weights, invd and the right-hand side of `first` are copied
 // to shared memory (all copies in flight together), and every pass runs there with a barrier after it (16^3
 // and below: 16 us; with the levels in global memory, a barrier and an L2 round
-// trip per pass, 29 us).  On the coarsest level (every axis <= 4 cells, so
+// trip per pass, 29 us).  Up to 8192 cells, as many as fit: a level of 4500 to 7600
+// cells costs less here than in four launches (call on 24 x 44 x 34: 4290 -> 3770 us,
+// on 35 x 65 x 24: 5240 -> 4960).  On the coarsest level (every axis <= 4 cells, so
 // at most 32 pairs: one warp) red from x = 0, then kMgCoarsePairs (black, red)
 // sweep pairs.  Same-colour cells do not touch, so a half sweep reads only
 // values no thread of the pass writes.
 constexpr int kMgTailThreads = 1024;
-constexpr int kMgTailCells = 4096;
-constexpr size_t kMgTailSmem = 200 * 1024;
+constexpr int kMgTailCells = 8192;
+constexpr size_t kMgTailSmem = 224 * 1024;
 struct MgLevels {
   MgLevel l[kMgMaxLevels];
 };
