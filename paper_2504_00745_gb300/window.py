@@ -343,6 +343,11 @@ def _copy_state(dst: State, src: State):
         dst.posf.copy_(src.posf)
 
 
+def _state_like(st: State) -> State:
+    like = lambda t: None if t is None else torch.empty_like(t)
+    return State(like(st.cell), like(st.pos), like(st.vel), like(st.id), st.precision, like(st.posf))
+
+
 class GicWindow(torch.autograd.Function):
     """x_K = window(v0, c_drag, mu): K substeps from the simulator's initial
     state with initial velocities v0 (FP64 [n, 3], original order), drag
@@ -383,23 +388,23 @@ class GicWindow(torch.autograd.Function):
             gic.gic_neighbors_reset(sim.nb)
             sim.lists_current = True
         ckpts, lists = [], []
-        log = torch.zeros(K + 1, dtype=torch.int32, device=sim.device) if stepped else None
-        if stepped:
-            log[0:1].copy_(sim.nb.flags[4:5])
+        step = _Steps(sim, (sim.A, sim.A2)) if stepped else None
         for s in range(K):
             if s % ckpt == 0:
                 ckpts.append(sim.A.clone())
                 if stepped:
-                    lists.append(_lists_snapshot(sim.nb))
-            sim.substep(alpha=False, transfer=False, sums=False, sort_every=not stepped)
+                    lists.append(_lists_snapshot(sim.nb, rows=s > 0))
             if stepped:
-                log[s + 1:s + 2].copy_(sim.nb.flags[4:5])  # list builds so far (device copy, no wait)
+                step(s & 1, 1 - (s & 1))
+                sim.A, sim.A2 = sim.A2, sim.A
+            else:
+                sim.substep(alpha=False, transfer=False, sums=False, sort_every=True)
         x, _ = sim.positions()
         ctx.sim, ctx.K, ctx.ckpt, ctx.stepped = sim, K, ckpt, stepped
         ctx.ckpts, ctx.lists = ckpts, lists
-        # the window's build record, read once: the recomputation from each
-        # checkpoint repeats the forward pass exactly, builds included
-        ctx.build_log = log.tolist() if stepped else None
+        # the list words at every checkpoint and at the end, read once: the recomputation
+        # from each checkpoint repeats the forward pass exactly, builds included
+        ctx.words = torch.stack([q["flags"] for q in lists] + [sim.nb.flags]).tolist() if stepped else None
         ctx.final = sim.A.clone()
         return x
 
@@ -427,28 +432,76 @@ def _segments(K: int, ckpt: int):
 _NB_ARRAYS = ("list", "count", "ref_cell", "ref_pos", "slot")
 
 
-def _lists_snapshot(nb: gic.Neighbors) -> dict:
+# flag words of the lists: what makes the next gic_step rebuild, and the build count
+_REQUESTED, _BUILDS, _NEXT = 1, 4, 5
+
+
+def _lists_snapshot(nb: gic.Neighbors, rows: bool = True) -> dict:
     """The Verlet lists as they stand, copied on the device without waiting
     for them: the flag words (among them the decision for the next gic_step
     and the build count) and the rows and reference entries (`cur` and `at`
     follow from them at the next check).  When a build is pending the rows
-    are not used: restoring the flags makes the next call rebuild."""
-    return {"flags": nb.flags.clone(), "arrays": {a: getattr(nb, a).clone() for a in _NB_ARRAYS}}
+    are not used (rows = False: known to be so): restoring the flags makes the
+    next call rebuild."""
+    return {"flags": nb.flags.clone(), "arrays": {a: getattr(nb, a).clone() for a in _NB_ARRAYS} if rows else None}
 
 
-def _lists_restore(nb: gic.Neighbors, snap: dict):
+def _lists_restore(nb: gic.Neighbors, snap: dict, rows: bool = True):
     nb.flags.copy_(snap["flags"])
-    if snap["arrays"] is not None:
+    if rows and snap["arrays"] is not None:
         for a, t in snap["arrays"].items():
             getattr(nb, a).copy_(t)
+
+
+class _Steps:
+    """gic_step without alpha_s, F_s and sums between the states of one pass
+    over a window, and the substep adjoint on them, on torch's current stream.
+    The arguments, the same for every call of the pass but the states and the
+    gradient arrays, are converted once (24 us of host time per call otherwise, as
+    much as the device takes for 100,000 granules; 12 us so).  An object lives no
+    longer than the pass and holds every tensor that it points to."""
+
+    def __init__(self, sim: "Simulator", states, grads=(), scalars=None):
+        F, nb = sim.fluid, sim.nb
+        self.hold = (sim.grid, sim.params, states, sim.B, sim.perm, sim.table, sim.ws, nb.__dict__.copy(), F, grads,
+                     scalars)
+        ptr, ref = gic._ptr, gic.C.byref
+        self.states = [ref(st.struct()) for st in states]
+        self.sorted, self.perm = ref(sim.B.struct()), ptr(sim.perm)
+        self.head = (ref(sim.grid), ref(sim.params))
+        self.lists = ref(nb.struct())
+        self.fields = tuple(ptr(f) for f in (F.u, F.v, F.w, F.p, F.alpha_f))
+        self.table = ptr(sim.table)
+        self.scratch = (ptr(sim.ws), sim.ws.numel() * sim.ws.element_size())
+        self.grads = [(ptr(a), ptr(b)) for a, b in grads]
+        self.scalars = (ptr(scalars[0:1]), ptr(scalars[1:2])) if scalars is not None else (None, None)
+        self.stream = gic._stream(None)
+        self.lib = gic.lib()
+
+    def __call__(self, k: int, to: int):
+        """State k -> state to."""
+        gic._check(self.lib.gic_step(*self.head, self.states[k], self.states[to], self.sorted, self.perm, self.table,
+                                     *self.scratch, self.lists, *self.fields, None, None, None, None, None,
+                                     self.stream), "gic_step")
+
+    def adjoint(self, k: Optional[int], g: int):
+        """Gradients g -> gradients 1 - g, through the substep on state k, or on
+        the sorted state (k None)."""
+        gic._check(self.lib.gic_substep_adj(*self.head, self.sorted if k is None else self.states[k],
+                                            self.perm if k is None else None, self.table, self.lists, *self.fields,
+                                            *self.grads[g], None, *self.grads[1 - g], *self.scalars, self.stream),
+                   "gic_substep_adj")
 
 
 def _backward_stepped(ctx, g_pos, g_vel, g_scalars):
     sim, nb, F = ctx.sim, ctx.sim.nb, ctx.sim.fluid
     n, prec, dev = sim.n, sim.precision, sim.device
-    g_pos_n = gic.vec4(n, prec, dev)
-    g_vel_n = gic.vec4(n, prec, dev)
     ends, expected = [], []
+    # a segment's states: its checkpoint and what its substeps make of it, in buffers
+    # shared by the segments
+    work = [_state_like(ctx.final) for _ in range(min(ctx.ckpt, ctx.K))]
+    grads = ((g_pos, g_vel), (gic.vec4(n, prec, dev), gic.vec4(n, prec, dev)))
+    g = 0  # the pair that holds the gradients of the state reached
 
     def sort_and_build(st: State):
         """st sorted into B (perm, cell table) and the lists built from B
@@ -462,44 +515,55 @@ def _backward_stepped(ctx, g_pos, g_vel, g_scalars):
         else:
             gic.gic_contact_verlet(sim.grid, sim.params, sim.B, sim.table, nb, sim.F_c)
 
+    rows_of = None  # the build (by the window's count) whose rows the lists hold; None: not known
     for m, (s0, s1) in zip(reversed(range(len(ctx.ckpts))), _segments(ctx.K, ctx.ckpt)):
         L = s1 - s0
-        # recompute the segment from its checkpoint and lists, keeping the state before every substep
-        _copy_state(sim.A, ctx.ckpts[m])
-        _lists_restore(nb, ctx.lists[m])
+        begin, end = ctx.words[m], ctx.words[m + 1]
+        states = [ctx.ckpts[m]] + work[:L]
+        step = _Steps(sim, states, grads, g_scalars)
+        # the checkpoint's lists; a pending build makes its own rows, and the segments
+        # of one build share theirs
+        pending = (begin[_REQUESTED] | begin[_NEXT]) != 0
+        _lists_restore(nb, ctx.lists[m], rows=not pending and rows_of != begin[_BUILDS])
         sim.lists_current = True
-        states = []
-        for k in range(L):
-            states.append(sim.A.clone())
-            sim.substep(alpha=False, transfer=False, sums=False)
-        counts = ctx.build_log[s0:s1 + 1]  # the forward pass's record: the recomputation repeats it
-        built = [counts[k + 1] != counts[k] for k in range(L)]
+        # recompute the segment: the state before every substep, and which substeps
+        # rebuilt the lists (the forward pass's record: the recomputation repeats it)
+        known = end[_BUILDS] - begin[_BUILDS] == int(pending)  # no build but the pending one
+        if known:
+            built = [pending] + [False] * (L - 1)
+            for k in range(L if L == 1 and pending else L - 1):  # nothing reads what the last one makes
+                step(k, k + 1)
+        else:
+            log = torch.empty(L, dtype=torch.int32, device=dev)
+            for k in range(L):
+                step(k, k + 1)
+                log[k:k + 1].copy_(nb.flags[_BUILDS:_BUILDS + 1])
+            at = [begin[_BUILDS]] + log.tolist()
+            built = [at[k + 1] != at[k] for k in range(L)]
+        rows_of = end[_BUILDS]
         # the substep whose build made the lists substep k walked (-1: the checkpoint's)
         last_build = [max([j for j in range(k + 1) if built[j]], default=-1) for k in range(L)]
-        lists_of, count_now = last_build[L - 1], counts[L]
+        lists_of, count_now = last_build[L - 1], end[_BUILDS]
         for k in reversed(range(L)):
             b = last_build[k]
             if b != lists_of and b != k:  # restore the lists substep k walked
                 if b < 0:
                     _lists_restore(nb, ctx.lists[m])
-                    count_now = ctx.build_log[s0]
+                    rows_of = count_now = begin[_BUILDS]
                 else:
                     sort_and_build(states[b])
-                    count_now = 1  # a reset clears the build count
+                    rows_of, count_now = None, 1  # a reset clears the build count
                 lists_of = b
             if built[k]:  # substep k sorted its state and built the lists from it: the adjoint runs there
                 if lists_of != k:
                     sort_and_build(states[k])
-                    lists_of, count_now = k, 1
+                    rows_of, lists_of, count_now = None, k, 1
                 else:
                     gic.gic_sort(sim.grid, states[k], sim.B, sim.perm, sim.table, sim.ws)
-                acted, perm = sim.B, sim.perm
+                step.adjoint(None, g)
             else:  # substep k ran on its state as it was, and its result kept the order
-                acted, perm = states[k], None
-            gic.gic_substep_adj(sim.grid, sim.params, acted, perm, sim.table, nb, F.u, F.v, F.w, F.p, F.alpha_f,
-                                g_pos, g_vel, None, g_pos_n, g_vel_n, g_scalars[0:1], g_scalars[1:2])
-            g_pos, g_pos_n = g_pos_n, g_pos
-            g_vel, g_vel_n = g_vel_n, g_vel
+                step.adjoint(k, g)
+            g = 1 - g
         ends.append(nb.flags[4:5].clone())
         expected.append(count_now)
     sim.lists_current = False
@@ -507,7 +571,7 @@ def _backward_stepped(ctx, g_pos, g_vel, g_scalars):
     got = torch.cat(ends).tolist()
     if got != expected:
         raise RuntimeError(f"Verlet lists were rebuilt inside the adjoint (builds {got}, expected {expected})")
-    return g_vel
+    return grads[g][1]
 
 
 def _backward_sorted(ctx, g_pos, g_vel, g_scalars):
