@@ -246,7 +246,7 @@ typedef struct GicNeighbors {
   uint32_t* flags;   /* [8]: [0] rebuild in this call, [1] bit 0 rebuild requested, bit 1 a list overflowed at the
                       * last build, [2] CTA counter, [3] overflow during a build, [4] builds performed, [5] a
                       * granule written by the last substep kernel is beyond skin / 2 (read by gic_step),
-                      * [6] arrivals at the sort's grid barriers */
+                      * [6] arrivals at the sort's grid barriers, [7] the sort of this gic_step is done */
 } GicNeighbors;
 
 int gic_contact_verlet(const GicGrid* grid, const GicParams* params, const GicGranules* sorted,

@@ -361,7 +361,10 @@ __device__ __forceinline__ void for_each_contact(const DGrid& G, const uint4* __
 // every call); kNbCounter -- CTAs done; kNbOverflow -- overflow during this
 // build; kNbBuilds -- builds so far; kNbNext -- a granule written by a
 // k_substep is beyond skin / 2 of its reference (gic_step's next call
-// rebuilds; gic_step consumes the word); kNbBarrier -- arrivals at the grid
+// rebuilds; gic_step consumes the word); kNbSorted -- this gic_step call sorted,
+// so its substep kernel takes the sorted state (set when the sort is done,
+// cleared with the call; unlike the request words it does not change
+// while that kernel's CTAs start); kNbBarrier -- arrivals at the grid
 // barriers of gic_step's sort (0 between calls).
 
 enum : int {
@@ -372,6 +375,7 @@ enum : int {
   kNbBuilds = 4,
   kNbNext = 5,
   kNbBarrier = 6,
+  kNbSorted = 7,
   kNbWords = 8
 };
 // The count of a row that overflowed in gic_step's build: the granule's contact
@@ -625,8 +629,9 @@ int verlet_view(const DGrid& G, const GicGranules* s, const void* table, const G
 int verlet_check(const DGrid& G, const GicGranules* s, const void* table, const GicNeighbors* nb,
                  cudaStream_t stream, const char* what, NbDev* out, GicGranules* copy_to, int32_t* perm);
 
-// This gic_step call rebuilds: a granule was beyond skin / 2 of its reference
-// after the last one, or a rebuild was requested.
+// This gic_step call is to rebuild: a granule was beyond skin / 2 of its reference
+// after the last one, or a rebuild was requested.  For the sort kernel alone:
+// a substep kernel's CTAs set kNbNext while others have yet to start.
 __device__ __forceinline__ bool step_rebuilds(const uint32_t* flags) {
   return (flags[kNbNext] | flags[kNbSticky]) != 0u;
 }
@@ -716,8 +721,8 @@ __device__ __forceinline__ void step_call_done(const NbDev& nb, bool rebuilt, bo
     if (far) atomicOr(&nb.flags[kNbNext], 1u);
     return;
   }
-  // the rebuild words are read by every CTA at its start: what this call asks of
-  // the next one goes to kNbRebuild until the last CTA is done
+  // kNbNext still holds what this call answered: what it asks of the next one
+  // goes to kNbRebuild until the last CTA is done
   if (far) atomicOr(&nb.flags[kNbRebuild], 1u);
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -727,6 +732,7 @@ __device__ __forceinline__ void step_call_done(const NbDev& nb, bool rebuilt, bo
       nb.flags[kNbNext] = atomicExch(&nb.flags[kNbRebuild], 0u);
       nb.flags[kNbSticky] = atomicExch(&nb.flags[kNbOverflow], 0u) ? 2u : 0u;
       nb.flags[kNbBuilds] += 1u;
+      nb.flags[kNbSorted] = 0u;
       nb.flags[kNbCounter] = 0u;
       __threadfence();
     }

@@ -90,9 +90,11 @@ __global__ void __launch_bounds__(kStepSortThreads, kStepSortCtas)
   for (int64_t k = blockIdx.x * (int64_t)kStepSortThreads + threadIdx.x; k < A.n;
        k += (int64_t)gridDim.x * kStepSortThreads)
     sort_gather<T>(A.G, A.n, k, keys, A.S, A.table, A.status);
-  // past the last barrier: the last CTA clears the count of arrivals
+  // past the last barrier: the last CTA clears the count of arrivals and tells the
+  // substep kernel
   if (threadIdx.x == 0 && atomicAdd(&A.flags[kNbCounter], 1u) == gridDim.x - 1) {
     A.flags[kNbBarrier] = 0u;
+    A.flags[kNbSorted] = 1u;
     A.flags[kNbCounter] = 0u;
   }
 }

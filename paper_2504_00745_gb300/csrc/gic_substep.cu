@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
               vec_t<T>* __restrict__ fex_out, double* __restrict__ alpha, T* __restrict__ Fs_u,
               T* __restrict__ Fs_v, T* __restrict__ Fs_w, double* __restrict__ sums, uint32_t* status) {
   // uniform over the launch
-  const bool resorted = kMode != kGeneral && step_rebuilds(nb.flags);
+  const bool resorted = kMode != kGeneral && nb.flags[kNbSorted] != 0u;
   const bool rebuild = kMode == kGeneral && (nb.flags[kNbRebuild] | nb.flags[kNbSticky]) != 0u;
   const StateIn<T> S = resorted ? sorted : state;
   const int32_t* __restrict__ cell = S.cell;
