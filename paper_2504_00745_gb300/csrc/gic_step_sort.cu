@@ -68,7 +68,10 @@ template <typename T>
 __global__ void __launch_bounds__(kStepSortThreads, kStepSortCtas)
     k_step_sort(const __grid_constant__ StepSortArgs<T> A) {
   __shared__ SortShared<kStepSortThreads> sh;
-  if (!step_rebuilds(A.flags)) return;  // uniform: the words change only in the substep kernels
+  if (!step_rebuilds(A.flags)) {  // uniform: the words change only in the substep kernels
+    asm volatile("griddepcontrol.launch_dependents;");  // the substep kernel may start
+    return;
+  }
   uint32_t arrived = 0;
   auto barrier = [&]() { return grid_barrier(&A.flags[kNbBarrier], arrived += gridDim.x, A.status); };
   // the radix passes, ping-ponging between the two key / value buffers
