@@ -796,6 +796,70 @@ __device__ __forceinline__ void for_each_list_contact(const DGrid& G, const NbDe
   }
 }
 
+// The partners j of granule i's Verlet row that pass the float pre-test reach(r_j)
+// (contact cells), in row order: f(j).  FP32 states with posf.  In two passes over up
+// to `most` partners at a time: the pre-test of the row, which leaves the
+// candidates in this thread's list (entry k at list[k * stride]), then f for those.
+// With both in one loop the warp runs f for every row position at which any
+// lane has a contact, as often as its longest row; so it runs it as often as its
+// longest list, and a candidate's records are loaded together.  A call that keeps
+// its lists: 8M bed (rows of 0 to 40) 1230 -> 903 us, dense packing of 1M 215 -> 195;
+// the adjoint there 1996 -> 1338 and 320 -> 299.  (The capillary walk, where
+// nearly every entry of a row is a bridge or a contact, is 5% slower with it.)
+template <typename Reach, typename F>
+__device__ __forceinline__ void for_each_list_candidate(const NbDev& nb, int64_t i, const float4& fi,
+                                                        const float4* __restrict__ posf, uint32_t* list, int stride,
+                                                        int most, Reach reach, F f) {
+  const int32_t s = nb.ident ? (int32_t)i : nb.at[i];
+  const int32_t* row = nb.list + (int64_t)s * nb.cap;
+  int cnt = nb.count[s];
+  if (!GIC_DBG_OK(nb.dbg, cnt >= 0 && cnt <= nb.cap)) cnt = 0;
+  for (int k = 0; k < cnt;) {
+    int hits = 0;
+    for (; k < cnt && hits + 4 <= most; k += 4) {
+      int32_t jj[4];
+      float4 fj[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        jj[u] = k + u < cnt ? (nb.ident ? row[k + u] : nb.cur[row[k + u]]) : -1;
+        if (jj[u] >= 0 && !GIC_DBG_OK(nb.dbg, jj[u] < nb.n)) jj[u] = -1;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) fj[u] = jj[u] >= 0 ? __ldg(&posf[jj[u]]) : fi;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float rx = fj[u].x - fi.x, ry = fj[u].y - fi.y, rz = fj[u].z - fi.z;
+        const float Rc = reach(fj[u].w);
+        if (jj[u] >= 0 && fmaf(rx, rx, fmaf(ry, ry, rz * rz)) < Rc * Rc) list[stride * hits++] = (uint32_t)jj[u];
+      }
+    }
+    for (int h = 0; h < hits; ++h) f(list[stride * h]);
+  }
+}
+
+// for_each_list_contact over candidate lists: f(j, g, v_j, r_j).
+template <typename F>
+__device__ __forceinline__ void for_each_list_hit(const DGrid& G, const NbDev& nb, int64_t i, int cx, int cy, int cz,
+                                                  const uint4& pi, float ri, const float4& fi,
+                                                  const int32_t* __restrict__ cell, const uint4* __restrict__ pos,
+                                                  const float4* __restrict__ posf, const float4* __restrict__ vel,
+                                                  uint32_t* list, int stride, int most, F f) {
+  for_each_list_candidate(
+      nb, i, fi, posf, list, stride, most, [&](float rj) { return fmaf(ri + rj, G.inv_hc_f, kPosfTol); },
+      [&](uint32_t j) {
+        const int32_t cj = __ldg(&cell[j]);
+        const uint4 pj = __ldg(&pos[j]);
+        const float4 vj = __ldg(&vel[j]);
+        const int ox = cell_x(cj) - cx, oy = cell_y(cj) - cy, oz = cell_z(cj) - cz;
+        // partners two or more cells apart are farther than h_c >= 2 r_max
+        if (ox < -1 || ox > 1 || oy < -1 || oy > 1 || oz < -1 || oz > 1) return;
+        int Dx, Dy, Dz;
+        int_sep(pi, pj, ox, oy, oz, Dx, Dy, Dz);
+        PairGeom<float> g;
+        if (pair_geom_exact(G, Dx, Dy, Dz, ri, radius_of(pj), g)) f(j, g, vj, radius_of(pj));
+      });
+}
+
 // Forces of the partners in granule i's Verlet row (the list walk of
 // gic_contact_verlet).
 template <typename T>

@@ -826,6 +826,9 @@ static_assert(kSpreadWords * kSpreadStride <= 3 * kSubTile, "spread inputs excee
 static_assert(kSubTile <= 1024, "three box indices in a word");
 __device__ __forceinline__ int spread_slot(int g) { return g + (g >> 5); }
 
+// This thread's words of that space, kSpreadStride apart.
+__device__ __forceinline__ uint32_t* spread_words(SubTile& sh) { return &sh.a[0][0] + spread_slot(threadIdx.x); }
+
 // (before the granule's forces are known; a thread without a granule parks -1)
 __device__ __forceinline__ void spread_put_stencil(SubTile& sh, bool valid, const SubStencil& S) {
   float* s = reinterpret_cast<float*>(&sh.a[0][0]) + spread_slot(threadIdx.x);

@@ -182,6 +182,9 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
   const bool spread = sizeof(T) == 4 && do_f && !do_a && B.tile;  // uniform over the CTA
   if constexpr (sizeof(T) == 4)
     if (spread && !valid) spread_put_stencil(sh, false, SubStencil{});
+  // the candidates' list of the contact walk: the words in which this thread parks
+  // its stencils afterwards
+  constexpr bool kHitList = sizeof(T) == 4 && kMode == kStep && kNoAlpha;
   if (valid) {
     pi = pos[i];
     vi = vel[i];
@@ -220,8 +223,18 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
         verlet_build_granule(G, P, nb, table, n, i, cx, cy, cz, ci, pi, ri, mi, vi, has_f, fi, skin, id, pos, posf,
                              vel, F0, F1, F2, coincident);
       } else {
-        verlet_list_force(G, P, nb, i, cx, cy, cz, ci, pi, ri, mi, vi, has_f, fi, cell, pos, posf, vel, F0, F1, F2,
-                          coincident);
+        bool walked = false;
+        if constexpr (kHitList)
+          if (has_f) {
+            for_each_list_hit(G, nb, i, cx, cy, cz, pi, ri, fi, cell, pos, posf, vel, spread_words(sh), kSpreadStride,
+                              kSpreadWords, [&](uint32_t, const PairGeom<float>& g, const float4& vj, float rj) {
+                                add_force(P, g, vi, vj, mi, rj, F0, F1, F2, coincident);
+                              });
+            walked = true;
+          }
+        if (!walked)
+          verlet_list_force(G, P, nb, i, cx, cy, cz, ci, pi, ri, mi, vi, has_f, fi, cell, pos, posf, vel, F0, F1, F2,
+                            coincident);
       }
       if (P.walls) {
         if constexpr (sizeof(T) == 4)
@@ -358,6 +371,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
 }
 
 constexpr int kSubstepAdjThreads = 128;
+constexpr int kAdjHits = 12;
 
 // Adjoint of k_substep's granule outputs (next position, velocity, f_ex) for
 // one granule of the sorted state: the integration's adjoint gives the
@@ -375,6 +389,7 @@ __global__ void __launch_bounds__(kSubstepAdjThreads, sizeof(T) == 4 ? 6 : 3) k_
     vec_t<T>* __restrict__ gxi, vec_t<T>* __restrict__ gvi, double* __restrict__ g_cdrag,
     double* __restrict__ g_mu) {
   __shared__ double s_red[64];
+  __shared__ uint32_t s_list[sizeof(T) == 4 ? kAdjHits : 1][kSubstepAdjThreads];  // candidates of the contact walk
   const bool rebuild = (nb.flags[kNbRebuild] | nb.flags[kNbSticky]) != 0u;  // uniform over the launch
   const int64_t i = blockIdx.x * (int64_t)kSubstepAdjThreads + threadIdx.x;
   T my_gc = T(0), my_gmu = T(0);
@@ -401,15 +416,14 @@ __global__ void __launch_bounds__(kSubstepAdjThreads, sizeof(T) == 4 ? 6 : 3) k_
     // a2: contact pairs (F_ji = -F_ij) and walls
     const T l0 = o.gFc[0], l1 = o.gFc[1], l2 = o.gFc[2];
     T gm = T(0);
-    auto pair = [&](int64_t j, const PairGeom<T>& g) {
-      const vec_t<T> vj = ldg(&vel[j]);
-      const T rj = radius_of(ldg(&pos[j]));
+    auto pair_of = [&](int64_t j, const PairGeom<T>& g, const vec_t<T>& vj, T rj) {
       const IntegrateAdj<T> oj =
           integrate_adj_granule(P, rj, ldg(&gxo[j]), ldg(&gvo[j]), gfe ? ldg(&gfe[j]) : zero);
       gm += pair_force_adj(P, g.x0, g.x1, g.x2, g.d, g.overlap, vi.x - vj.x, vi.y - vj.y, vi.z - vj.z,
                            pair_mass(P, mi, rj), l0 - oj.gFc[0], l1 - oj.gFc[1], l2 - oj.gFc[2], l0, l1, l2, gx[0],
                            gx[1], gx[2], gv[0], gv[1], gv[2]);
     };
+    auto pair = [&](int64_t j, const PairGeom<T>& g) { pair_of(j, g, ldg(&vel[j]), radius_of(ldg(&pos[j]))); };
     const int cx = cell_x(ci), cy = cell_y(ci), cz = cell_z(ci);
     const bool has_f = sizeof(T) == 4 && posf != nullptr;
     const float4 fi = has_f ? __ldg(&posf[i]) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -437,7 +451,14 @@ __global__ void __launch_bounds__(kSubstepAdjThreads, sizeof(T) == 4 ? 6 : 3) k_
     } else if (rebuild) {
       verlet_build_row<T>(G, nb, table, n, i, cx, cy, cz, ci, pi, ri, has_f, fi, skin, id, pos, posf, pair);
     } else {
-      for_each_list_contact<T>(G, nb, i, cx, cy, cz, ci, pi, ri, has_f, fi, cell, pos, posf, pair);
+      bool walked = false;
+      if constexpr (sizeof(T) == 4)
+        if (has_f) {
+          for_each_list_hit(G, nb, i, cx, cy, cz, pi, ri, fi, cell, pos, posf, vel, &s_list[0][threadIdx.x],
+                            kSubstepAdjThreads, kAdjHits, pair_of);
+          walked = true;
+        }
+      if (!walked) for_each_list_contact<T>(G, nb, i, cx, cy, cz, ci, pi, ri, has_f, fi, cell, pos, posf, pair);
     }
     if (P.walls)
       gm += add_walls_adj(G, P, pi, ri, mi, vi, cx, cy, cz, l0, l1, l2, gx[0], gx[1], gx[2], gv[0], gv[1], gv[2]);
