@@ -11,6 +11,7 @@
 #include "gic_contact.cuh"
 #include "gic_grid.cuh"
 #include "gic_integrate.cuh"
+#include "gic_sort.cuh"
 #include "gic_tile.cuh"
 
 namespace gic {
@@ -116,6 +117,25 @@ static __device__ __noinline__ void step_build(const DGrid& G, const DParams<T>&
   __syncthreads();  // the shared memory is the tile's from here on
 }
 
+// The moisture ratio of every granule of the state that a gic_step call steps, for
+// the capillary walk: from each of its ~11 partners a granule otherwise
+// interpolates the partner's fluid fraction again (8 gathers and ~130
+// instructions each).  The same values; 300,000 wet granules: 92 -> 79 us per call
+// that keeps its lists, this kernel's 5 included.  In the sort's second key and
+// index lists, which nothing uses after the sort.
+template <typename T>
+__global__ void __launch_bounds__(256) k_moisture(const __grid_constant__ DGrid G,
+                                                  const __grid_constant__ DParams<T> P, int64_t n,
+                                                  const __grid_constant__ StateIn<T> state,
+                                                  const __grid_constant__ StateIn<T> sorted, const uint32_t* flags,
+                                                  const T* __restrict__ af, T* __restrict__ sr) {
+  const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
+  if (i >= n) return;
+  const bool resorted = flags[kNbSorted] != 0u;  // as k_substep
+  sr[i] = moisture_ratio_at(G, P, af, resorted ? sorted.cell[i] : state.cell[i],
+                            resorted ? sorted.pos[i] : state.pos[i], (T*)nullptr);
+}
+
 // kMode: kGeneral is gic_substep's kernel, which reads from the list flags
 // whether it rebuilds; kStep and kStepCap are gic_step's, without and with the
 // capillary force: in a call that rebuilds they read `sorted` and build its rows
@@ -132,7 +152,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
               const __grid_constant__ Fields<T> Fd, int32_t* __restrict__ cell_out, pos_t<T>* __restrict__ pos_out,
               vec_t<T>* __restrict__ vel_out, int32_t* __restrict__ id_out, float4* __restrict__ posf_out,
               vec_t<T>* __restrict__ fex_out, double* __restrict__ alpha, T* __restrict__ Fs_u,
-              T* __restrict__ Fs_v, T* __restrict__ Fs_w, double* __restrict__ sums, uint32_t* status) {
+              T* __restrict__ Fs_v, T* __restrict__ Fs_w, double* __restrict__ sums, uint32_t* status,
+              const T* moisture) {
   // after gic_step's sort kernel, whose launch may overlap it (see substep_launch):
   // returns when that kernel is complete
   if constexpr (kMode != kGeneral) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -207,13 +228,18 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
         F1 = Fc.y;
         F2 = Fc.z;
       } else if (kMode == kStepCap || (kMode == kGeneral && P.cap)) {  // with the capillary bridges (Sec. 5.4): contacts and bridge candidates
-        const T sri = moisture_ratio_at(G, P, Fd.af, ci, pi, (T*)nullptr);
+        auto ratio = [&](int64_t j, int32_t cj, const pos_t<T>& pj) {  // kStepCap: k_moisture's
+          if constexpr (kMode == kStepCap)
+            return __ldg(&moisture[j]);
+          else
+            return moisture_ratio_at(G, P, Fd.af, cj, pj, (T*)nullptr);
+        };
+        const T sri = ratio(i, ci, pi);
         auto near = [&](int64_t j, int32_t cj, const pos_t<T>& pj, const PairGeom<T>& g) {
           if (g.overlap > T(0))
             add_force(P, g, vi, ldg(&vel[j]), mi, radius_of(pj), F0, F1, F2, coincident);
           else
-            add_bridge(P, g, ri, radius_of(pj), sri, moisture_ratio_at(G, P, Fd.af, cj, pj, (T*)nullptr), F0, F1,
-                       F2);
+            add_bridge(P, g, ri, radius_of(pj), sri, ratio(j, cj, pj), F0, F1, F2);
         };
         if (rebuild)
           verlet_build_row_near<T>(G, P, nb, table, n, i, cx, cy, cz, ci, pi, ri, skin, id, pos, near);
@@ -517,7 +543,7 @@ static int substep_launch(const DGrid& G, const GicParams* params, const GicGran
                           const void* cell_table, const GicNeighbors* nb, const NbDev& d, const void* u, const void* v,
                           const void* w, const void* p, const void* alpha_f, GicGranules* next, void* f_ex,
                           double* alpha_s, void* Fs_u, void* Fs_v, void* Fs_w, double* sums2, cudaStream_t stream,
-                          void* scratch = nullptr) {
+                          void* scratch = nullptr, void* moisture = nullptr) {
   int rc;
   const int64_t ncell = (int64_t)G.nx * G.ny * G.nz;
   if (alpha_s && (rc = alpha_begin(alpha_s, ncell, sums2, stream, scratch))) return rc;
@@ -529,6 +555,11 @@ static int substep_launch(const DGrid& G, const GicParams* params, const GicGran
       if (smem > 48 * 1024 &&
           cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return set_error(GIC_ERR_CUDA, "substep: %zu bytes of shared memory refused", smem);
+      if (sorted && P.cap) {
+        k_moisture<T><<<grid_blocks(s->n, 256), 256, 0, stream>>>(G, P, s->n, state_in<T>(s), state_in<T>(sorted),
+                                                                  d.flags, (const T*)alpha_f, (T*)moisture);
+        count_launches(1);
+      }
       // In a gic_step call the kernel directly follows the sort kernel, which returns
       // at once unless the call rebuilds: it may be launched while that one runs,
       // and waits for it itself: 2 us of every call (29.0 -> 27.5 us on 8,000 FP64
@@ -551,7 +582,7 @@ static int substep_launch(const DGrid& G, const GicParams* params, const GicGran
           &cfg, kern, G, P, s->n, state_in<T>(s), state_in<T>(sorted ? sorted : s), d, (const uint4*)cell_table,
           (T)nb->skin, fields<T>(u, v, w, p, alpha_f), next->cell, (pos_t<T>*)next->pos, (vec_t<T>*)next->vel,
           next->id, sizeof(T) == 4 ? (float4*)next->posf : (float4*)nullptr, (vec_t<T>*)f_ex, alpha_s, (T*)Fs_u,
-          (T*)Fs_v, (T*)Fs_w, sums2, status_word());
+          (T*)Fs_v, (T*)Fs_w, sums2, status_word(), (const T*)moisture);
       if (e != cudaSuccess) return set_error(GIC_ERR_CUDA, "substep: launch: %s", cudaGetErrorString(e));
       return GIC_OK;
     };
@@ -666,7 +697,7 @@ extern "C" int gic_step(const GicGrid* grid, const GicParams* params, const GicG
   const cudaStream_t st = (cudaStream_t)stream;
   if ((rc = launch_step_sort(G, state, sorted, perm, cell_table, ws, d.flags, st))) return rc;
   if ((rc = substep_launch(G, params, state, sorted, cell_table, nb, d, u, v, w, p, alpha_f, next, nullptr, alpha_s,
-                           Fs_u, Fs_v, Fs_w, sums2, st, ws)))
+                           Fs_u, Fs_v, Fs_w, sums2, st, ws, (char*)ws + sort_layout(G, state->n).off_keys_b)))
     return rc;
   GIC_CHECK_LAUNCH("gic_step");
   return GIC_OK;
