@@ -564,7 +564,7 @@ struct BoxSplit {
 };
 
 // CTA-wide (every thread calls it): the box, the staged fields and the zeroed
-// accumulators.
+// accumulators (do_a: also alpha_s's).
 __device__ __forceinline__ SubBox sub_tile_begin(SubTile& sh, const DGrid& G, const Fields<float>& Fd, bool valid,
                                                  int32_t c, bool do_a, bool do_f) {
   const SubBox B = sub_box<kSubThreads>(sh.wlo, sh.whi, G, valid, c, kSubTile);
@@ -861,6 +861,13 @@ __device__ __forceinline__ void spread_deposit(SubTile& sh, const SubBox& B, con
   for (int comp = 0; comp < 3; ++comp)
     sub_add_face(sh.f[comp], B, G, (e >> (10 * comp)) & 1023, comp == 0 ? wf[0] : wc[0], comp == 1 ? wf[1] : wc[1],
                  comp == 2 ? wf[2] : wc[2], s[(7 + comp) * kSpreadStride] * inv_unit);
+}
+
+// CTA-wide: alpha_s's accumulators zeroed after the contact walk used their words.
+__device__ __forceinline__ void sub_zero_alpha(SubTile& sh, const SubBox& B) {
+  __syncthreads();
+  for (int e = threadIdx.x; e < B.vol; e += kSubThreads) sh.a[0][e] = sh.a[1][e] = sh.a[2][e] = 0u;
+  __syncthreads();
 }
 
 // alpha_s deposits of one granule at its new position: into the tile when

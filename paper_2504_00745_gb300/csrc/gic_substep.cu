@@ -190,10 +190,13 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
       prefetch_l2(reinterpret_cast<const pos_t<T>*>(nb.ref_pos) + sl);
     }
   }
+  // the candidates' list of the contact walk: the words in which this thread parks
+  // its stencils afterwards, or alpha_s is accumulated
+  constexpr bool kHitList = sizeof(T) == 4 && kMode == kStep;
   // the CTA's tile: the fields staged for G2P, and (FP32) F_s / alpha_s accumulators
   SubBox B;
   if constexpr (sizeof(T) == 4)
-    B = sub_tile_begin(sh, G, Fd, valid, ci, do_a, do_f);
+    B = sub_tile_begin(sh, G, Fd, valid, ci, do_a && !kHitList, do_f);
   else
     B = sub_tile64_begin<NT>(sh, G, Fd, valid, ci);
 
@@ -203,9 +206,6 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
   const bool spread = sizeof(T) == 4 && do_f && !do_a && B.tile;  // uniform over the CTA
   if constexpr (sizeof(T) == 4)
     if (spread && !valid) spread_put_stencil(sh, false, SubStencil{});
-  // the candidates' list of the contact walk: the words in which this thread parks
-  // its stencils afterwards
-  constexpr bool kHitList = sizeof(T) == 4 && kMode == kStep && kNoAlpha;
   if (valid) {
     pi = pos[i];
     vi = vel[i];
@@ -334,6 +334,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
     }
     float* Fs[3] = {Fs_u, Fs_v, Fs_w};
     unsigned long long S = 0;
+    if (kHitList && do_a) sub_zero_alpha(sh, B);
     if (valid && do_a) {
       int ia[3];
       long long va[8];

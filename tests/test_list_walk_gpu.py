@@ -1,7 +1,10 @@
-"""The contact walk over candidate lists (gic_step without alpha_s, the substep's
-adjoint) against the plain walk of the rows: rows of no partner, of fewer and of
-more than a list holds, and partial warps.  The partners and their order are the
-same, so positions and velocities are the same bits."""
+"""The contact walk over candidate lists (gic_step, with and without alpha_s) against
+the plain walk of the rows (a state without its float position copies): rows of
+no partner, of fewer and of more than a list holds, and partial warps.  The
+partners and their order are the same, so positions and velocities are the same
+bits; alpha_s, accumulated where the lists were, is the separate entry point's."""
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -30,14 +33,18 @@ def test_candidate_lists_give_the_rows_own_forces(name):
     if name == "long_rows":
         assert int(sim.nb.count.max()) > 10  # entries of the substep's list
     out = []
-    for alpha in (None, sim.alpha_s):  # the lists; the rows
+    alpha_s = torch.zeros_like(sim.alpha_s)
+    for alpha, st in ((None, sim.A), (sim.alpha_s, sim.A), (None, dataclasses.replace(sim.A, posf=None))):
         for dst, src in zip((sim.A.cell, sim.A.pos, sim.A.vel), before):
             assert torch.equal(dst, src)
-        gic.gic_step(sim.grid, sim.params, sim.A, sim.A2, sim.B, sim.perm, sim.table, sim.ws, sim.nb, F.u, F.v, F.w,
+        gic.gic_step(sim.grid, sim.params, st, sim.A2, sim.B, sim.perm, sim.table, sim.ws, sim.nb, F.u, F.v, F.w,
                      F.p, F.alpha_f, alpha, (None, None, None), None)
         torch.cuda.synchronize()
         out.append([t.cpu().numpy() for t in (sim.A2.cell, sim.A2.pos, sim.A2.vel)])
         sim.nb.flags[5] = 0  # this call's request is not the next one's
     assert gic.gic_check_status() == 0 and sim.nb.builds() == 1
-    for a, b in zip(*out):
-        assert np.array_equal(a, b)
+    for a, b, c in zip(*out):
+        assert np.array_equal(a, b) and np.array_equal(a, c)
+    gic.gic_p2g(sim.grid, sim.params, sim.A, sim.A2, sim.f_ex, alpha_s)
+    torch.cuda.synchronize()
+    assert torch.equal(alpha_s, sim.alpha_s)
