@@ -92,7 +92,8 @@ enum {
   GIC_STATUS_FAST = 32u,         /* a granule moved more than one contact cell in a substep */
   GIC_STATUS_DEBUG_INDEX = 64u,  /* a library built with GIC_DEBUG found an index out of its array; the access
                                     was skipped (release builds never set it) */
-  GIC_STATUS_STALL = 128u        /* a wait inside a kernel ran out of its limit; the call's results are not valid */
+  GIC_STATUS_STALL = 128u        /* a wait inside a gic_step's sort ran out of its limit: that call and every later
+                                    gic_step on its lists made no step (see gic_step) */
 };
 
 typedef struct GicGrid {
@@ -246,7 +247,7 @@ typedef struct GicNeighbors {
   uint32_t* flags;   /* [8]: [0] rebuild in this call, [1] bit 0 rebuild requested, bit 1 a list overflowed at the
                       * last build, [2] CTA counter, [3] overflow during a build, [4] builds performed, [5] a
                       * granule written by the last substep kernel is beyond skin / 2 (read by gic_step),
-                      * [6] arrivals at the sort's grid barriers, [7] the sort of this gic_step is done */
+                      * [6] arrivals in the sort of a gic_step, [7] 1: that sort is done, 2: it stalled */
 } GicNeighbors;
 
 int gic_contact_verlet(const GicGrid* grid, const GicParams* params, const GicGranules* sorted,
@@ -298,6 +299,11 @@ int gic_substep(const GicGrid* grid, const GicParams* params, const GicGranules*
  *   returns at once otherwise, and the substep kernel, which then builds the
  *   rows of `sorted` and reads it, or reads `state`.  Nothing is kept between
  *   calls.
+ *   The sort's waits are limited (some seconds).  If one runs out, the status
+ *   gets GIC_STATUS_STALL, and that call and every later one on the same lists,
+ *   until gic_neighbors_reset, raise it again and make no step: `next` is a copy
+ *   of `state`, F_s and the lists stay as they were, alpha_s and sums2 come out 0
+ *   (`sorted`, perm and the cell table are incomplete).
  *   Arguments as for gic_sort and gic_substep (state, next and sorted must
  *   carry ids and share no array); errors as for those calls.  With sums2
  *   the first 32 bytes of ws also hold the exact alpha_s totals while the
@@ -542,6 +548,14 @@ int gic_contact_pairs(const GicGrid* grid, const GicGranules* sorted, const void
  * stream; clear it if clear != 0.  The wait polls with a deadline of
  * timeout_ms (<= 0: 60 s) and returns GIC_ERR_TIMEOUT if it passes. */
 int gic_check_status(uint32_t* flags, int32_t clear, int32_t timeout_ms, gic_stream_t stream);
+
+/* The sort of the next gic_step call alone: sorts `state` into `sorted` if the
+ * lists ask for a rebuild (which the next gic_step does again), with a limit of
+ * `polls` looks per wait (< 0: the library's).  It exists to see what a wait that
+ * runs out leaves behind: with polls = 0 the first one does.  Errors as for
+ * gic_step. */
+int gic_step_sort(const GicGrid* grid, const GicGranules* state, GicGranules* sorted, int32_t* perm, void* cell_table,
+                  void* ws, size_t ws_bytes, const GicNeighbors* nb, int32_t polls, gic_stream_t stream);
 
 /* Text of the last host-side error on this thread. */
 const char* gic_last_error(void);

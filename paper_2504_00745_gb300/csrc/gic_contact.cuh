@@ -361,11 +361,13 @@ __device__ __forceinline__ void for_each_contact(const DGrid& G, const uint4* __
 // every call); kNbCounter -- CTAs done; kNbOverflow -- overflow during this
 // build; kNbBuilds -- builds so far; kNbNext -- a granule written by a
 // k_substep is beyond skin / 2 of its reference (gic_step's next call
-// rebuilds; gic_step consumes the word); kNbSorted -- this gic_step call sorted,
+// rebuilds; gic_step consumes the word); kNbSorted -- 1: this gic_step call sorted,
 // so its substep kernel takes the sorted state (set when the sort is done,
 // cleared with the call; unlike the request words it does not change
-// while that kernel's CTAs start); kNbBarrier -- arrivals at the grid
-// barriers of gic_step's sort (0 between calls).
+// while that kernel's CTAs start), kNbStalled: a grid barrier of a sort ran out of
+// its limit, and gic_step does nothing on these lists until gic_neighbors_reset;
+// kNbBarrier -- arrivals at the grid barriers and the end of gic_step's sort (0
+// between calls).
 
 enum : int {
   kNbRebuild = 0,
@@ -381,6 +383,10 @@ enum : int {
 // The count of a row that overflowed in gic_step's build: the granule's contact
 // force comes from the 27 cells.
 constexpr int32_t kNbWalked = -1;
+// kNbSorted after a sort whose grid barrier ran out: its results are incomplete
+// and the count of arrivals is off, so neither that call's substep (on a first call
+// the lists hold no rows at all) nor a later sort may run.
+constexpr uint32_t kNbStalled = 2u;
 
 struct NbDev {
   int cap;
@@ -637,9 +643,11 @@ __device__ __forceinline__ bool step_rebuilds(const uint32_t* flags) {
 }
 
 // gic_step's sort (gic_step_sort.cu): if the call rebuilds, `in` is sorted into
-// `out` (perm, cell table as gic_sort; scratch in ws); one launch either way.
+// `out` (perm, cell table as gic_sort; scratch in ws); one launch either way.  polls: how
+// often a CTA looks at a grid barrier before it gives up.
+constexpr int kBarrierPolls = 1 << 23;  // some seconds
 int launch_step_sort(const DGrid& G, const GicGranules* in, const GicGranules* out, int32_t* perm, void* table,
-                     void* ws, uint32_t* flags, cudaStream_t st);
+                     void* ws, uint32_t* flags, int polls, cudaStream_t st);
 
 // The list build of granule i: walks the 27 cells with the pre-test radius
 // r_i + r_j + skin, writes row i (slot = sorted index) and its reference

@@ -20,19 +20,21 @@
 
 namespace gic {
 
-// Grid barrier of a cooperative launch: the CTAs' arrivals counted in *cnt,
-// target = barriers so far x CTAs.  Waits at most kBarrierPolls polls (some
-// seconds); past that the launch cannot be complete, the status word is
-// flagged, and every CTA returns (the others run out in the same way).
-constexpr int kBarrierPolls = 1 << 23;
-__device__ __forceinline__ bool grid_barrier(uint32_t* cnt, uint32_t target, uint32_t* status) {
+// Grid barrier of a cooperative launch: the CTAs' arrivals counted in a word of
+// the lists' flags, target = barriers so far x CTAs.  Waits at most `polls` looks;
+// past that the launch cannot be complete: the CTA flags the status word, marks
+// the lists as stalled and returns.  The others run out in the same way: one that
+// arrives late may still pass this barrier (everyone arrived at it, so what it reads
+// is complete), but not the next.
+__device__ __forceinline__ bool grid_barrier(uint32_t* flags, uint32_t target, int polls, uint32_t* status) {
   __shared__ int s_ok;
+  uint32_t* cnt = &flags[kNbBarrier];
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(cnt, 1u);
     int ok = 0;
-    for (int k = 0; k < kBarrierPolls; ++k) {
+    for (int k = 0; k < polls; ++k) {
       uint32_t v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
       if (v >= target) {
@@ -42,7 +44,10 @@ __device__ __forceinline__ bool grid_barrier(uint32_t* cnt, uint32_t target, uin
       __nanosleep(40);
     }
     __threadfence();
-    if (!ok) raise_status(status, GIC_STATUS_STALL);
+    if (!ok) {
+      flags[kNbSorted] = kNbStalled;
+      raise_status(status, GIC_STATUS_STALL);
+    }
     s_ok = ok;
   }
   __syncthreads();
@@ -58,7 +63,7 @@ struct StepSortArgs {
   int64_t n;
   ScatterState S;
   uint32_t *keys_a, *vals_a, *keys_b, *vals_b, *counts, *totals;
-  int tiles, passes;
+  int tiles, passes, polls;
   uint4* table;
   uint32_t* flags;  // of the lists
   uint32_t* status;
@@ -68,12 +73,14 @@ template <typename T>
 __global__ void __launch_bounds__(kStepSortThreads, kStepSortCtas)
     k_step_sort(const __grid_constant__ StepSortArgs<T> A) {
   __shared__ SortShared<kStepSortThreads> sh;
-  if (!step_rebuilds(A.flags)) {  // uniform: the words change only in the substep kernels
+  const bool stalled = A.flags[kNbSorted] == kNbStalled;  // by an earlier call
+  if (stalled || !step_rebuilds(A.flags)) {  // uniform: the words change only in the substep kernels
+    if (stalled && blockIdx.x == 0 && threadIdx.x == 0) raise_status(A.status, GIC_STATUS_STALL);
     asm volatile("griddepcontrol.launch_dependents;");  // the substep kernel may start
     return;
   }
   uint32_t arrived = 0;
-  auto barrier = [&]() { return grid_barrier(&A.flags[kNbBarrier], arrived += gridDim.x, A.status); };
+  auto barrier = [&]() { return grid_barrier(A.flags, arrived += gridDim.x, A.polls, A.status); };
   // the radix passes, ping-ponging between the two key / value buffers
   for (int p = 0; p < A.passes; ++p) {
     const bool first = p == 0, last = p == A.passes - 1;
@@ -93,12 +100,11 @@ __global__ void __launch_bounds__(kStepSortThreads, kStepSortCtas)
   for (int64_t k = blockIdx.x * (int64_t)kStepSortThreads + threadIdx.x; k < A.n;
        k += (int64_t)gridDim.x * kStepSortThreads)
     sort_gather<T>(A.G, A.n, k, keys, A.S, A.table, A.status);
-  // past the last barrier: the last CTA clears the count of arrivals and tells the
-  // substep kernel
-  if (threadIdx.x == 0 && atomicAdd(&A.flags[kNbCounter], 1u) == gridDim.x - 1) {
+  // past the last barrier: the last CTA (of all: one that gave up there does not
+  // arrive here) clears the count of arrivals and tells the substep kernel
+  if (threadIdx.x == 0 && atomicAdd(&A.flags[kNbBarrier], 1u) == arrived + gridDim.x - 1) {
     A.flags[kNbBarrier] = 0u;
     A.flags[kNbSorted] = 1u;
-    A.flags[kNbCounter] = 0u;
   }
 }
 
@@ -122,7 +128,7 @@ static int resident_ctas() {
 
 template <typename T>
 static int launch(const DGrid& G, const GicGranules* in, const GicGranules* out, int32_t* perm, void* table, char* ws,
-                  uint32_t* flags, cudaStream_t st) {
+                  uint32_t* flags, int polls, cudaStream_t st) {
   const SortLayout L = sort_layout(G, in->n);
   StepSortArgs<T> A{G,
                     in->n,
@@ -136,6 +142,7 @@ static int launch(const DGrid& G, const GicGranules* in, const GicGranules* out,
                     (uint32_t*)(ws + L.off_totals),
                     L.tiles,
                     L.passes,
+                    polls,
                     (uint4*)table,
                     flags,
                     status_word()};
@@ -151,9 +158,9 @@ static int launch(const DGrid& G, const GicGranules* in, const GicGranules* out,
 }
 
 int launch_step_sort(const DGrid& G, const GicGranules* in, const GicGranules* out, int32_t* perm, void* table,
-                     void* ws, uint32_t* flags, cudaStream_t st) {
-  return in->precision == GIC_FP32 ? launch<float>(G, in, out, perm, table, (char*)ws, flags, st)
-                                   : launch<double>(G, in, out, perm, table, (char*)ws, flags, st);
+                     void* ws, uint32_t* flags, int polls, cudaStream_t st) {
+  return in->precision == GIC_FP32 ? launch<float>(G, in, out, perm, table, (char*)ws, flags, polls, st)
+                                   : launch<double>(G, in, out, perm, table, (char*)ws, flags, polls, st);
 }
 
 }  // namespace gic

@@ -130,10 +130,28 @@ __global__ void __launch_bounds__(256) k_moisture(const __grid_constant__ DGrid 
                                                   const __grid_constant__ StateIn<T> sorted, const uint32_t* flags,
                                                   const T* __restrict__ af, T* __restrict__ sr) {
   const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || flags[kNbSorted] == kNbStalled) return;
   const bool resorted = flags[kNbSorted] != 0u;  // as k_substep
   sr[i] = moisture_ratio_at(G, P, af, resorted ? sorted.cell[i] : state.cell[i],
                             resorted ? sorted.pos[i] : state.pos[i], (T*)nullptr);
+}
+
+// The substep of a call whose sort stalled: `next` becomes a copy of `state`, so that
+// what the caller does with it (ids are indices in gic_unpack) stays in bounds.  (In line:
+// out of line, nvcc 13.0's FP64 kernel with bridges stored x alone of each record.)
+template <typename T, int NT>
+static __device__ __forceinline__ void step_stalled(int64_t n, const StateIn<T>& S, int32_t* cell_out, pos_t<T>* pos_out,
+                                                 vec_t<T>* vel_out, int32_t* id_out, float4* posf_out) {
+  const int64_t i = blockIdx.x * (int64_t)NT + threadIdx.x;
+  if (i >= n) return;
+  const int32_t c = S.cell[i];
+  const pos_t<T> p = S.pos[i];
+  cell_out[i] = c;
+  pos_out[i] = p;
+  vel_out[i] = S.vel[i];
+  if (id_out && S.id) id_out[i] = S.id[i];
+  if constexpr (sizeof(T) == 4)
+    if (posf_out) posf_out[i] = posf_of(c, p);
 }
 
 // kMode: kGeneral is gic_substep's kernel, which reads from the list flags
@@ -158,7 +176,12 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
   // returns when that kernel is complete
   if constexpr (kMode != kGeneral) asm volatile("griddepcontrol.wait;" ::: "memory");
   // uniform over the launch
-  const bool resorted = kMode != kGeneral && nb.flags[kNbSorted] != 0u;
+  const uint32_t sort_done = kMode != kGeneral ? nb.flags[kNbSorted] : 0u;
+  if (kMode != kGeneral && sort_done == kNbStalled) {  // no sorted state, perhaps no rows
+    step_stalled<T, NT>(n, state, cell_out, pos_out, vel_out, id_out, posf_out);
+    return;
+  }
+  const bool resorted = sort_done != 0u;
   const bool rebuild = kMode == kGeneral && (nb.flags[kNbRebuild] | nb.flags[kNbSticky]) != 0u;
   const StateIn<T> S = resorted ? sorted : state;
   const int32_t* __restrict__ cell = S.cell;
@@ -657,6 +680,16 @@ static bool share_array(const GicGranules* a, const GicGranules* b) {
          (a->posf && a->posf == b->posf);
 }
 
+static int check_sort_workspace(const GicGrid* grid, const GicGranules* s, const void* ws, size_t ws_bytes,
+                                const char* what) {
+  size_t need = 0;
+  if (int rc = gic_workspace_size(grid, s->n, s->precision, &need)) return rc;
+  if (!ws || ws_bytes < need)
+    return set_error(GIC_ERR_WORKSPACE, "%s: workspace of %zu bytes needed, %zu given", what, need, ws_bytes);
+  if ((uintptr_t)ws % 256) return set_error(GIC_ERR_ALIGN, "%s: workspace must be 256-byte aligned", what);
+  return GIC_OK;
+}
+
 extern "C" int gic_step(const GicGrid* grid, const GicParams* params, const GicGranules* state, GicGranules* next,
                         GicGranules* sorted, int32_t* perm, void* cell_table, void* ws, size_t ws_bytes,
                         const GicNeighbors* nb, const void* u, const void* v, const void* w, const void* p,
@@ -688,19 +721,39 @@ extern "C" int gic_step(const GicGrid* grid, const GicParams* params, const GicG
   NbDev d;
   if ((rc = verlet_view(G, state, cell_table, nb, "gic_step", true, &d))) return rc;
   if (state->n == 0) return GIC_OK;
-  {  // the sort's workspace
-    size_t need = 0;
-    if ((rc = gic_workspace_size(grid, state->n, state->precision, &need))) return rc;
-    if (!ws || ws_bytes < need)
-      return set_error(GIC_ERR_WORKSPACE, "gic_step: workspace of %zu bytes needed, %zu given", need, ws_bytes);
-    if ((uintptr_t)ws % 256) return set_error(GIC_ERR_ALIGN, "gic_step: workspace must be 256-byte aligned");
-  }
+  if ((rc = check_sort_workspace(grid, state, ws, ws_bytes, "gic_step"))) return rc;
   const cudaStream_t st = (cudaStream_t)stream;
-  if ((rc = launch_step_sort(G, state, sorted, perm, cell_table, ws, d.flags, st))) return rc;
+  if ((rc = launch_step_sort(G, state, sorted, perm, cell_table, ws, d.flags, kBarrierPolls, st))) return rc;
   if ((rc = substep_launch(G, params, state, sorted, cell_table, nb, d, u, v, w, p, alpha_f, next, nullptr, alpha_s,
                            Fs_u, Fs_v, Fs_w, sums2, st, ws, (char*)ws + sort_layout(G, state->n).off_keys_b)))
     return rc;
   GIC_CHECK_LAUNCH("gic_step");
+  return GIC_OK;
+}
+
+extern "C" int gic_step_sort(const GicGrid* grid, const GicGranules* state, GicGranules* sorted, int32_t* perm,
+                             void* cell_table, void* ws, size_t ws_bytes, const GicNeighbors* nb, int32_t polls,
+                             gic_stream_t stream) {
+  GIC_RANGE("gic_step_sort");
+  DGrid G;
+  int rc = make_grid(grid, &G);
+  if (rc) return rc;
+  if ((rc = check_granules(state, "gic_step_sort state", true))) return rc;
+  if ((rc = check_granules(sorted, "gic_step_sort sorted", true))) return rc;
+  if (sorted->n != state->n || sorted->precision != state->precision)
+    return set_error(GIC_ERR_INVALID, "gic_step_sort: state/sorted size or precision differ");
+  if (share_array(state, sorted))
+    return set_error(GIC_ERR_INVALID, "gic_step_sort: state and sorted must not share arrays");
+  if (state->n > 0 && !perm) return set_error(GIC_ERR_INVALID, "gic_step_sort: perm is NULL");
+  if (!nb) return set_error(GIC_ERR_INVALID, "gic_step_sort: neighbours struct is NULL");
+  NbDev d;
+  if ((rc = verlet_view(G, state, cell_table, nb, "gic_step_sort", true, &d))) return rc;
+  if (state->n == 0) return GIC_OK;
+  if ((rc = check_sort_workspace(grid, state, ws, ws_bytes, "gic_step_sort"))) return rc;
+  if ((rc = launch_step_sort(G, state, sorted, perm, cell_table, ws, d.flags, polls < 0 ? kBarrierPolls : polls,
+                             (cudaStream_t)stream)))
+    return rc;
+  GIC_CHECK_LAUNCH("gic_step_sort");
   return GIC_OK;
 }
 

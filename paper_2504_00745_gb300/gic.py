@@ -92,6 +92,7 @@ _SIGS = {
     "gic_contact_verlet_adj": [_P] * 11,
     "gic_substep_adj": [_P] * 19,
     "gic_step": [_P, _P, _P, _P, _P, _P, _P, _P, C.c_size_t, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P],
+    "gic_step_sort": [_P, _P, _P, _P, _P, _P, C.c_size_t, _P, C.c_int32, _P],
     "gic_project_workspace_size": [_P, _P],
     "gic_project": [_P] * 16 + [C.c_size_t, _P, _P],
 }
@@ -350,6 +351,14 @@ def gic_step(grid: GicGrid, params: GicParams, state: State, next_: State, sorte
                           _ptr(cell_table), _ptr(ws), ws.numel() * ws.element_size(), C.byref(b), _ptr(u), _ptr(v),
                           _ptr(w), _ptr(p), _ptr(alpha_f), _ptr(alpha_s), _ptr(Fs[0]), _ptr(Fs[1]), _ptr(Fs[2]),
                           _ptr(sums2), _stream(stream)), "gic_step")
+
+
+def gic_step_sort(grid: GicGrid, state: State, sorted_: State, perm, cell_table, ws, nb: Neighbors, polls: int = -1,
+                  stream=None):
+    """The sort of the next gic_step alone, its waits limited to `polls` looks."""
+    a, s, b = state.struct(), sorted_.struct(), nb.struct()
+    _check(lib().gic_step_sort(C.byref(grid), C.byref(a), C.byref(s), _ptr(perm), _ptr(cell_table), _ptr(ws),
+                               ws.numel() * ws.element_size(), C.byref(b), polls, _stream(stream)), "gic_step_sort")
 
 
 def gic_neighbors_reset(nb: Neighbors, stream=None):
