@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kP2GThreads, 2) k_p2g_f32(DGrid G, DParams<flo
       ext.add_force(fc);
     }
   }
-  const P2GBox B = p2g_box(sh, ext, do_a, do_f);
+  const P2GBox B = p2g_box(sh, G, ext, do_a, do_f);
   float* Fs[3] = {Fs_u, Fs_v, Fs_w};
   unsigned long long S = 0;
   if (valid && do_a) {

@@ -300,9 +300,10 @@ __device__ __forceinline__ void p2g_box_init(P2GShared& sh) {
   if (threadIdx.x == 0) sh.M = 0u;
 }
 
-// CTA-wide: reduce the extents, decide the tile and zero it.  Every thread
-// of the CTA must call it (it synchronises the CTA).
-__device__ __forceinline__ P2GBox p2g_box(P2GShared& sh, const P2GExtent& ext, bool do_a, bool do_f) {
+// CTA-wide: reduce the extents, decide the tile (none with a cell beyond the grid,
+// as in sub_box) and zero it.  Every thread of the CTA must call it (it
+// synchronises the CTA).
+__device__ __forceinline__ P2GBox p2g_box(P2GShared& sh, const DGrid& G, const P2GExtent& ext, bool do_a, bool do_f) {
   __syncthreads();
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -326,7 +327,8 @@ __device__ __forceinline__ P2GBox p2g_box(P2GShared& sh, const P2GExtent& ext, b
   B.b[2] = max(sh.lo[2], 0);
   const int ex = sh.hi[0] - B.b[0] + 1, ey = sh.hi[1] - B.b[1] + 1, ez = sh.hi[2] - B.b[2] + 1;
   // a CTA without granules has lo > hi
-  B.tile = ex > 0 && ey > 0 && ez > 0 && (int64_t)ex * ey * ez <= kP2GTile;
+  B.tile = ex > 0 && ey > 0 && ez > 0 && sh.hi[0] <= G.nx && sh.hi[1] <= G.ny && sh.hi[2] <= G.nz &&
+           (int64_t)ex * ey * ez <= kP2GTile;
   const float Mc = __uint_as_float(sh.M);
   B.ftile = B.tile && do_f && Mc >= 1e-30f && Mc <= 3.0e38f;
   const int bits = 30 - (32 - __clz((int)blockDim.x - 1));  // 22 for 256 threads, 21 for 512
@@ -486,7 +488,8 @@ struct SubBox {
 // CTA-wide (every thread calls it; one barrier): the box of samples m - 1 .. m + 1
 // per axis around the MAC cells of the CTA's granules, used as a tile when it
 // holds at most `most` of them.  valid: this thread has a granule in contact
-// cell c.
+// cell c.  A CTA with a granule in a cell beyond the grid (GIC_STATUS_BAD_CELL) takes
+// no tile: the stencils are clamped into the grid, which that box is not in.
 template <int NT>
 __device__ __forceinline__ SubBox sub_box(int (&wlo)[3][kSubWarps], int (&whi)[3][kSubWarps], const DGrid& G,
                                           bool valid, int32_t c, int most) {
@@ -519,7 +522,7 @@ __device__ __forceinline__ SubBox sub_box(int (&wlo)[3][kSubWarps], int (&whi)[3
   B.ex = any ? hi[0] + 1 - B.b[0] + 1 : 1;
   B.ey = any ? hi[1] + 1 - B.b[1] + 1 : 1;
   B.ez = any ? hi[2] + 1 - B.b[2] + 1 : 1;
-  B.tile = any && (int64_t)B.ex * B.ey * B.ez <= most;
+  B.tile = any && hi[0] < G.nx && hi[1] < G.ny && hi[2] < G.nz && (int64_t)B.ex * B.ey * B.ez <= most;
   B.sy = B.ex;
   B.sz = B.ex * B.ey;
   B.vol = B.tile ? B.ex * B.ey * B.ez : 0;

@@ -109,7 +109,9 @@ __device__ __forceinline__ TileBox tile_stage(TileShared<NT>& sh, const DGrid& G
   B.by = min(hi[1] + 1, G.nc[1] - 1) - B.by0 + 1;
   B.bz = min(hi[2] + 1, G.nc[2] - 1) - B.bz0 + 1;
   const int ncell = B.bx * B.by * B.bz;
-  B.staged = hi[0] >= 0 && ncell <= kCells;  // a CTA without granules stages nothing
+  // a CTA without granules stages nothing, nor does one with a granule in a cell beyond
+  // the grid (GIC_STATUS_BAD_CELL), whose own cell and slot the box does not hold
+  B.staged = hi[0] >= 0 && hi[0] < G.nc[0] && hi[1] < G.nc[1] && hi[2] < G.nc[2] && ncell <= kCells;
   B.start = reinterpret_cast<uint32_t*>(sh.buf);
   B.off = nullptr;
   B.pf = nullptr;
