@@ -58,8 +58,9 @@ __device__ __forceinline__ void advance_axis(const DGrid& G, double dt, double v
                                              double& o_out, int& c_out, uint32_t& flags) {
   double x = fma(dt, v, o);
   // still in the cell: 0 <= x < h_c, compared as integers (a negative or NaN x is
-  // above every such value), without the floor and its conversions
-  if ((unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(G.hc)) {
+  // above every such value), without the floor and its conversions; a cell beyond the
+  // grid is clamped below
+  if (c < nc && (unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(G.hc)) {
     o_out = x;
     c_out = c;
     return;

@@ -71,3 +71,22 @@ def test_lists_built_with_cells_beyond_the_grid():
     torch.cuda.synchronize()
     assert torch.equal(sim.nb.count, want)
     assert gic.gic_check_status(clear=True) == gic.STATUS_BAD_CELL
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
+def test_integration_clamps_cells_beyond_the_grid(prec):
+    """A granule at rest in such a cell leaves it for the last cell of the grid,
+    and the status says so."""
+    _, sim = _simulators(prec)
+    nc = sim.grid.nx * sim.grid.k_contact
+    sim.A.vel.zero_()
+    out = gic.State.empty(sim.n, prec)
+    zero = [gic.vec4(sim.n, prec) for _ in range(3)]
+    gic.gic_integrate(sim.grid, sim.params, sim.A, *zero, out, sim.f_ex)
+    torch.cuda.synchronize()
+    assert gic.gic_check_status(clear=True) == gic.STATUS_OUT_OF_DOMAIN
+    cell = [int(out.cell[i]) for i in (7, 900, 1500, 2999)]
+    last = nc - 1
+    assert [c & 1023 for c in cell] == [last, 20, 20, last]
+    assert [c >> 10 & 1023 for c in cell] == [20, last, 20, last]
+    assert [c >> 20 for c in cell] == [20, 20, last, last]
