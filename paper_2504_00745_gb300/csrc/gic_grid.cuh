@@ -601,7 +601,7 @@ __device__ __forceinline__ SubBox sub_tile_begin(SubTile& sh, const DGrid& G, co
 //
 // As the FP32 tile, for G2P alone: the face velocities and face pressure
 // gradients of the box, each with its difference to the next sample along x, so
-// that a granule's six interpolations take 66 FP64 operations instead of 141
+// that a granule's six interpolations take 69 FP64 operations instead of 141
 // and the gradients' differences are formed once per sample.  The values and
 // their order are interp_value's: the same bits as from global memory.
 // (F_s in the tile as fixed-point limbs: 1% faster, and its unit, tied to the CTA's
@@ -654,14 +654,15 @@ __device__ __forceinline__ double sub_g2p64(const SubTile64<NT>& sh, const SubBo
     const int e0 = B.index(S.i0[0], S.i0[1], S.i0[2]);
     uf[comp] = gp[comp] = 0.0;
     if (!GIC_DBG_OK(G.dbg, e0 >= 0 && e0 + 1 + B.sy + B.sz < B.vol)) continue;
+    const LerpX lerp = lerp_x(S.w[0]);
 #pragma unroll
     for (int cc = 0; cc < 2; ++cc)
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
         const int e = e0 + b * B.sy + cc * B.sz;
         const double w = (b ? S.w[1] : 1.0 - S.w[1]) * (cc ? S.w[2] : 1.0 - S.w[2]);
-        uf[comp] = fma(w, fma(S.w[0], sh.d[comp][e], sh.f[comp][e]), uf[comp]);
-        gp[comp] = fma(w, fma(S.w[0], sh.d[3 + comp][e], sh.f[3 + comp][e]), gp[comp]);
+        uf[comp] = fma(w, lerp(sh.f[comp][e + lerp.up], sh.d[comp][e]), uf[comp]);
+        gp[comp] = fma(w, lerp(sh.f[3 + comp][e + lerp.up], sh.d[3 + comp][e]), gp[comp]);
       }
   }
   return coupling_forces<double>(P, radius_of(pi), vi, uf, gp, F, a);

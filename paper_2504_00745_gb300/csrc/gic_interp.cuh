@@ -110,23 +110,39 @@ __device__ __forceinline__ T interp(const Stencil3<T>& S, Load load, T inv_dx, T
   return acc;
 }
 
+// The x-lerp of a row of two samples from the nearer one: f0 + w (f1 - f0) below
+// 1/2, f1 + (w - 1) (f1 - f0) from there on (w - 1 is exact).  A point beyond the last
+// sample (w = 1) takes its value exactly, and the difference's rounding enters with
+// at most 1/2; from f0 alone it entered whole at w = 1 (standard normal samples, w
+// uniform in [0, 1]: rms error 0.51 x 2^-53, the products (1 - w) f0 + w f1 0.42, this
+// 0.39).  up: the sample to start from; the compare is on integers.
+struct LerpX {
+  int up;
+  double w;
+  __device__ __forceinline__ double operator()(double near, double diff) const { return fma(w, diff, near); }
+};
+__device__ __forceinline__ LerpX lerp_x(double w) {
+  const bool up = __double2hiint(w) >= 0x3FE00000;
+  return LerpX{up ? 1 : 0, up ? w - 1.0 : w};
+}
+
 // The value alone.  FP64: an x-lerp per row and the (y, z) products, 16 FP64
-// operations and 6 for the weights instead of 31 (8 products of three weights,
+// operations and 7 for the weights instead of 31 (8 products of three weights,
 // 8 fused multiply-adds): that pipe bounds the FP64 path.
 template <typename T, typename Load>
 __device__ __forceinline__ T interp_value(const Stencil3<T>& S, Load load, T inv_dx) {
   if constexpr (sizeof(T) == 4) {
     return interp<T>(S, load, inv_dx, nullptr);
   } else {
+    const LerpX lerp = lerp_x(S.w[0]);
     T acc = 0;
 #pragma unroll
     for (int c = 0; c < 2; ++c)
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
-        const T f0 = load(S.i0[0], S.i0[1] + b, S.i0[2] + c);
-        const T d = load(S.i0[0] + 1, S.i0[1] + b, S.i0[2] + c) - f0;
+        const T f0 = load(S.i0[0], S.i0[1] + b, S.i0[2] + c), f1 = load(S.i0[0] + 1, S.i0[1] + b, S.i0[2] + c);
         const T w = (b ? S.w[1] : T(1) - S.w[1]) * (c ? S.w[2] : T(1) - S.w[2]);
-        acc = fma(w, fma(S.w[0], d, f0), acc);
+        acc = fma(w, lerp(lerp.up ? f1 : f0, f1 - f0), acc);
       }
     return acc;
   }
