@@ -520,48 +520,65 @@ __device__ __forceinline__ float mg_sweep(const MgLevel& L, unsigned c, unsigned
   return x;
 }
 
-// The passes grid-wide: a CTA takes tiles of 2^lx pairs x (256 >> lx) rows x kc
-// layers, tile blockIdx.x, + gridDim.x, ... (two divisions per tile, none per
-// cell).  f(p, j, k) for every pair (or coarse cell) p < np.
+// The passes grid-wide: a CTA takes tiles of 2^lx pairs x 2^ly rows x 2^lz runs of kc
+// layers (lx + ly + lz = 8: a thread per run), tile blockIdx.x, + gridDim.x, ... (two
+// divisions per tile, none per cell).  f(p, j, k) for every pair (or coarse cell) p < np.
+// kDeep: lz > 0.  A kernel of its own, because the split in three cost the other grids
+// 0.9% of a call at 128^3 (another schedule of the same loop).
 struct MgTiles {
   unsigned np, ny, nz;       // extent
-  unsigned lx, kc;           // tile shape
+  unsigned lx, ly, lz, kc;   // tile shape
   unsigned tx, ty, tiles;    // tiles along x, y; in all
 };
-template <typename F>
+static_assert(kProjThreads == 256, "mg_tiles splits 8 bits");
+template <bool kDeep, typename F>
 __device__ __forceinline__ void mg_tiles(const MgTiles& T, F&& f) {
-  const unsigned px = threadIdx.x & ((1u << T.lx) - 1u), py = threadIdx.x >> T.lx;
+  const unsigned px = threadIdx.x & ((1u << T.lx) - 1u);
+  if constexpr (!kDeep) {
+    const unsigned py = threadIdx.x >> T.lx;
+    for (unsigned t = blockIdx.x; t < T.tiles; t += gridDim.x) {
+      const unsigned txy = T.tx * T.ty, tz = t / txy, r = t - tz * txy, y = r / T.tx, x = r - y * T.tx;
+      const unsigned p = (x << T.lx) + px, j = y * ((unsigned)kProjThreads >> T.lx) + py;
+      if (p >= T.np || j >= T.ny) continue;
+      const unsigned k1 = min((tz + 1) * T.kc, T.nz);
+#pragma unroll 2
+      for (unsigned k = tz * T.kc; k < k1; ++k) f(p, j, k);
+    }
+    return;
+  }
+  const unsigned py = (threadIdx.x >> T.lx) & ((1u << T.ly) - 1u), pz = threadIdx.x >> (T.lx + T.ly);
   for (unsigned t = blockIdx.x; t < T.tiles; t += gridDim.x) {
     const unsigned txy = T.tx * T.ty, tz = t / txy, r = t - tz * txy, y = r / T.tx, x = r - y * T.tx;
-    const unsigned p = (x << T.lx) + px, j = y * ((unsigned)kProjThreads >> T.lx) + py;
+    const unsigned p = (x << T.lx) + px, j = (y << T.ly) + py;
     if (p >= T.np || j >= T.ny) continue;
-    const unsigned k1 = min((tz + 1) * T.kc, T.nz);
+    const unsigned k0 = ((tz << T.lz) + pz) * T.kc, k1 = min(k0 + T.kc, T.nz);
 #pragma unroll 2
-    for (unsigned k = tz * T.kc; k < k1; ++k) f(p, j, k);
+    for (unsigned k = k0; k < k1; ++k) f(p, j, k);
   }
 }
 
-template <bool kAp>
+template <bool kAp, bool kDeep>
 __global__ void __launch_bounds__(kProjThreads, 4) k_mg_down(MgLevel L, MgTiles T, const ProjRed* red) {
   if (stopped(red)) return;
-  mg_tiles(T, [&](unsigned p, unsigned j, unsigned k) { mg_down<kAp>(L, mg_pair(L, p, j, k)); });
+  mg_tiles<kDeep>(T, [&](unsigned p, unsigned j, unsigned k) { mg_down<kAp>(L, mg_pair(L, p, j, k)); });
 }
 
-template <bool kAp>
+template <bool kAp, bool kDeep>
 __global__ void __launch_bounds__(kProjThreads, 4) k_mg_restrict(MgLevel F, MgLevel C, MgTiles T, const ProjRed* red) {
   if (stopped(red)) return;
-  mg_tiles(T, [&](unsigned p, unsigned J, unsigned K) { mg_restrict<kAp>(F, C, p >> 2, p & 3u, J, K); });
+  mg_tiles<kDeep>(T, [&](unsigned p, unsigned J, unsigned K) { mg_restrict<kAp>(F, C, p >> 2, p & 3u, J, K); });
 }
 
-template <bool kAp>
+template <bool kAp, bool kDeep>
 __global__ void __launch_bounds__(kProjThreads, 4) k_mg_up_black(MgLevel L, MgLevel C, MgTiles T, const ProjRed* red) {
   if (stopped(red)) return;
-  mg_tiles(T, [&](unsigned p, unsigned j, unsigned k) { mg_up_black<kAp>(L, C, mg_pair(L, p, j, k)); });
+  mg_tiles<kDeep>(T, [&](unsigned p, unsigned j, unsigned k) { mg_up_black<kAp>(L, C, mg_pair(L, p, j, k)); });
 }
 
+template <bool kDeep>
 __global__ void __launch_bounds__(kProjThreads, 4) k_mg_up_red(MgLevel L, MgTiles T, const ProjRed* red) {
   if (stopped(red)) return;
-  mg_tiles(T, [&](unsigned p, unsigned j, unsigned k) {
+  mg_tiles<kDeep>(T, [&](unsigned p, unsigned j, unsigned k) {
     const MgPair q = mg_pair(L, p, j, k);
     if (q.red) mg_sweep<false>(L, q.row + q.ir, q.ir, j, k);
   });
@@ -569,12 +586,13 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_mg_up_red(MgLevel L, MgTile
 
 // The same on level 0, where x = z = M^-1 r is complete after it, with rho =
 // r . z into red->rz[cur] (b is r): a thread has both cells of its pair at hand.
+template <bool kDeep>
 __global__ void __launch_bounds__(kProjThreads, 4) k_mg_up_red_dot(MgLevel L, MgTiles T, int cur,
                                                                    double* __restrict__ P, ProjRed* red) {
   __shared__ double smem[32];
   if (stopped(red)) return;
   KahanF sum;
-  mg_tiles(T, [&](unsigned p, unsigned j, unsigned k) {
+  mg_tiles<kDeep>(T, [&](unsigned p, unsigned j, unsigned k) {
     const MgPair q = mg_pair(L, p, j, k);
     if (q.red) sum.add(L.b[q.row + q.ir] * mg_sweep<true>(L, q.row + q.ir, q.ir, j, k));
     if (q.black) sum.add(L.b[q.row + q.ib] * L.x[q.row + q.ib]);
@@ -726,6 +744,7 @@ __global__ void __launch_bounds__(kProjThreads) k_cg_dot(int64_t n64, int cur, c
 // iteration), y = A d_new and d_new . y into red->dy.  d_old and d_new are
 // different buffers: neighbours' d_new is formed from their z and d_old.
 // The face weights are formed again from alpha_f' (mg_faces).
+template <bool kDeep>
 __global__ void __launch_bounds__(kProjThreads, 4) k_cg_dir_apply(MgLevel L, MgTiles T, int cur,
                                                                   const float* __restrict__ z,
                                                                   const float* __restrict__ d_old,
@@ -738,7 +757,7 @@ __global__ void __launch_bounds__(kProjThreads, 4) k_cg_dir_apply(MgLevel L, MgT
   KahanF dyk;
   // beta = 0 takes z alone (the old direction is not read into the sum)
   auto dn = [&](unsigned q) { return be != 0.f ? fmaf(be, d_old[q], z[q]) : z[q]; };
-  mg_tiles(T, [&](unsigned i, unsigned j, unsigned k) {
+  mg_tiles<kDeep>(T, [&](unsigned i, unsigned j, unsigned k) {
     const unsigned c = i + (unsigned)L.nx * (j + (unsigned)L.ny * k);
     const MgNear m = mg_near(L, c, i, j, k);
     const MgFaces w = mg_faces<true>(L, m, c, i, j, k);
@@ -1078,21 +1097,34 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
   if (tail_bytes > 48 * 1024 &&
       cudaFuncSetAttribute(k_mg_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMgTailSmem) != cudaSuccess)
     return set_error(GIC_ERR_CUDA, "gic_project: shared memory of the coarse levels refused");
-  // tiles of a pass over np x ny x nz pairs (or cells): wide enough for the rows, and
-  // up to four layers per tile where that still leaves a tile for every CTA
+  // tiles of a pass over np x ny x nz pairs (or cells): wide enough for the rows (up to
+  // a warp), the other lanes over rows and layers so that the fewest fall outside the
+  // grid.  (All of them on rows, a column of 1 x 1 x 20000 cells had one lane of 256 at
+  // work: 10.5 ms a call, now 2.5; 2 x 2 x 65536 13.0 -> 4.5, 4 x 4 x 4096 15.6 -> 10.9,
+  // 300 x 1 x 300 6.9 -> 5.7; 128^3 keeps its 32 x 8 lanes, 10.6.)  And up to four
+  // layers per thread where that still leaves a tile for every CTA
   auto tiles = [&](unsigned np, unsigned ny, unsigned nz) {
     MgTiles T;
     T.np = np, T.ny = ny, T.nz = nz;
     T.lx = 0;
     while (T.lx < 5 && (1u << T.lx) < np) ++T.lx;
-    const unsigned rows = (unsigned)kProjThreads >> T.lx;
-    T.tx = (np + (1u << T.lx) - 1) >> T.lx;
-    T.ty = (ny + rows - 1) / rows;
+    auto over = [](unsigned n, unsigned l) { return ((uint64_t)n + (1u << l) - 1) >> l; };  // ceil(n / 2^l)
+    uint64_t fewest = UINT64_MAX;
+    for (int ly = 8 - (int)T.lx; ly >= 0; --ly) {
+      const unsigned lz = 8 - T.lx - ly;
+      const uint64_t lanes = over(ny, ly) * over(nz, lz);
+      if (lanes < fewest) fewest = lanes, T.ly = ly, T.lz = lz;
+    }
+    T.tx = (unsigned)over(np, T.lx);
+    T.ty = (unsigned)over(ny, T.ly);
     T.kc = 1;
-    while (T.kc < 4 && (uint64_t)T.tx * T.ty * ((nz + 2 * T.kc - 1) / (2 * T.kc)) >= 608) T.kc *= 2;
-    T.tiles = T.tx * T.ty * ((nz + T.kc - 1) / T.kc);
+    unsigned lk = 0;  // log2 kc
+    while (lk < 2 && (uint64_t)T.tx * T.ty * over(nz, T.lz + lk + 1) >= 608) ++lk;
+    T.kc = 1u << lk;
+    T.tiles = T.tx * T.ty * (unsigned)over(nz, T.lz + lk);
     return T;
   };
+  auto deep = [](const MgTiles& T, auto* flat, auto* layered) { return T.lz ? layered : flat; };
   auto pairs = [&](const MgLevel& L) { return tiles((unsigned)(L.nx + 1) / 2, L.ny, L.nz); };
   auto quads = [&](const MgLevel& L) { return tiles(4 * (unsigned)L.nx, L.ny, L.nz); };  // four lanes per cell
   auto ctas = [&](const MgTiles& T) { return (int)(T.tiles < (unsigned)nblk ? T.tiles : (unsigned)nblk); };
@@ -1103,22 +1135,29 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
     for (int l = 0; l < first; ++l) {
       const MgLevel &L = W.lev[l], &C = W.lev[l + 1];
       const MgTiles T = pairs(L), Q = quads(C);
-      (l == 0 ? k_mg_down<true> : k_mg_down<false>)<<<ctas(T), kProjThreads, 0, st>>>(L, T, W.red);
-      (l == 0 ? k_mg_restrict<true> : k_mg_restrict<false>)<<<ctas(Q), kProjThreads, 0, st>>>(L, C, Q, W.red);
+      (l == 0 ? deep(T, k_mg_down<true, false>, k_mg_down<true, true>)
+              : deep(T, k_mg_down<false, false>, k_mg_down<false, true>))<<<ctas(T), kProjThreads, 0, st>>>(L, T, W.red);
+      (l == 0 ? deep(Q, k_mg_restrict<true, false>, k_mg_restrict<true, true>)
+              : deep(Q, k_mg_restrict<false, false>, k_mg_restrict<false, true>))<<<ctas(Q), kProjThreads, 0, st>>>(
+          L, C, Q, W.red);
     }
     k_mg_tail<<<1, kMgTailThreads, tail_bytes, st>>>(levels, first, top, W.red);
     for (int l = first - 1; l >= 0; --l) {
       const MgLevel &L = W.lev[l], &C = W.lev[l + 1];
       const MgTiles T = pairs(L);
-      (l == 0 ? k_mg_up_black<true> : k_mg_up_black<false>)<<<ctas(T), kProjThreads, 0, st>>>(L, C, T, W.red);
+      (l == 0 ? deep(T, k_mg_up_black<true, false>, k_mg_up_black<true, true>)
+              : deep(T, k_mg_up_black<false, false>, k_mg_up_black<false, true>))<<<ctas(T), kProjThreads, 0, st>>>(
+          L, C, T, W.red);
       if (l > 0)
-        k_mg_up_red<<<ctas(T), kProjThreads, 0, st>>>(L, T, W.red);
+        deep(T, k_mg_up_red<false>, k_mg_up_red<true>)<<<ctas(T), kProjThreads, 0, st>>>(L, T, W.red);
       else
-        k_mg_up_red_dot<<<ctas(T), kProjThreads, 0, st>>>(L, T, cur, W.P, W.red);
+        deep(T, k_mg_up_red_dot<false>, k_mg_up_red_dot<true>)<<<ctas(T), kProjThreads, 0, st>>>(L, T, cur, W.P,
+                                                                                                 W.red);
     }
     if (first == 0) k_cg_dot<<<nblk, kProjThreads, 0, st>>>(g.n, cur, W.r, W.z, W.P, W.red);
     const MgTiles T = tiles(g.nx, g.ny, g.nz);
-    k_cg_dir_apply<<<ctas(T), kProjThreads, 0, st>>>(W.lev[0], T, cur, W.z, W.d[cur ^ 1], W.d[cur], W.y, W.P, W.red);
+    deep(T, k_cg_dir_apply<false>, k_cg_dir_apply<true>)<<<ctas(T), kProjThreads, 0, st>>>(
+        W.lev[0], T, cur, W.z, W.d[cur ^ 1], W.d[cur], W.y, W.P, W.red);
     k_cg_update<<<nblk, kProjThreads, 0, st>>>(g.n, cur, W.d[cur], W.y, W.e, W.r, W.P, W.red);
     launches += 4 * first + (first == 0 ? 4 : 3);
   };
@@ -1130,7 +1169,7 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
       rc2 = set_error(GIC_ERR_CUDA, "gic_project: clearing p failed");
       break;
     }
-    int last_iters = 4;  // of the previous CG run
+    int last_iters = 0;  // of the previous CG run
     for (int outer = 0;; ++outer) {
       const double tol2 = P->inner_tol * P->inner_tol;
       if (outer == 0)  // p = 0
@@ -1154,9 +1193,10 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
       if (outer >= P->max_outer) break;
       // the FP32 preconditioned CG on A e = r to a reduction of inner_tol (of
       // the FP32 copy's r . r): as many iterations as the previous run took,
-      // less one, are queued before the stop flag is read, then two at a time
-      // (iterations queued past the stop return at once)
-      int it = 0, want = last_iters > 2 ? last_iters - 1 : 2;
+      // less one in runs of more than four (a read costs about as much as an
+      // iteration queued past the stop, whose kernels return at once), three in the
+      // first run, are queued before the stop flag is read, then two at a time
+      int it = 0, want = last_iters == 0 ? 3 : last_iters > 4 ? last_iters - 1 : last_iters > 2 ? last_iters : 2;
       for (;;) {
         for (int q = 0; q < want && it < P->max_inner; ++q, ++it) cg_iteration(it & 1);
         cudaError_t le = cudaGetLastError();
