@@ -317,13 +317,19 @@ __device__ __forceinline__ bool build_row(const TileShared<NT>& sh, const TileBo
                     if (d2 < Rs * Rs) keep((int64_t)B.start[bj] + (t - B.off[bj]));
                   });
   } else {  // the box exceeds the tile: the 27 cells from global memory
-    for_each_partner(G, table, epoch, i, cx, cy, cz, [&](int64_t j, int, int, int) {
-      const float4 fj = fpos(j);
-      const float rx = fj.x - fi.x, ry = fj.y - fi.y, rz = fj.z - fi.z;
-      const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-      const float Rs = reach(fj.w);
-      if (d2 < Rs * Rs) keep(j);
-    });
+    auto walk = [&](auto at) {
+      for_each_partner(G, table, epoch, i, cx, cy, cz, [&](int64_t j, int, int, int) {
+        const float4 fj = at(j);
+        const float rx = fj.x - fi.x, ry = fj.y - fi.y, rz = fj.z - fi.z;
+        const float d2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+        const float Rs = reach(fj.w);
+        if (d2 < Rs * Rs) keep(j);
+      });
+    };
+    if (sizeof(T) == 4 && fpos.posf)  // the choice outside the loop
+      walk([&](int64_t j) { return __ldg(&fpos.posf[j]); });
+    else
+      walk(fpos);
   }
   nb.count[i] = kStep && over ? kNbWalked : cnt;
   nb.at[i] = (int32_t)i;
