@@ -813,7 +813,8 @@ __device__ __forceinline__ void for_each_list_contact(const DGrid& G, const NbDe
 // longest list, and a candidate's records are loaded together.  A call that keeps
 // its lists: 8M bed (rows of 0 to 40) 1230 -> 903 us, dense packing of 1M 215 -> 195;
 // the adjoint there 1996 -> 1338 and 320 -> 299; a call with alpha_s, whose
-// accumulators are then cleared after the walk, 1550 -> 1251 on the bed.  (The capillary walk, where
+// accumulators are then cleared after the walk, 1550 -> 1251 on the bed;
+// gic_substep on a dense packing of 98,000 40.8 -> 39.3.  (The capillary walk, where
 // nearly every entry of a row is a bridge or a contact, is 5% slower with it.)
 template <typename Reach, typename F>
 __device__ __forceinline__ void for_each_list_candidate(const NbDev& nb, int64_t i, const float4& fi,

@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 || NT == kSmallThreads ? 4 
   }
   // the candidates' list of the contact walk: the words in which this thread parks
   // its stencils afterwards, or alpha_s is accumulated
-  constexpr bool kHitList = sizeof(T) == 4 && kMode == kStep;
+  constexpr bool kHitList = sizeof(T) == 4 && kMode != kStepCap;
   // the CTA's tile: the fields staged for G2P, and (FP32) F_s / alpha_s accumulators
   SubBox B;
   if constexpr (sizeof(T) == 4)
