@@ -13,6 +13,8 @@
 // per simulator), and about 14 us per call on the device (1M dam break, a
 // list-keeping call: 93.2 -> 78.1 us; 8k granules FP64, a 10-substep window:
 // 1003 -> 566 us).
+#include <cuda.h>
+
 #include <mutex>
 
 #include "gic_contact.cuh"
@@ -108,22 +110,50 @@ __global__ void __launch_bounds__(kStepSortThreads, kStepSortCtas)
   }
 }
 
-// CTAs of the cooperative launch that the current device holds at once.
+// SMs of a stream that owns a part of the device's (a green context's), 0 for any
+// other.
+static int partition_sms(cudaStream_t st) {
+  using StreamGetCtx = CUresult (*)(CUstream, CUcontext*, CUgreenCtx*);
+  using GetDevResource = CUresult (*)(CUgreenCtx, CUdevResource*, CUdevResourceType);
+  static const auto entry = [](const char* name, unsigned version) {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    return cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &found) == cudaSuccess &&
+                   found == cudaDriverEntryPointSuccess
+               ? f
+               : nullptr;
+  };
+  static const StreamGetCtx get_ctx = (StreamGetCtx)entry("cuStreamGetCtx", 12050);
+  static const GetDevResource get_resource = (GetDevResource)entry("cuGreenCtxGetDevResource", 12040);
+  if (!get_ctx || !get_resource) return 0;
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  CUdevResource r;
+  if (get_ctx((CUstream)st, &ctx, &green) != CUDA_SUCCESS || !green ||
+      get_resource(green, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS)
+    return 0;
+  return (int)r.sm.smCount;
+}
+
+// CTAs of the cooperative launch that are resident at once on the SMs the stream
+// has: more would wait at a barrier for CTAs that cannot start.
 template <typename T>
-static int resident_ctas() {
+static int resident_ctas(cudaStream_t st) {
   static std::mutex mu;
-  static int ctas[64] = {0};
+  static int sms[64] = {0}, per[64] = {0};
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  const int part = partition_sms(st);
   std::lock_guard<std::mutex> lock(mu);
-  if (!ctas[dev]) {
-    int sms = 0, per = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step_sort<T>, kStepSortThreads, 0) != cudaSuccess)
+  if (!sms[dev]) {
+    int m = 0, p = 0;
+    if (cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p, k_step_sort<T>, kStepSortThreads, 0) != cudaSuccess)
       return 0;
-    ctas[dev] = sms * (per < kStepSortCtas ? per : kStepSortCtas);
+    sms[dev] = m;
+    per[dev] = p < kStepSortCtas ? p : kStepSortCtas;
   }
-  return ctas[dev];
+  return (part > 0 && part < sms[dev] ? part : sms[dev]) * per[dev];
 }
 
 template <typename T>
@@ -146,7 +176,7 @@ static int launch(const DGrid& G, const GicGranules* in, const GicGranules* out,
                     (uint4*)table,
                     flags,
                     status_word()};
-  const int most = resident_ctas<T>();
+  const int most = resident_ctas<T>(st);
   if (most < 1) return set_error(GIC_ERR_CUDA, "gic_step: no room for the sort kernel on this device");
   const unsigned want = grid_blocks(in->n, kStepSortThreads);
   void* args[] = {&A};
