@@ -1,7 +1,7 @@
-"""gic_step's cooperative sort and early-launched substep on streams other than one
-ordinary one: several at once, two host threads on one, and one that owns a part of
-the SMs.
-Every simulator must end in the bits that it has when it runs alone."""
+"""gic_step's cooperative sort and early-launched substep elsewhere than on one ordinary
+stream: on several at once, from two host threads on one, on a stream that owns a part
+of the SMs, and in a captured graph.  Every simulator must end in the bits that it has
+when it runs alone."""
 import ctypes as C
 import threading
 
@@ -126,3 +126,30 @@ def test_a_stream_with_a_part_of_the_sms(prec):
     finally:
         torch.cuda.synchronize()
         part.close()
+
+
+@pytest.mark.parametrize("prec", [FP32, FP64])
+@pytest.mark.parametrize("name", ["loose", "wet_block"])
+def test_a_captured_call_replays_like_the_direct_one(name, prec):
+    """Two gic_step calls (A -> A2 -> A, the second with alpha_s) in a graph: each
+    replay decides anew on the device whether it sorts."""
+    prob = _problem() if name == "loose" else shuffled(gi.make(name))
+    direct, graphed = (Simulator.from_problem(prob, prec) for _ in range(2))
+
+    def pair(sim, stream=None):
+        sim.substep(alpha=False, sums=False, stream=stream)
+        sim.substep(stream=stream)
+
+    replays = 5
+    for _ in range(replays + 1):
+        pair(direct)
+    pair(graphed)  # (the first call of a process loads the kernels, which a capture may not)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        pair(graphed)
+    for _ in range(replays):
+        graph.replay()
+    _same(_result(graphed), _result(direct), prec)
+    assert graphed.nb.builds() == direct.nb.builds() and (name != "loose" or direct.nb.builds() > 2)
+    assert gic.gic_check_status() == 0
