@@ -34,8 +34,10 @@ int set_error(int code, const char* fmt, ...) {
 void count_launches(int64_t k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 
 // Poll the stream against a deadline instead of blocking forever: for the first
-// milliseconds without sleeping (a sleep of 20 us takes 70-80), then with.
-int wait_stream(cudaStream_t stream, int64_t timeout_ms, const char* what) {
+// spin_ms without sleeping, then with.  A sleep of 20 us takes 70-80, which counts
+// where a call waits for short kernels again and again; a spin keeps a host core
+// busy, so a caller that waits once for long asks for little or none.
+int wait_stream(cudaStream_t stream, int64_t timeout_ms, const char* what, int64_t spin_ms) {
   auto t0 = std::chrono::steady_clock::now();
   for (;;) {
     cudaError_t q = cudaStreamQuery(stream);
@@ -43,7 +45,7 @@ int wait_stream(cudaStream_t stream, int64_t timeout_ms, const char* what) {
     if (q != cudaErrorNotReady) return set_error(GIC_ERR_CUDA, "%s: %s", what, cudaGetErrorString(q));
     auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count();
     if (ms > timeout_ms) return set_error(GIC_ERR_TIMEOUT, "%s: stream still busy after %lld ms", what, (long long)ms);
-    if (ms >= 20) std::this_thread::sleep_for(std::chrono::microseconds(20));
+    if (ms >= spin_ms) std::this_thread::sleep_for(std::chrono::microseconds(20));
   }
 }
 
@@ -339,7 +341,7 @@ int gic_check_status(uint32_t* flags, int32_t clear, int32_t timeout_ms, gic_str
   if (!flags) return set_error(GIC_ERR_INVALID, "flags is NULL");
   uint32_t* st = status_word();
   if (!st) return set_error(GIC_ERR_CUDA, "status word unavailable");
-  int rc = wait_stream((cudaStream_t)stream, timeout_ms > 0 ? timeout_ms : 60000, "gic_check_status");
+  int rc = wait_stream((cudaStream_t)stream, timeout_ms > 0 ? timeout_ms : 60000, "gic_check_status", 0);
   if (rc) return rc;
   uint32_t h = 0;
   cudaError_t e = cudaMemcpy(&h, st, sizeof(uint32_t), cudaMemcpyDeviceToHost);

@@ -978,7 +978,7 @@ static int proj_grid(const GicGrid* grid, PGrid* g) {
 static int read_red(const ProjRed* dev, ProjRed* host, cudaStream_t st) {
   if (cudaMemcpyAsync(host, dev, sizeof(ProjRed), cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return set_error(GIC_ERR_CUDA, "gic_project: reading the solver's scalars failed");
-  return wait_stream(st, 60000, "gic_project");
+  return wait_stream(st, 60000, "gic_project", 20);
 }
 
 }  // namespace gic

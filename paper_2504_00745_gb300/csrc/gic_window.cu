@@ -383,5 +383,5 @@ extern "C" int gic_window_forward_host(const GicGrid* grid, const GicParams* par
   if (Fs_w) GIC_CU(cudaMemcpyAsync(Fs_w, sw, real * L.n_fields_w, cudaMemcpyDeviceToHost, st));
   if (sums2) GIC_CU(cudaMemcpyAsync(sums2, d_sums, 16, cudaMemcpyDeviceToHost, st));
 #undef GIC_CU
-  return wait_stream(st, 600000, "gic_window_forward_host");
+  return wait_stream(st, 600000, "gic_window_forward_host", 5);  // (a window of a million granules: 3 ms)
 }
