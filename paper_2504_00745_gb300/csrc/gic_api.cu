@@ -33,6 +33,14 @@ int set_error(int code, const char* fmt, ...) {
 
 void count_launches(int64_t k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 
+int sm_count() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
+    return sms;
+  return 152;  // without a device (sizes may be asked for all the same)
+}
+
 // Poll the stream against a deadline instead of blocking forever: for the first
 // spin_ms without sleeping, then with.  A sleep of 20 us takes 70-80, which counts
 // where a call waits for short kernels again and again; a spin keeps a host core

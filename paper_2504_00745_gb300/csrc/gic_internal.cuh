@@ -44,6 +44,7 @@ struct alignas(32) d4 {
 int set_error(int code, const char* fmt, ...);
 void count_launches(int64_t k);
 int wait_stream(cudaStream_t stream, int64_t timeout_ms, const char* what, int64_t spin_ms);
+int sm_count();           // SMs of the current device
 uint32_t* status_word();  // device address of the sticky status word (current device)
 
 #define GIC_CHECK_LAUNCH(what)                                                                           \

@@ -904,10 +904,8 @@ struct ProjWs {
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 static int proj_blocks(int64_t n) {
-  int dev = 0, sms = 152;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t want = (n + kProjThreads - 1) / kProjThreads;
-  const int64_t cap = 8 * (int64_t)(sms > 0 ? sms : 152);
+  const int64_t cap = 8 * (int64_t)sm_count();
   return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
 
@@ -1102,7 +1100,9 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
   // grid.  (All of them on rows, a column of 1 x 1 x 20000 cells had one lane of 256 at
   // work: 10.5 ms a call, now 2.5; 2 x 2 x 65536 13.0 -> 4.5, 4 x 4 x 4096 15.6 -> 10.9,
   // 300 x 1 x 300 6.9 -> 5.7; 128^3 keeps its 32 x 8 lanes, 10.6.)  And up to four
-  // layers per thread where that still leaves a tile for every CTA
+  // layers per thread where that still leaves a tile for every CTA that is resident at
+  // once (four per SM)
+  const uint64_t resident = 4 * (uint64_t)sm_count();
   auto tiles = [&](unsigned np, unsigned ny, unsigned nz) {
     MgTiles T;
     T.np = np, T.ny = ny, T.nz = nz;
@@ -1119,7 +1119,7 @@ extern "C" int gic_project(const GicGrid* grid, const GicProjParams* P, const do
     T.ty = (unsigned)over(ny, T.ly);
     T.kc = 1;
     unsigned lk = 0;  // log2 kc
-    while (lk < 2 && (uint64_t)T.tx * T.ty * over(nz, T.lz + lk + 1) >= 608) ++lk;
+    while (lk < 2 && (uint64_t)T.tx * T.ty * over(nz, T.lz + lk + 1) >= resident) ++lk;
     T.kc = 1u << lk;
     T.tiles = T.tx * T.ty * (unsigned)over(nz, T.lz + lk);
     return T;

@@ -16,15 +16,18 @@
 
 namespace gic {
 
-// CTAs of 256 threads; a small FP64 state takes CTAs of 64, at most four per SM, so
+// CTAs of 256 threads; a small FP64 state takes CTAs of 64, at most three per SM, so
 // that it is spread over the chip: 8,000 granules in 32 CTAs kept 32 SMs busy and
-// 120 idle, and FP64 instructions issue at 1.8 lanes per clock and SM.  The 10-substep
-// window of 8,000 granules with one rebuild: 552 us in CTAs of 256, 433 in these.
+// 120 idle, and FP64 instructions issue at 1.8 lanes per clock and SM.  Windows of 20
+// substeps in CTAs of 256 and of 64 (152 SMs: the line at 29,184), dense packing: 2590
+// and 1746 us at 9,000 granules, 2925 and 2549 at 27,000, 2974 and 2941 at 32,000, 3029
+// and 3079 at 37,000; loose packing, where the staging of the tiles weighs more: 727
+// and 687 at 8,000, 831 and 837 at 29,000, 792 and 855 at 32,000, 1221 and 1422 at 50,000.
 // (FP32 stays at 256: 467 against 446 us at 7,000 granules, and two partners'
 // opposite deposits cancel exactly inside one CTA's integer tile only.)
 constexpr int kSubstepThreads = kSubThreads;
 constexpr int kSmallThreads = 64;
-constexpr int64_t kSmallGranules = 4 * 152 * kSmallThreads;
+constexpr int kSmallPerSm = 3;
 
 // The granule arrays a substep reads.
 template <typename T>
@@ -624,7 +627,7 @@ static int substep_launch(const DGrid& G, const GicParams* params, const GicGran
     } else {
       DParams<double> P;
       if ((rc = make_params(params, &P))) return rc;
-      if (sorted && s->n <= kSmallGranules)
+      if (sorted && s->n <= (int64_t)kSmallPerSm * kSmallThreads * sm_count())
         rc = go(0.0, kSmall,
                 P.cap ? k_substep<double, kStepCap, false, kSmallThreads>
                       : k_substep<double, kStep, false, kSmallThreads>,
