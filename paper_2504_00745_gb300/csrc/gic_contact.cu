@@ -262,25 +262,10 @@ __global__ void k_contact_pairs(DGrid G, int64_t n, const int32_t* __restrict__ 
   if (counts) counts[i] = cnt;
 }
 
-// Optional copy of the checked state into a second state (same order), for a
-// caller whose sort may be skipped: cell, position record, velocity, id, the
-// FP32 float positions and an identity permutation.
-template <typename T>
-struct StateCopy {
-  const vec_t<T>* vel;
-  int32_t* cell_out;
-  pos_t<T>* pos_out;
-  vec_t<T>* vel_out;
-  int32_t* id_out;
-  float4* posf_out;
-  int32_t* perm_out;
-};
-
 template <typename T>
 __global__ void __launch_bounds__(256) k_verlet_check(DGrid G, int64_t n, const int32_t* __restrict__ cell,
                                                        const pos_t<T>* __restrict__ pos,
-                                                       const int32_t* __restrict__ id, NbDev nb, T lim2,
-                                                       StateCopy<T> cp) {
+                                                       const int32_t* __restrict__ id, NbDev nb, T lim2) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   bool far = false;
   if (i < n) {
@@ -295,17 +280,6 @@ __global__ void __launch_bounds__(256) k_verlet_check(DGrid G, int64_t n, const 
         far = moved_far(G, c, p, nb.ref_cell[s], reinterpret_cast<const pos_t<T>*>(nb.ref_pos)[s], lim2);
       } else {
         far = true;  // ids outside 0..n-1: rebuild (the build path does not need them)
-      }
-    }
-    if (cp.cell_out) {
-      cp.cell_out[i] = c;
-      cp.pos_out[i] = p;
-      cp.vel_out[i] = cp.vel[i];
-      cp.id_out[i] = k;
-      cp.perm_out[i] = (int32_t)i;
-      if constexpr (sizeof(T) == 4) {
-        if (cp.posf_out)
-          cp.posf_out[i] = posf_of(c, p);
       }
     }
   }
@@ -507,31 +481,20 @@ int verlet_view(const DGrid& G, const GicGranules* s, const void* table, const G
   return GIC_OK;
 }
 
-int verlet_check(const DGrid& G, const GicGranules* s, const void* table, const GicNeighbors* nb,
-                 cudaStream_t stream, const char* what, NbDev* out, GicGranules* copy_to, int32_t* perm) {
-  int rc;
-  if ((rc = check_table(table))) return rc;
-  if ((rc = check_neighbors(nb, s, what))) return rc;
-  const NbDev d = nb_dev(G, nb, false);
-  *out = d;
+// Maps the current sorted indices to slots and checks every displacement (sets the
+// call's rebuild word).
+static int verlet_check(const DGrid& G, const GicGranules* s, const void* table, const GicNeighbors* nb,
+                        cudaStream_t stream, const char* what, NbDev* out) {
+  if (int rc = verlet_view(G, s, table, nb, what, false, out)) return rc;
   if (s->n == 0) return GIC_OK;
-  if (copy_to && (!perm || !copy_to->id)) return set_error(GIC_ERR_INVALID, "%s: copy needs ids and perm", what);
   const double half = 0.5 * nb->skin;
   if (s->precision == GIC_FP32) {
     const double lim = half * G.inv_unit;  // skin / 2 in 2^-30 h_c units
-    StateCopy<float> cp{};
-    if (copy_to)
-      cp = StateCopy<float>{(const float4*)s->vel, copy_to->cell, (uint4*)copy_to->pos, (float4*)copy_to->vel,
-                            copy_to->id, (float4*)copy_to->posf, perm};
-    k_verlet_check<float><<<grid_blocks(s->n, 256), 256, 0, stream>>>(G, s->n, s->cell, (const uint4*)s->pos, s->id, d,
-                                                                      (float)(lim * lim), cp);
+    k_verlet_check<float><<<grid_blocks(s->n, 256), 256, 0, stream>>>(G, s->n, s->cell, (const uint4*)s->pos, s->id,
+                                                                      *out, (float)(lim * lim));
   } else {
-    StateCopy<double> cp{};
-    if (copy_to)
-      cp = StateCopy<double>{(const d4*)s->vel, copy_to->cell, (d4*)copy_to->pos, (d4*)copy_to->vel, copy_to->id,
-                             nullptr, perm};
-    k_verlet_check<double><<<grid_blocks(s->n, 256), 256, 0, stream>>>(G, s->n, s->cell, (const d4*)s->pos, s->id, d,
-                                                                       half * half, cp);
+    k_verlet_check<double><<<grid_blocks(s->n, 256), 256, 0, stream>>>(G, s->n, s->cell, (const d4*)s->pos, s->id,
+                                                                       *out, half * half);
   }
   count_launches(1);
   return GIC_OK;
@@ -543,7 +506,7 @@ int verlet_prelude(const DGrid& G, const GicParams* params, const GicGranules* s
   int rc;
   if (launch_build && !F_c) return set_error(GIC_ERR_INVALID, "%s: F_c is NULL", what);
   if ((rc = check_vecs(s->precision, what, {F_c}))) return rc;
-  if ((rc = verlet_check(G, s, table, nb, stream, what, out, nullptr, nullptr))) return rc;
+  if ((rc = verlet_check(G, s, table, nb, stream, what, out))) return rc;
   if (s->n == 0 || !launch_build) return GIC_OK;
   const NbDev d = *out;
   if (s->precision == GIC_FP32) {

@@ -629,11 +629,6 @@ int verlet_prelude(const DGrid& G, const GicParams* params, const GicGranules* s
 NbDev nb_dev(const DGrid& G, const GicNeighbors* nb, bool ident);
 int verlet_view(const DGrid& G, const GicGranules* s, const void* table, const GicNeighbors* nb, const char* what,
                 bool ident, NbDev* out);
-// The displacement check alone (maps the state's ids to slots, sets the
-// rebuild word); with copy_to, it also copies the state into copy_to in the
-// same order and writes the identity into perm.
-int verlet_check(const DGrid& G, const GicGranules* s, const void* table, const GicNeighbors* nb,
-                 cudaStream_t stream, const char* what, NbDev* out, GicGranules* copy_to, int32_t* perm);
 
 // This gic_step call is to rebuild: a granule was beyond skin / 2 of its reference
 // after the last one, or a rebuild was requested.  For the sort kernel alone:

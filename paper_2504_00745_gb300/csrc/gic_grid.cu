@@ -527,8 +527,8 @@ __global__ void __launch_bounds__(256) k_p2g_adj(DGrid G, DParams<T> P, int64_t 
 }
 
 // The cluster size of k_alpha_total_f32 is beyond the portable 8: allowed
-// once per device, before any capture.
-int alpha_prepare() {
+// once per device.
+static int alpha_prepare() {
   static std::mutex mu;
   static bool done[64] = {false};
   int dev = 0;

@@ -938,8 +938,6 @@ inline Fields<T> fields(const void* u, const void* v, const void* w, const void*
 // lends for the exact totals; with it the totals come out of the conversion
 // pass (one read of the grid), without it from a separate cluster pass.
 int alpha_begin(double* alpha_s, int64_t ncell, double* sums2, cudaStream_t stream, void* scratch = nullptr);
-// one-time per-device set-up of the exact totals' kernel (call before any capture)
-int alpha_prepare();
 int alpha_end(const DGrid& G, int32_t precision, double* alpha_s, int64_t ncell, double* sums2, cudaStream_t stream,
               void* scratch = nullptr);
 

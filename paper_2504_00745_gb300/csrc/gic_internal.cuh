@@ -305,51 +305,6 @@ __device__ __forceinline__ double mac_frac_fp64(const DGrid& G, int c, int m, ui
 }
 __device__ __forceinline__ double mac_frac_fp64(const DGrid& G, int c, int m, double o) { return mac_frac(G, c, m, o); }
 
-// Tent-kernel stencil along one axis.  Samples sit at (i + s) dx, i = 0..ns-1,
-// with s = 0 (the axis normal to a face) or 1/2 (cell centres).  The point is
-// at m + t (grid units).  Returns the lower sample i0 and the weight w of
-// sample i0 + 1; points beyond the end samples clamp onto them (G2P), which
-// is also the folding rule of the scatter (P2G).
-template <typename T>
-__device__ __forceinline__ void stencil_axis(int m, T t, bool face, int ns, int& i0, T& w) {
-  if (face) {
-    i0 = m;
-    w = t;
-  } else if (t >= T(0.5)) {
-    i0 = m;
-    w = t - T(0.5);
-  } else {
-    i0 = m - 1;
-    w = t + T(0.5);
-  }
-  if (i0 < 0) {
-    i0 = 0;
-    w = T(0);
-  } else if (i0 > ns - 2) {
-    i0 = ns - 2;
-    w = T(1);
-  }
-}
-
-template <typename T>
-struct Stencil {
-  int i0[3];
-  T w[3];
-};
-
-// stencil of MAC component comp (0,1,2: faces normal to x,y,z; 3: centres)
-template <typename T>
-__device__ __forceinline__ Stencil<T> stencil_of(const DGrid& G, const int m[3], const T t[3], int comp) {
-  Stencil<T> S;
-  const int n[3] = {G.nx, G.ny, G.nz};
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    bool face = (a == comp);
-    stencil_axis<T>(m[a], t[a], face, n[a] + (face ? 1 : 0), S.i0[a], S.w[a]);
-  }
-  return S;
-}
-
 __device__ __forceinline__ int64_t sample_index(int nsx, int nsy, int i, int j, int k) {
   return i + (int64_t)nsx * (j + (int64_t)nsy * k);
 }

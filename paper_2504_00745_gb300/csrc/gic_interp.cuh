@@ -15,6 +15,11 @@ struct Stencil3 {
   int ns[3];
 };
 
+// Tent-kernel stencil of MAC component comp (0, 1, 2: the faces normal to x, y, z; 3:
+// the centres) for a point at m + t in MAC cells.  Samples sit at i + s, i = 0 .. ns -
+// 1, with s = 0 on the axis normal to a face and 1/2 otherwise; i0 is the lower
+// sample, w the weight of the next.  Points beyond the end samples clamp onto them
+// (G2P), which is also the folding rule of the scatter (P2G).
 template <typename T>
 __device__ __forceinline__ Stencil3<T> make_stencil(const DGrid& G, const int m[3], const T t[3], int comp) {
   Stencil3<T> S;
