@@ -360,9 +360,11 @@ class GicWindow(torch.autograd.Function):
 
     With Verlet lists and the fused path, forward and recomputation run
     gic_step (the sort only on list rebuilds).  The window opens with a list
-    build, and every checkpoint also keeps the lists as they stand (a new
-    copy only after a build), so the recomputation from it repeats the
-    forward pass exactly.  The recomputation keeps the state before every
+    build, and every checkpoint after the first also copies the lists as they
+    stand (whether a build happened is known on the device only, until the end of
+    the forward pass: the checkpoints of one build then share one copy, 4 cap +
+    28 bytes a granule in FP32), so the recomputation from it repeats the forward
+    pass exactly.  The recomputation keeps the state before every
     substep and notes which substeps rebuilt the lists; going back, the
     lists each substep used are restored (from the checkpoint, or by sort +
     build from the state of the substep that built them), and each
@@ -405,6 +407,9 @@ class GicWindow(torch.autograd.Function):
         # the list words at every checkpoint and at the end, read once: the recomputation
         # from each checkpoint repeats the forward pass exactly, builds included
         ctx.words = torch.stack([q["flags"] for q in lists] + [sim.nb.flags]).tolist() if stepped else None
+        for m in range(2, len(lists)):  # the rows of one build: one copy of them is enough
+            if ctx.words[m][_BUILDS] == ctx.words[m - 1][_BUILDS]:
+                lists[m]["arrays"] = lists[m - 1]["arrays"]
         ctx.final = sim.A.clone()
         return x
 
