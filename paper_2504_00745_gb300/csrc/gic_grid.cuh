@@ -462,7 +462,7 @@ __device__ __forceinline__ void p2g_sums(double* sums, long long v) {
 // for G2P and F_s, deposits rounded by the multiply-add that forms them.
 // 1702 -> 1400 instructions per warp on the 16M sweep; a gic_step call that
 // keeps its lists 1180 -> 1020 us there, 78 -> 67 us on the 1M dam break.
-constexpr int kSubTile = 960;  // 46 KB of static shared memory
+constexpr int kSubTile = 960;  // 46 KB of shared memory
 constexpr int kSubThreads = 256;
 constexpr int kSubWarps = kSubThreads / 32;
 

@@ -326,7 +326,10 @@ __device__ __forceinline__ bool build_row(const TileShared<NT>& sh, const TileBo
         if (d2 < Rs * Rs) keep(j);
       });
     };
-    if (sizeof(T) == 4 && fpos.posf)  // the choice outside the loop
+    // gic_neighbors_build has float copies: without the question for every candidate
+    // 10,976 granules in cells of 190 take 358 us instead of 465.  (gic_step may have
+    // none; both walks in its kernel made the 16M sweep's rebuild 1.3% slower.)
+    if constexpr (sizeof(T) == 4 && !kStep)
       walk([&](int64_t j) { return __ldg(&fpos.posf[j]); });
     else
       walk(fpos);
