@@ -85,8 +85,7 @@ def parse():
                     help="with --profile-substeps: instead of substeps, that many list builds of the sorted state "
                          "(gic_sort + gic_neighbors_build), for a capture of the staged build")
     ap.add_argument("--profile-direct", action="store_true",
-                    help="with --profile-substeps: gic_sort + gic_substep every substep , so that "
-                         "a profiler sees each kernel")
+                    help="with --profile-substeps: gic_sort + gic_substep every substep instead of gic_step")
     return ap.parse_args()
 
 

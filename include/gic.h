@@ -294,20 +294,22 @@ int gic_substep(const GicGrid* grid, const GicParams* params, const GicGranules*
  * The caller swaps state and next between calls.
  *   FP32: `next` receives float positions (posf, if set) for the next
  *   call's contact pre-tests, read from `state` (if set) when no sort runs.
- *   Two launches (four with alpha_s), the same in every call, and no host
- *   sync: a cooperative kernel that sorts when the flags ask for it and
- *   returns at once otherwise, and the substep kernel, which then builds the
- *   rows of `sorted` and reads it, or reads `state`.  Nothing is kept between
- *   calls.
+ *   Two launches, the same in every call, and no host sync: a cooperative
+ *   kernel that sorts when the flags ask for it and returns at once otherwise,
+ *   and the substep kernel, which then builds the rows of `sorted` and reads
+ *   it, or reads `state`.  With sigma > 0 one more between them (every granule's
+ *   moisture ratio); with alpha_s one before the substep kernel (it is cleared)
+ *   and one after it (FP32: the conversion; FP64: the sum, with sums2 only).
+ *   Nothing is kept between calls.
  *   The sort's waits are limited (some seconds).  If one runs out, the status
  *   gets GIC_STATUS_STALL, and that call and every later one on the same lists,
  *   until gic_neighbors_reset, raise it again and make no step: `next` is a copy
  *   of `state`, F_s and the lists stay as they were, alpha_s and sums2 come out 0
  *   (`sorted`, perm and the cell table are incomplete).
  *   Arguments as for gic_sort and gic_substep (state, next and sorted must
- *   carry ids and share no array); errors as for those calls.  With sums2
- *   the first 32 bytes of ws also hold the exact alpha_s totals while the
- *   call runs. */
+ *   carry ids and share no array); errors as for those calls.  While the call
+ *   runs, ws also holds, after the sort, the exact alpha_s totals (with sums2;
+ *   its first 32 bytes) and the moisture ratios (with sigma > 0). */
 int gic_step(const GicGrid* grid, const GicParams* params, const GicGranules* state, GicGranules* next,
              GicGranules* sorted, int32_t* perm, void* cell_table, void* ws, size_t ws_bytes, const GicNeighbors* nb,
              const void* u, const void* v, const void* w, const void* p, const void* alpha_f, double* alpha_s,
